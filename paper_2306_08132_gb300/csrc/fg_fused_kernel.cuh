@@ -50,6 +50,7 @@ struct FusedSmem {
   float loss;
   int cand;                        // the candidate claimed by this CTA
   int bad_object;
+  int free;                        // the candidate has no contact in any simulation
   int n_active;
   int next_unit;                   // adjoint sweep: next unclaimed work unit
   int next_chunk;                  // forward sweep: next unclaimed active chunk
@@ -103,8 +104,9 @@ __device__ __forceinline__ void world_point(const float4* f4, const float4& sp, 
 }
 
 // Adjoint of one hand point (index i, link frames in smem): dL/dp through the 7
-// simulations, the normal and the SDF lookup.  v = (g, (p - t0) x g).
-template <bool ANY>
+// simulations, the normal and the SDF lookup.  v = (g, (p - t0) x g).  FREE: a
+// candidate without contacts (point_sims_adjoint_free).
+template <bool ANY, bool FREE>
 __device__ __forceinline__ void point_adjoint(const HandDev& H, const float4 (*frame4)[3], const SimAdjoints& G,
                                               const SimConsts& K, const ObjDev& O,
                                               const ParamsDev& Pm, float r, const float t0[3], int i, bool valid,
@@ -118,7 +120,10 @@ __device__ __forceinline__ void point_adjoint(const HandDev& H, const float4 (*f
   PointState ps;
   point_state(smp, p, r, ps);
   float dphi = 0.0f, dn[3] = {0.0f, 0.0f, 0.0f}, dp[3] = {0.0f, 0.0f, 0.0f};
-  point_sims_adjoint(ps, G, K, Pm, O, dphi, dn, dp);
+  if constexpr (FREE)
+    point_sims_adjoint_free(ps, K, dphi, dn);
+  else
+    point_sims_adjoint(ps, G, K, Pm, O, dphi, dn, dp);
   sdf_adjoint(smp, ps, dphi, dn, dp);
   if (valid) {
     const float rel[3] = {p[0] - t0[0], p[1] - t0[1], p[2] - t0[2]};
@@ -134,7 +139,7 @@ __device__ __forceinline__ void point_adjoint(const HandDev& H, const float4 (*f
 
 // The same for two points (a, b) at once, in packed f32x2 arithmetic: positions
 // and grid indices per point, everything after the corner gathers on pairs.
-template <bool ANY>
+template <bool ANY, bool FREE>
 __device__ __forceinline__ void point_adjoint_pair(const HandDev& H, const float4 (*frame4)[3], const SimAdjoints& G,
                                                    const SimConsts& K, const ObjDev& O, const ParamsDev& Pm, float r,
                                                    const float t0[3], int ia, int ib, bool va, bool vb,
@@ -173,7 +178,10 @@ __device__ __forceinline__ void point_adjoint_pair(const HandDev& H, const float
   point_state(smp, p, r, ps);
   const float2 zero = make_float2(0.0f, 0.0f);
   float2 dphi = zero, dn[3] = {zero, zero, zero}, dp[3] = {zero, zero, zero};
-  point_sims_adjoint(ps, G, K, Pm, O, dphi, dn, dp);
+  if constexpr (FREE)
+    point_sims_adjoint_free(ps, K, dphi, dn);
+  else
+    point_sims_adjoint(ps, G, K, Pm, O, dphi, dn, dp);
   sdf_adjoint(smp, ps, dphi, dn, dp);
   const float2 rel[3] = {vsub(p[0], vsplat<float2>(t0[0])), vsub(p[1], vsplat<float2>(t0[1])),
                          vsub(p[2], vsplat<float2>(t0[2]))};
@@ -288,6 +296,77 @@ __device__ __forceinline__ void link_accumulate(float (*lacc)[6], int lane, int 
   }
 #pragma unroll
   for (int k = 0; k < 6; ++k) acc[k] = 0.0f;
+}
+
+// Sweep 2 of one candidate: the adjoint of every point, reduced per link.
+template <int NW, int PPT, bool ANY, bool FREE>
+__device__ __forceinline__ void adjoint_sweep(FusedSmem<NW>& S, const ObjDev& O, float r, int lane, int warp) {
+  const HandDev& H = S.H;
+  const ParamsDev& Pm = S.Pm;
+  const int P = H.P;
+  const float t0[3] = {S.q[0], S.q[1], S.q[2]};
+  if (H.nunits <= kMaxUnits) {
+    // Warps claim work units (<= 64 points of one link) from a shared
+    // counter, so a warp that meets contacts (general adjoint) does not hold
+    // the others at the barrier; each unit's sums go to its own slot, so the
+    // result does not depend on which warp ran it.  The next claim is issued
+    // before the current unit so that its latency is hidden.
+    auto claim = [&]() {
+      int j = 0;
+      if (lane == 0) j = atomicAdd(&S.next_unit, 1);
+      return __shfl_sync(kFull, j, 0);
+    };
+    int u = claim();
+    while (u < H.nunits) {
+      const int nu = claim();
+      const int4 U = __ldg(H.units + u);      // first point, count, link
+      float sum[6];
+      if (PPT == 2) {
+        // one point of each half of the unit per lane, packed arithmetic
+        float v[2][6];
+        int link[2];
+        const bool va = lane < U.y, vb = lane + 32 < U.y;
+        point_adjoint_pair<ANY, FREE>(H, S.frame4, S.G, S.K, O, Pm, r, t0, va ? U.x + lane : U.x,
+                                      vb ? U.x + 32 + lane : U.x, va, vb, v, link);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) sum[k] = v[0][k] + v[1][k];
+      } else {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) sum[k] = 0.0f;
+        for (int h = 0; h < U.y; h += 32) {
+          float v[6];
+          int link;
+          const bool valid = h + lane < U.y;
+          point_adjoint<ANY, FREE>(H, S.frame4, S.G, S.K, O, Pm, r, t0, valid ? U.x + h + lane : U.x, valid, v, link);
+#pragma unroll
+          for (int k = 0; k < 6; ++k) sum[k] += v[k];
+        }
+      }
+      unit_reduce_store(sum, lane, S.uacc[u]);
+      u = nu;
+    }
+  } else {
+    // fixed, contiguous 32-aligned point ranges per warp
+    int cur = -1;
+    float acc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    const int span = ((P + 32 * NW - 1) / (32 * NW)) * 32;
+    const int pb = warp * span, pe = min(P, pb + span);
+    for (int base = pb; base < pe; base += 32) {
+      float v[6];
+      int link;
+      const int i = base + lane;
+      const bool valid = i < pe;
+      point_adjoint<ANY, FREE>(H, S.frame4, S.G, S.K, O, Pm, r, t0, valid ? i : base, valid, v, link);
+      link_accumulate(S.lacc[warp], lane, link, valid, v, cur, acc);
+    }
+    if (cur >= 0) {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        const float sum = warp_sum(acc[k]);
+        if (lane == 0) S.lacc[warp][cur][k] += sum;
+      }
+    }
+  }
 }
 
 // ANY = false: grid objects only (the mesh lookup is compiled out).
@@ -555,6 +634,11 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
             if (th < H.q_low[lane]) g -= Pm.w_limit;
             S.grad[6 + lane] = g;
           }
+          // no contact in any simulation: the object keeps its test velocity
+          const bool busy = lane < kSims && S.Wtot[lane < kSims ? lane : 0][6] > 0.0f;
+          const bool is_free = !__any_sync(kFull, busy);
+          if (lane == 1) sim_constants_free(Pm, S.G.s[1][0].x, S.K);     // this lane wrote simulation 1
+          if (lane == 0) S.free = is_free;
           if (lane == 0) S.loss = Ls + Pm.w_range * rn + Pm.w_limit * lims + Pm.w_pen * S.Wtot[0][7];
         }
       }
@@ -575,71 +659,11 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
       }
 
       // ---------------------------------------------------------------- sweep 2
-      {
-        const float t0[3] = {S.q[0], S.q[1], S.q[2]};
-        int cur = -1;
-        float acc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-        if (H.nunits <= kMaxUnits) {
-          // Warps claim work units (<= 64 points of one link) from a shared
-          // counter, so a warp that meets contacts (general adjoint) does not hold
-          // the others at the barrier; each unit's sums go to its own slot, so the
-          // result does not depend on which warp ran it.  The next claim is issued
-          // before the current unit so that its latency is hidden.
-          auto claim = [&]() {
-            int j = 0;
-            if (lane == 0) j = atomicAdd(&S.next_unit, 1);
-            return __shfl_sync(kFull, j, 0);
-          };
-          int u = claim();
-          while (u < H.nunits) {
-            const int nu = claim();
-            const int4 U = __ldg(H.units + u);      // first point, count, link
-            float sum[6];
-            if (PPT == 2) {
-              // one point of each half of the unit per lane, packed arithmetic
-              float v[2][6];
-              int link[2];
-              const bool va = lane < U.y, vb = lane + 32 < U.y;
-              point_adjoint_pair<ANY>(H, S.frame4, S.G, S.K, O, Pm, r, t0, va ? U.x + lane : U.x,
-                                 vb ? U.x + 32 + lane : U.x, va, vb, v, link);
-#pragma unroll
-              for (int k = 0; k < 6; ++k) sum[k] = v[0][k] + v[1][k];
-            } else {
-#pragma unroll
-              for (int k = 0; k < 6; ++k) sum[k] = 0.0f;
-              for (int h = 0; h < U.y; h += 32) {
-                float v[6];
-                int link;
-                const bool valid = h + lane < U.y;
-                point_adjoint<ANY>(H, S.frame4, S.G, S.K, O, Pm, r, t0, valid ? U.x + h + lane : U.x, valid, v, link);
-#pragma unroll
-                for (int k = 0; k < 6; ++k) sum[k] += v[k];
-              }
-            }
-            unit_reduce_store(sum, lane, S.uacc[u]);
-            u = nu;
-          }
-        } else {
-          // fixed, contiguous 32-aligned point ranges per warp
-          const int span = ((P + 32 * NW - 1) / (32 * NW)) * 32;
-          const int pb = warp * span, pe = min(P, pb + span);
-          for (int base = pb; base < pe; base += 32) {
-            float v[6];
-            int link;
-            const int i = base + lane;
-            const bool valid = i < pe;
-            point_adjoint<ANY>(H, S.frame4, S.G, S.K, O, Pm, r, t0, valid ? i : base, valid, v, link);
-            link_accumulate(S.lacc[warp], lane, link, valid, v, cur, acc);
-          }
-        }
-        if (cur >= 0) {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) {
-            const float sum = warp_sum(acc[k]);
-            if (lane == 0) S.lacc[warp][cur][k] += sum;
-          }
-        }
-      }
+      // The whole CTA takes the short form when its candidate has no contact.
+      if (S.free)
+        adjoint_sweep<NW, PPT, ANY, true>(S, O, r, lane, warp);
+      else
+        adjoint_sweep<NW, PPT, ANY, false>(S, O, r, lane, warp);
       __syncthreads();
 
       // ------------------------------------------------------------------ tree
