@@ -103,6 +103,36 @@ __device__ __forceinline__ void world_point(const float4* f4, const float4& sp, 
   p[2] = fma_(c.x, sp.x, fma_(c.y, sp.y, fma_(c.z, sp.z, c.w)));
 }
 
+// Lower bound of the SDF (float32 slack taken off) over the points of one link inside
+// the sphere cs (centre and radius in the link frame f4).  Grid: the interpolated
+// field over the sphere's box is bounded below by the min-pyramid.  Mesh: the Phong
+// point lies within phong_shift of the flat closest point, so with the centre outside
+// the mesh at flat distance d > R every point of the sphere has rho >= d - R -
+// phong_shift; otherwise there is no bound.  The slack covers float32 rounding of
+// positions and values.
+template <bool ANY>
+__device__ __forceinline__ float sphere_bound(const ObjDev& O, const float4* f4, const float4& cs) {
+  float cw[3];
+  world_point(f4, cs, cw);
+  const float slack = 1e-6f + 1e-5f * (fabsf(cw[0]) + fabsf(cw[1]) + fabsf(cw[2]));
+  if (ANY && O.kind == kObjMesh) {
+    const float dc = mesh_flat_distance(O, cw);
+    const float R = cs.w + slack;
+    return dc > R ? dc - R - O.phong_shift - (1e-6f + 1e-5f * fabsf(dc)) : -3.0e38f;
+  }
+  const float R = (cs.w + slack) * O.inv_h;
+  const float org[3] = {O.ox, O.oy, O.oz};
+  float lo[3], hi[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float u = (cw[k] - org[k]) * O.inv_h;
+    lo[k] = u - R - 1e-3f;
+    hi[k] = u + R + 1e-3f;
+  }
+  const float mn = region_min(O, lo, hi);
+  return mn - (1e-6f + 1e-5f * fabsf(mn));
+}
+
 // Adjoint of one hand point (index i, link frames in smem): dL/dp through the 7
 // simulations, the normal and the SDF lookup.  v = (g, (p - t0) x g).  FREE: a
 // candidate without contacts (point_sims_adjoint_free).
@@ -453,15 +483,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
 
       // --------------------------------------------------------- chunk culling
       // A chunk of 32 points (one link) can only hold a contact if some point has
-      // phi_m = phi_hat - dt V n_k < 0, i.e. phi(p) < r + dt V.  Every point lies in
-      // the chunk's bounding sphere (centre c, radius R), and the interpolated
-      // field over that sphere is bounded below by the min-pyramid over its box,
-      // so a chunk with  min - r - dt V (1 + 1e-5) - slack > 0  has no contact in
-      // any simulation; the slack covers float32 rounding of positions and values.
-      // Its contact flags are all zero and its forces are not computed.
-      // Mesh objects: the Phong point lies within phong_shift of the flat closest
-      // point, so if the chunk's centre c is outside the mesh at flat distance
-      // d > R, every point of the chunk has rho >= d - R - phong_shift.
+      // phi_m = phi_hat - dt V n_k < 0, i.e. phi(p) < r + dt V.  A chunk whose bounding
+      // sphere has sphere_bound > r + dt V (1 + 1e-5) has no contact in any simulation:
+      // its contact flags are all zero and its forces are not computed.
       const bool cull = H.nchunks <= kMaxCullChunks;
       if (cull) {
         for (int j0 = warp * 32; j0 < H.nchunks; j0 += NW * 32) {
@@ -470,31 +494,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
           if (j < H.nchunks) {
             active = true;
             const int l = H.chunk_link[j];
-            if (l >= 0 && ANY && O.kind == kObjMesh) {
-              const float4 cs = __ldg(H.chunk_sphere + j);
-              float cw[3];
-              world_point(S.frame4[l], cs, cw);
-              const float slack = 1e-6f + 1e-5f * (fabsf(cw[0]) + fabsf(cw[1]) + fabsf(cw[2]));
-              const float dc = mesh_flat_distance(O, cw);
-              const float R = cs.w + slack;
-              const float lbm = dc - R - O.phong_shift;
-              active = !(dc > R && lbm - r - dtV * (1.0f + 1e-5f) - (1e-6f + 1e-5f * fabsf(dc)) > 0.0f);
-            } else if (l >= 0) {
-              const float4 cs = __ldg(H.chunk_sphere + j);
-              float cw[3];
-              world_point(S.frame4[l], cs, cw);
-              const float slack = 1e-6f + 1e-5f * (fabsf(cw[0]) + fabsf(cw[1]) + fabsf(cw[2]));
-              const float R = (cs.w + slack) * O.inv_h;
-              const float org[3] = {O.ox, O.oy, O.oz};
-              float lo[3], hi[3];
-#pragma unroll
-              for (int k = 0; k < 3; ++k) {
-                const float u = (cw[k] - org[k]) * O.inv_h;
-                lo[k] = u - R - 1e-3f;
-                hi[k] = u + R + 1e-3f;
-              }
-              const float mn = region_min(O, lo, hi);
-              active = !(mn - r - dtV * (1.0f + 1e-5f) - (1e-6f + 1e-5f * fabsf(mn)) > 0.0f);
+            if (l >= 0) {
+              const float lb = sphere_bound<ANY>(O, S.frame4[l], __ldg(H.chunk_sphere + j));
+              active = !(lb - r - dtV * (1.0f + 1e-5f) > 0.0f);
             }
             if (MODE == kModeWrench && !active && a.bits) {
 #pragma unroll 1

@@ -234,3 +234,50 @@ def test_quality_ragged_hand(fg):
     bad = torch.tensor([0, 5], device=_dev(), dtype=torch.int32)
     eb, nb = fg.grasp_epsilon(hand, scene, q[:2], TAU, MU, EDGES, 20.0, torch.tensor(U, device=_dev()), obj_of_cand=bad)
     assert np.isnan(eb.cpu().numpy()[1]) and nb.cpu().numpy()[1] == -1
+
+
+@pytest.mark.parametrize("edges", [1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16, 20, 31, 32])
+@pytest.mark.parametrize("n_dirs", [1, 63, 300, 1100])
+def test_epsilon_every_cone_and_direction_count(fg, batch, edges, n_dirs):
+    """Cone edges of each symmetry (odd, even, multiples of 4) and direction counts on both sides of the
+    threads x directions split (one direction; contacts dealt out to several thread groups; two passes)."""
+    w, hand, scene, S, ok = batch[1]
+    U = synth.unit_directions(n_dirs)
+    q = torch.tensor(w.q0, device=_dev())
+    oc = torch.tensor(w.obj_of_cand, device=_dev(), dtype=torch.int32)
+    eps, nc = fg.grasp_epsilon(hand, scene, q, TAU, MU, edges, 20.0, torch.tensor(U, device=_dev()), obj_of_cand=oc)
+    eps, nc = eps.cpu().numpy().astype(np.float64), nc.cpu().numpy()
+    checked = 0
+    for b in np.nonzero(ok)[0]:
+        p, n, phi, idx = Q.contacts(S.hand, S.objs[int(w.obj_of_cand[b])], w.q0[b], TAU)
+        assert nc[b] == len(p)
+        ref = Q.support_min(Q.cone_wrenches(p, n, MU, edges, 0.05), U.astype(np.float64))
+        assert _eps_close(np.array([eps[b]]), np.array([ref]))[0], (b, eps[b], ref)
+        checked += len(p) > 0
+    assert checked >= 3
+
+
+@pytest.mark.parametrize("points_per_link,tau", [(64, 0.2), (256, 0.05), (900, 0.005)])
+def test_quality_many_contacts_and_large_hands(fg, points_per_link, tau):
+    """Every point a contact (several batches of 32 chunks), thousands of contacts, and a hand of 9,000 points,
+    whose chunks are not culled."""
+    w = synth.tiny_sphere_workload(n_cand=6)
+    h = synth.make_hand(3, points_per_link)
+    qs = synth.sample_candidates(np.random.default_rng(11), h, 6, 0.095)
+    hand = fg.Hand.from_synth(h)
+    scene = fg.Scene([fg.Sdf.from_synth(o) for o in w.objects])
+    S = O.Setup(h, w.objects, w.params)
+    q = torch.tensor(qs, device=_dev())
+    U = synth.unit_directions(96)
+    ca = fg.contact_measure(hand, scene, q, torch.tensor(h["point_area"], device=_dev()), tau).cpu().numpy()
+    eps, nc = fg.grasp_epsilon(hand, scene, q, tau, MU, EDGES, 20.0, torch.tensor(U, device=_dev()))
+    eps, nc = eps.cpu().numpy().astype(np.float64), nc.cpu().numpy()
+    for b in range(len(qs)):
+        p, n, phi, idx = Q.contacts(S.hand, S.objs[0], qs[b], tau)
+        ref_ca = Q.measure(S.hand, S.objs[0], qs[b], h["point_area"], tau)
+        slack = 4 * float(np.max(h["point_area"]))          # a few points may sit within rounding of the threshold
+        assert abs(int(nc[b]) - len(p)) <= 4, (nc[b], len(p))
+        assert abs(float(ca[b]) - ref_ca) <= 1e-5 * max(ref_ca, 1e-6) + slack
+        if len(p) and nc[b] == len(p):
+            ref = Q.support_min(Q.cone_wrenches(p, n, MU, EDGES, 0.05), U.astype(np.float64))
+            assert abs(eps[b] - ref) <= 1e-4 + 1e-4 * abs(ref), (b, eps[b], ref)
