@@ -226,12 +226,12 @@ __device__ __forceinline__ void point_adjoint_pair(const HandDev& H, const float
   }
 }
 
-// Sums a[0..5] over the 32 lanes in a fixed pattern and stores the 6 totals in
-// slot.  Eight values (6 and two zeros) are halved across lanes at each exchange
+// Sums a[0..5] over the 32 lanes in a fixed pattern; lane 4k returns the total of
+// value k.  Eight values (6 and two zeros) are halved across lanes at each exchange
 // (xor 16, 8, 4: a lane keeps half of its values and adds its partner's copy of
-// them), then the last value is summed over groups of 4; lane 4k ends with the
-// total of value k.  The order of additions never depends on timing.
-__device__ __forceinline__ void unit_reduce_store(const float a[6], int lane, float* slot) {
+// them), then the last value is summed over groups of 4.  The order of additions
+// never depends on timing.
+__device__ __forceinline__ float unit_reduce(const float a[6], int lane) {
   const float v[8] = {a[0], a[1], a[2], a[3], a[4], a[5], 0.0f, 0.0f};
   const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0, h4 = (lane & 4) != 0;
   float w4[4], w2[2];
@@ -250,8 +250,18 @@ __device__ __forceinline__ void unit_reduce_store(const float a[6], int lane, fl
   float w = (h4 ? w2[1] : w2[0]) + __shfl_xor_sync(kFull, h4 ? w2[0] : w2[1], 4);
   w += __shfl_xor_sync(kFull, w, 2);
   w += __shfl_xor_sync(kFull, w, 1);
+  return w;
+}
+// The 6 totals stored in, or added to, slot[0..5].
+__device__ __forceinline__ void unit_reduce_store(const float a[6], int lane, float* slot) {
+  const float w = unit_reduce(a, lane);
   const int k = lane >> 2;
   if ((lane & 3) == 0 && k < 6) slot[k] = w;
+}
+__device__ __forceinline__ void unit_reduce_add(const float a[6], int lane, float* slot) {
+  const float w = unit_reduce(a, lane);
+  const int k = lane >> 2;
+  if ((lane & 3) == 0 && k < 6) slot[k] += w;
 }
 
 // Fixed point with 44 fractional bits: every force and torque sum here is far
@@ -261,27 +271,9 @@ __device__ __forceinline__ unsigned long long to_fixed(float v) {
 }
 __device__ __forceinline__ float from_fixed(long long x) { return __fmul_rn(__ll2float_rn(x), 0x1p-44f); }
 
-// The warp's sums of a[0..5] (the fixed pattern of unit_reduce_store) added in
-// fixed point to slot[0..5]: lane 4k holds the total of value k.
+// The warp's sums of a[0..5] (unit_reduce) added in fixed point to slot[0..5].
 __device__ __forceinline__ void unit_reduce_add_fixed(const float a[6], int lane, unsigned long long* slot) {
-  const float v[8] = {a[0], a[1], a[2], a[3], a[4], a[5], 0.0f, 0.0f};
-  const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0, h4 = (lane & 4) != 0;
-  float w4[4], w2[2];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float send = h16 ? v[j] : v[4 + j];
-    const float keep = h16 ? v[4 + j] : v[j];
-    w4[j] = keep + __shfl_xor_sync(kFull, send, 16);
-  }
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const float send = h8 ? w4[j] : w4[2 + j];
-    const float keep = h8 ? w4[2 + j] : w4[j];
-    w2[j] = keep + __shfl_xor_sync(kFull, send, 8);
-  }
-  float w = (h4 ? w2[1] : w2[0]) + __shfl_xor_sync(kFull, h4 ? w2[0] : w2[1], 4);
-  w += __shfl_xor_sync(kFull, w, 2);
-  w += __shfl_xor_sync(kFull, w, 1);
+  const float w = unit_reduce(a, lane);
   const int k = lane >> 2;
   if ((lane & 3) == 0 && k < 6) atomicAdd(slot + k, to_fixed(w));
 }

@@ -157,3 +157,24 @@ def test_tstep_is_refused_where_only_the_one_step_metric_exists(fg, tiny):
     for bad in (-1, 9):
         with pytest.raises(_lib.FgError):
             fg.loss_and_grad(tiny.hand, tiny.scene, q, dict(w.params, sim_steps=bad), 0.004)
+
+
+@pytest.mark.parametrize("T", [1, 2])
+@pytest.mark.parametrize("points_per_link", [21, 100, 1300])
+def test_tstep_ragged_and_large_hands(fg, T, points_per_link):
+    """Links whose points are not 32-aligned (chunks across links, work units of 21 and 36 points) and a hand of
+    13,000 points, more than the first step's unit table and the chunk culling take."""
+    w = synth.tiny_sphere_workload(n_cand=12)
+    h = synth.make_hand(3, points_per_link)
+    qs = synth.sample_candidates(np.random.default_rng(7), h, 12, 0.095)
+    case = Case(fg, synth.Workload("ragged", h, w.objects, qs, np.zeros(12, dtype=np.int32), w.params, 10))
+    params = dict(w.params, sim_steps=T)
+    S = case.oracle(params)
+    q = torch.tensor(qs, device=_dev())
+    loss, grad = fg.loss_and_grad(case.hand, case.scene, q, params, 0.004)
+    ref = O.batch_loss_and_grad(S, qs, case.w.obj_of_cand, 0.004)
+    clean = case.clean(S, qs, 0.004)
+    assert clean.sum() >= 1
+    _compare(loss.cpu().numpy(), grad.cpu().numpy(), ref, clean)
+    l2, g2 = fg.loss_and_grad(case.hand, case.scene, q, params, 0.004)
+    assert torch.equal(loss, l2) and torch.equal(grad, g2)
