@@ -464,6 +464,7 @@ fg_status fg_contact_wrench(const fg_hand* h, const fg_scene* sc, const int* oc,
   FusedArgs a{};
   a.hand = h->dev;
   a.hand_D = h->host.D;
+  a.hand_P = h->host.P;
   a.objs = sc->dev;
   a.n_obj = sc->n;
   a.any_mesh = sc->has_mesh;
@@ -492,6 +493,7 @@ fg_status fg_loss_and_grad(const fg_hand* h, const fg_scene* sc, const int* oc, 
   FusedArgs a{};
   a.hand = h->dev;
   a.hand_D = h->host.D;
+  a.hand_P = h->host.P;
   a.objs = sc->dev;
   a.n_obj = sc->n;
   a.any_mesh = sc->has_mesh;
@@ -526,6 +528,7 @@ fg_status fg_optimize_step(const fg_hand* h, const fg_scene* sc, const int* oc, 
   FusedArgs a{};
   a.hand = h->dev;
   a.hand_D = h->host.D;
+  a.hand_P = h->host.P;
   a.objs = sc->dev;
   a.n_obj = sc->n;
   a.any_mesh = sc->has_mesh;
@@ -580,6 +583,7 @@ fg_status fg_contact_measure(const fg_hand* h, const fg_scene* sc, const int* oc
   FusedArgs a{};
   a.hand = h->dev;
   a.hand_D = h->host.D;
+  a.hand_P = h->host.P;
   a.objs = sc->dev;
   a.n_obj = sc->n;
   a.any_mesh = sc->has_mesh;
@@ -605,6 +609,7 @@ fg_status fg_grasp_epsilon(const fg_hand* h, const fg_scene* sc, const int* oc, 
   FusedArgs a{};
   a.hand = h->dev;
   a.hand_D = h->host.D;
+  a.hand_P = h->host.P;
   a.objs = sc->dev;
   a.n_obj = sc->n;
   a.any_mesh = sc->has_mesh;
@@ -676,6 +681,7 @@ fg_status fg_autotune(const fg_hand* h, const fg_scene* sc, const int* oc, const
   FusedArgs a{};
   a.hand = h->dev;
   a.hand_D = h->host.D;
+  a.hand_P = h->host.P;
   a.objs = sc->dev;
   a.n_obj = sc->n;
   a.any_mesh = sc->has_mesh;

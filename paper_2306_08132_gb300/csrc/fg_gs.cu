@@ -50,9 +50,11 @@ namespace fg {
 
 namespace {
 
-constexpr int kGW = kSims;                    // one warp per simulation
+constexpr int kGW = kSims;                    // warps of a candidate: one per simulation
+constexpr int kGWMesh = 2 * kSims;            // scenes with mesh objects: the search and the adjoint take twice as many
 constexpr int kSnapWords = 14;                // per chunk and simulation: state (6), adjoint (6), event mask, pad
 
+template <int GW>
 struct GsSmem {
   HandDev H;
   ObjDev O;
@@ -65,9 +67,10 @@ struct GsSmem {
   float sfin[kSims][6];            // final state per simulation
   __align__(8) float afin[kSims][6];   // dL/d(final state)
   float red[kSims][8];             // per simulation: sum f (3), sum d x f (3), contacts, penetration
-  float lacc[kGW][kMaxLinks][6];   // per warp, per link: sum g, sum (p - t) x g
+  float lacc[GW][kMaxLinks][6];    // per warp, per link: sum g, sum (p - t) x g
   float loss;
   int cand;                        // the candidate claimed by this CTA
+  int next_chunk;                  // closest-face search: next unclaimed chunk
   int bad_object;
   const HandDev* hand_loaded;
 };
@@ -409,10 +412,20 @@ __device__ __forceinline__ void gs_chunk_reverse(const PointState& ps, const flo
   }
 }
 
+// Lookup of point i: from its closest face when the faces are kept (mesh objects).
+template <bool kHess, bool ANY>
+__device__ __forceinline__ void gs_lookup(const ObjDev& O, const float p[3], const int* faces, int i, SdfSample& smp) {
+  if (ANY && faces != nullptr)
+    mesh_eval(O, p, faces[i], smp);
+  else
+    sdf_lookup<kHess, ANY>(O, p, smp);
+}
+
 // ANY = false: grid objects only; true: grids and meshes (the lookup dispatches on the kind).
 template <int MODE, bool ANY>
-__global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
-  __shared__ GsSmem S;
+__global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_kernel(FusedArgs a) {
+  constexpr int GW = ANY ? kGWMesh : kGW;
+  __shared__ GsSmem<GW> S;
   extern __shared__ float dyn[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) S.hand_loaded = nullptr;
@@ -431,7 +444,7 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
     if (a.hand != S.hand_loaded) {              // uniform: every thread reads the same words
       const int* src = reinterpret_cast<const int*>(a.hand);
       int* dst = reinterpret_cast<int*>(&S.H);
-      for (int k = tid; k < (int)(sizeof(HandDev) / sizeof(int)); k += kGW * 32) dst[k] = src[k];
+      for (int k = tid; k < (int)(sizeof(HandDev) / sizeof(int)); k += GW * 32) dst[k] = src[k];
     }
     __syncthreads();
     if (tid == 0) S.hand_loaded = a.hand;
@@ -441,7 +454,7 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
     if (S.bad_object) {
       const float nan = __int_as_float(0x7fc00000);
       if (MODE == kModeWrench) {
-        for (int idx = tid; idx < kSims * 6; idx += kGW * 32) a.wrench[(size_t)c * kSims * 6 + idx] = nan;
+        for (int idx = tid; idx < kSims * 6; idx += GW * 32) a.wrench[(size_t)c * kSims * 6 + idx] = nan;
         if (tid < kSims) a.ncontact[(size_t)c * kSims + tid] = -1;
       } else if (MODE == kModeLossGrad) {
         if (tid == 0) a.loss[c] = nan;
@@ -458,7 +471,8 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
       const float r = MODE == kModeOptimize ? dilation_at(Pm, a.step0 + s, a.total_steps) : a.r_fixed;
       __syncthreads();
       if (warp == 0) fk_warp(H, S.q, S.frame4, lane);
-      for (int idx = tid; idx < kGW * kMaxLinks * 6; idx += kGW * 32) (&S.lacc[0][0][0])[idx] = 0.0f;
+      for (int idx = tid; idx < GW * kMaxLinks * 6; idx += GW * 32) (&S.lacc[0][0][0])[idx] = 0.0f;
+      if (tid == 0) S.next_chunk = 0;
       __syncthreads();
 
       // ------------------------------------------------- chunk bounds (culling)
@@ -466,7 +480,40 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
       // the interpolated field over the sphere's box is bounded below by the
       // min-pyramid, so phi_hat >= lb = min - r over the chunk.  For a mesh: if the
       // centre is outside at flat distance d > R, rho >= d - R - (the Phong shift bound).
-      for (int j = tid; j < nch; j += kGW * 32) {
+      // A mesh object whose adjoint follows has every point's closest face searched here,
+      // once, by all warps (each later lookup evaluates from the face, where the seven
+      // simulations' walks used to search again), and lb is the chunk's smallest phi_hat itself.
+      // GS_8 objects x 128 candidates of 4,352 points, 2,208 faces
+      // each: 3.7-4.6 -> 2.6 ms, with 16 warps a candidate 1.3-1.7 ms.
+      int* faces = nullptr;
+      if (ANY && MODE != kModeWrench && O.kind == kObjMesh && P <= a.face_cap && (MODE == kModeOptimize || a.grad != nullptr))
+        faces = reinterpret_cast<int*>(dyn + (size_t)nch * kSims * kSnapWords);
+      if (ANY && faces != nullptr) {
+        for (;;) {
+          int j = 0;
+          if (lane == 0) j = atomicAdd(&S.next_chunk, 1);
+          j = __shfl_sync(kFull, j, 0);
+          if (j >= nch) break;
+          const int i = 32 * j + lane;
+          const bool valid = i < P;
+          const float4 sp = __ldg(H.pts + (valid ? i : 32 * j));
+          float p[3];
+          world_point(S.frame4[(int)sp.w], sp, p);
+          const int f = mesh_find(O, p);
+          if (valid) faces[i] = f;
+          SdfSample smp;
+          mesh_eval(O, p, f, smp);
+          float mn = sub_(smp.phi, r), far = sqrtf(p[0] * p[0] + p[1] * p[1] + p[2] * p[2]);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            mn = fminf(mn, __shfl_xor_sync(kFull, mn, o));
+            far = fmaxf(far, __shfl_xor_sync(kFull, far, o));
+          }
+          if (lane == 0) S.lb[j] = mn;
+          if (lane < kSims) S.reach[j][lane] = far + dtV;
+        }
+      } else
+      for (int j = tid; j < nch; j += GW * 32) {
         const int l = H.chunk_link[j];
         float lbj = -3.0e38f;
         float4 cwj = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -510,7 +557,7 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
       __syncthreads();
 
       // ------------------------------------------------------------- forward
-      {
+      if (GW == kSims || warp < kSims) {
         const int m = warp;
         float xt[3];
         sim_pred(m, dtV, xt);
@@ -565,7 +612,7 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
           }
           if (!__all_sync(kFull, clear)) {
             SdfSample smp;
-            sdf_lookup<false, ANY>(O, p, smp);
+            gs_lookup<false, ANY>(O, p, faces, valid ? i : 32 * jn, smp);
             PointState ps;
             point_state(smp, p, r, ps);
             int last = -1;
@@ -616,11 +663,11 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
       __syncthreads();
       if (MODE == kModeWrench) {
         // the sums of the corrections applied, the points projected, and their lanes per chunk
-        for (int idx = tid; idx < kSims * 6; idx += kGW * 32)
+        for (int idx = tid; idx < kSims * 6; idx += GW * 32)
           a.wrench[(size_t)c * kSims * 6 + idx] = S.red[idx / 6][idx % 6];
         if (tid < kSims) a.ncontact[(size_t)c * kSims + tid] = (int)S.red[tid][6];
         if (a.bits)
-          for (int idx = tid; idx < kSims * nch; idx += kGW * 32) {
+          for (int idx = tid; idx < kSims * nch; idx += GW * 32) {
             const int m = idx / nch, j = idx - m * nch;
             a.bits[((size_t)c * kSims + m) * nch + j] = __float_as_uint(snap(dyn, j, m)[12]);
           }
@@ -687,7 +734,7 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
       int cur = -1;
       float acc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
       const float t0[3] = {S.q[0], S.q[1], S.q[2]};
-      {
+      if (GW == kSims || warp < kSims) {
         const int m = warp;
         float xt[3];
         sim_pred(m, dtV, xt);
@@ -719,7 +766,7 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
             float p[3];
             world_point(S.frame4[link], sp, p);
             SdfSample smp;
-            sdf_lookup<true, ANY>(O, p, smp);
+            gs_lookup<true, ANY>(O, p, faces, valid ? i : 32 * je, smp);
             PointState ps;
             point_state(smp, p, r, ps);
             float st0[6], smine[6], amine[6], dphi = 0.0f, dn[3] = {0.0f, 0.0f, 0.0f}, dp[3] = {0.0f, 0.0f, 0.0f};
@@ -749,7 +796,7 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
 
       // ----------------------------------------------- adjoint of every point
       {
-        for (int j = warp; j < nch; j += kGW) {
+        for (int j = warp; j < nch; j += GW) {
           const int i = 32 * j + lane;
           const bool valid = i < P;
           const float4 sp = __ldg(H.pts + (valid ? i : 32 * j));
@@ -757,7 +804,7 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
           float p[3];
           world_point(S.frame4[link], sp, p);
           SdfSample smp;
-          sdf_lookup<true, ANY>(O, p, smp);
+          gs_lookup<true, ANY>(O, p, faces, valid ? i : 32 * j, smp);
           PointState ps;
           point_state(smp, p, r, ps);
           float dphi = 0.0f, dn[3] = {0.0f, 0.0f, 0.0f}, dp[3] = {0.0f, 0.0f, 0.0f};
@@ -821,7 +868,7 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
           float x = 0.0f;
           if (lane < L) {
 #pragma unroll
-            for (int w = 0; w < kGW; ++w) x += S.lacc[w][lane][k];
+            for (int w = 0; w < GW; ++w) x += S.lacc[w][lane][k];
           }
 #pragma unroll
           for (int o = 1; o < 32; o <<= 1) {
@@ -881,7 +928,10 @@ __global__ void __launch_bounds__(kGW * 32, 3) gs_kernel(FusedArgs a) {
 
 template <int MODE, bool ANY>
 cudaError_t launch_gs_mode(const FusedArgs& a, int nchunks, cudaStream_t st) {
-  const size_t dyn = sizeof(float) * (size_t)nchunks * kSims * kSnapWords;
+  constexpr int GW = ANY ? kGWMesh : kGW;
+  FusedArgs b = a;
+  b.face_cap = ANY && MODE != kModeWrench ? a.hand_P : 0;          // nchunks <= kMaxCullChunks: at most 32 KB
+  const size_t dyn = sizeof(float) * ((size_t)nchunks * kSims * kSnapWords + b.face_cap);
   static size_t attr_set[64] = {0};
   int dev = 0;
   cudaGetDevice(&dev);
@@ -891,16 +941,15 @@ cudaError_t launch_gs_mode(const FusedArgs& a, int nchunks, cudaStream_t st) {
     attr_set[dev & 63] = dyn;
   }
   int bps = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, gs_kernel<MODE, ANY>, kGW * 32, dyn);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, gs_kernel<MODE, ANY>, GW * 32, dyn);
   if (e != cudaSuccess) return e;
   if (bps < 1) bps = 1;
   long long grid = (long long)device_sm_count() * bps;
   if (grid > a.B) grid = a.B;
   if (grid < 1) return cudaSuccess;
-  FusedArgs b = a;
   e = work_pair(&b.work, st);
   if (e != cudaSuccess) return e;
-  gs_kernel<MODE, ANY><<<(int)grid, kGW * 32, dyn, st>>>(b);
+  gs_kernel<MODE, ANY><<<(int)grid, GW * 32, dyn, st>>>(b);
   return cudaGetLastError();
 }
 

@@ -78,6 +78,8 @@ struct FusedArgs {
   int* ncontact;
   uint32_t* bits;
   int hand_D;
+  int hand_P;                  // points of the hand (queue mode: of the round's largest hand); 0 when not given
+  int face_cap;                // closest faces kept per candidate in shared memory (set by the launcher)
   const QueueSlotDev* slots;   // queue mode: slot table (device), sorted by cand_start
   int nslots;
   int any_mesh;                // some object is a mesh: the kernels with the mesh lookup

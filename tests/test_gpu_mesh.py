@@ -369,3 +369,34 @@ def test_mesh_full_size_sampled_parity(fg):
     assert clean.sum() >= 2
     step = ((q1 - q).cpu().numpy()[sample]).astype(np.float64) / -w.params["lr"]
     _compare(loss.cpu().numpy()[sample], step, ref, clean)
+
+
+@pytest.mark.parametrize("gauss_seidel", [0, 1])
+@pytest.mark.parametrize("points_per_link", [21, 128])
+def test_mesh_kept_faces_equal_searched_ones(fg, gauss_seidel, points_per_link):
+    """With a gradient the closest faces are searched once and kept; the loss alone searches per culled chunk.
+    The loss is the same either way (one lookup of the same face), on ragged and aligned links; a torus's inner
+    half and points inside the mesh take the BVH walk."""
+    w = synth.tiny_sphere_workload(n_cand=24)
+    h = synth.make_hand(3, points_per_link)
+    qs = synth.sample_candidates(np.random.default_rng(9), h, 24, 0.07)
+    for mesh in (SM.icosphere(0.04, 2), SM.torus_mesh(0.04, 0.015, 16, 8)):
+        c = Case(fg, h, [mesh], np.zeros(24, dtype=np.int32), qs, w.params)
+        params = dict(w.params, gauss_seidel=gauss_seidel)
+        q = torch.tensor(qs, device=_dev())
+        loss, grad = fg.loss_and_grad(c.hand, c.scene, q, params, 0.004)
+        alone, none = fg.loss_and_grad(c.hand, c.scene, q, params, 0.004, want_grad=False)
+        assert none is None and torch.isfinite(grad).all()
+        assert torch.allclose(loss, alone, rtol=1e-5, atol=1e-7), float((loss - alone).abs().max())
+
+
+def test_mesh_hand_beyond_the_kept_faces(fg):
+    """A hand of 8,400 points: its faces are not kept, both sweeps search."""
+    w = synth.tiny_sphere_workload(n_cand=3)
+    h = synth.make_hand(3, 840)
+    qs = synth.sample_candidates(np.random.default_rng(9), h, 3, 0.095)
+    c = Case(fg, h, [SM.icosphere(0.04, 2)], np.zeros(3, dtype=np.int32), qs, w.params)
+    loss, grad = fg.loss_and_grad(c.hand, c.scene, torch.tensor(qs, device=_dev()), w.params, 0.004)
+    ref = O.batch_loss_and_grad(c.S, qs, c.oc_np, 0.004)
+    assert np.all(np.abs(loss.cpu().numpy() - ref["L"]) <= 1e-3 * np.abs(ref["L"]) + 1e-4)
+    assert torch.isfinite(grad).all()
