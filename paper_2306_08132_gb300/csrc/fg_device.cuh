@@ -227,22 +227,41 @@ struct SdfIndex {
   const float* cell;   // corner (i0, j0, k0)
 };
 
+// Index along one axis: the clamped cell, the fraction in it and the excess u - u_c.
+struct AxisIndex {
+  float f, du;
+  int i;
+  bool clamped;
+};
+__device__ __forceinline__ AxisIndex sdf_axis(const ObjDev& O, int k, float x) {
+  const float n_max = (float)((k == 0 ? O.nx : k == 1 ? O.ny : O.nz) - 1);
+  AxisIndex a;
+  const float u = fma_(x, O.inv_h, O.uo[k]);
+  const float uc = fminf(fmaxf(u, 0.0f), n_max);        // NaN -> 0
+  a.clamped = uc != u;
+  a.du = sub_(u, uc);                                   // 0 unless clamped
+  const int ii = __float2int_rd(uc);                    // floor (uc >= 0)
+  const int cap = (int)n_max - 1;
+  a.i = ii < cap ? ii : cap;
+  a.f = sub_(uc, (float)a.i);
+  return a;
+}
+// fewer than 2^31 nodes per grid (checked at creation): the index fits 32 bits
+__device__ __forceinline__ const float* sdf_cell(const ObjDev& O, int i, int j, int k) {
+  return O.grid + (unsigned)((k * O.ny + j) * O.nx + i);
+}
+
 __device__ __forceinline__ void sdf_index(const ObjDev& O, const float p[3], SdfIndex& ix) {
-  const float n_max[3] = {(float)(O.nx - 1), (float)(O.ny - 1), (float)(O.nz - 1)};
   int i0[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const float u = fma_(p[k], O.inv_h, O.uo[k]);
-    const float uc = fminf(fmaxf(u, 0.0f), n_max[k]);     // NaN -> 0
-    ix.clamped[k] = uc != u;
-    ix.du[k] = sub_(u, uc);                               // 0 unless clamped
-    const int ii = __float2int_rd(uc);                   // floor (uc >= 0)
-    const int cap = (int)n_max[k] - 1;
-    i0[k] = ii < cap ? ii : cap;
-    ix.f[k] = sub_(uc, (float)i0[k]);
+    const AxisIndex a = sdf_axis(O, k, p[k]);
+    ix.clamped[k] = a.clamped;
+    ix.du[k] = a.du;
+    ix.f[k] = a.f;
+    i0[k] = a.i;
   }
-  // fewer than 2^31 nodes per grid (checked at creation): the index fits 32 bits
-  ix.cell = O.grid + (unsigned)((i0[2] * O.ny + i0[1]) * O.nx + i0[0]);
+  ix.cell = sdf_cell(O, i0[0], i0[1], i0[2]);
 }
 
 __device__ __forceinline__ void sdf_gather(const ObjDev& O, const float* G, float c[8]) {

@@ -362,18 +362,66 @@ __device__ __forceinline__ void first_forward_chunk(const ObjDev& O, const Param
 //   |d x t|^2 = sg^2 + (U_k/rho)^2,   gf . t = s (gf_k - n_k (gf . n))/rho
 // (gf = Gl + Ga x d).  Simulations in which some lane of the warp is in contact go
 // through the general adjoint afterwards, for those lanes.
-template <bool ANY>
+//
+// NEAR: the queries lie at most one cell from the point (near_queries), so along each
+// axis they read the point's own cell or the next one: the 8 corners are read once and
+// a moved query replaces one plane of 4 where it has left the cell, 8 + 6 x 4 predicated loads
+// a point instead of 56.  Same batch: 1.86 -> 1.54 ms, L1 data pipe 72% -> 49%; the four warps a
+// scheduler that 128 registers leave no longer cover the latencies.
+template <bool ANY, bool NEAR>
 __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const ParamsDev& Pm, const float (*G)[6],
                                                     const float p[3], bool valid, float rdil, float c, float pb[3]) {
   pb[0] = pb[1] = pb[2] = 0.0f;
   unsigned touch = 0u;
   const float mu = c > 0.0f ? Pm.mu : 0.0f;      // no displacement, no friction
+  SdfIndex ix;
+  int cell[3];
+  float c0[8];
+  if constexpr (NEAR) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const AxisIndex a = sdf_axis(O, k, p[k]);
+      ix.f[k] = a.f;
+      ix.du[k] = a.du;
+      ix.clamped[k] = a.clamped;
+      cell[k] = a.i;
+    }
+    ix.cell = sdf_cell(O, cell[0], cell[1], cell[2]);
+    sdf_gather(O, ix.cell, c0);
+  }
 #pragma unroll
   for (int m = 0; m < kSims; ++m) {
     float r[3];
     first_query(p, m, c, r);
     SdfSample smp;
-    sdf_lookup<false, ANY>(O, r, smp);
+    if constexpr (NEAR) {
+      SdfIndex q = ix;
+      float cc[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) cc[e] = c0[e];
+      if (m > 0) {
+        // the query moves against the velocity: down for m odd, up for m even
+        const int k = sim_axis(m);
+        const bool down = m & 1;
+        const AxisIndex a = sdf_axis(O, k, r[k]);
+        q.f[k] = a.f;
+        q.du[k] = a.du;
+        q.clamped[k] = a.clamped;
+        const bool moved = a.i != cell[k];
+        const int st[3] = {1, O.nx, O.nx * O.ny}, u = (k + 1) % 3, v = (k + 2) % 3;
+        const float* E = ix.cell + (down ? -st[k] : 2 * st[k]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int lo = ((e & 1) << u) | ((e >> 1) << v), hi = lo | (1 << k);
+          const float x = moved ? __ldg(E + (e & 1) * st[u] + (e >> 1) * st[v]) : 0.0f;
+          cc[lo] = moved ? (down ? x : c0[hi]) : c0[lo];
+          cc[hi] = moved ? (down ? c0[lo] : x) : c0[hi];
+        }
+      }
+      sdf_finish<false>(O, q, cc, smp);
+    } else {
+      sdf_lookup<false, ANY>(O, r, smp);
+    }
     PointState ps;
     point_state(smp, r, rdil, ps);
     const float* n = ps.n;
@@ -422,6 +470,12 @@ __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const Param
   }
 }
 
+// Whether every query p - s c e_k lies within one cell of p: c below the pitch, with room for
+// the rounding of the index coordinates (below 2^12 + 1 nodes an axis, 2^-11 cells).
+__device__ __forceinline__ bool near_queries(const ObjDev& O, float c) {
+  return O.kind == kObjGrid && c * O.inv_h < 0.998f && max(O.nx, max(O.ny, O.nz)) <= 4096;
+}
+
 // (g, (p - t0) x g) of one point, zero for a lane without one.
 __device__ __forceinline__ void point_wrench(const float p[3], const float t0[3], const float g[3], bool valid,
                                              float v[6]) {
@@ -438,7 +492,7 @@ __device__ __forceinline__ void point_wrench(const float p[3], const float t0[3]
 // The first step's reverse sweep: per-link sums of (g, (p - t0) x g), by work units
 // claimed from a counter (as in the one-step kernel), or by fixed ranges of points for
 // hands with more units than uacc holds.
-template <bool ANY>
+template <bool ANY, bool NEAR>
 __device__ __forceinline__ void first_reverse_sweep(TstepSmem& S, const ObjDev& O, float rdil, int lane, int warp) {
   const HandDev& H = S.H;
   const float c = mul_(S.Pm.dt, S.Pm.V);
@@ -457,7 +511,7 @@ __device__ __forceinline__ void first_reverse_sweep(TstepSmem& S, const ObjDev& 
         const float4 sp = __ldg(H.pts + (valid ? U.x + h + lane : U.x));
         float p[3], pb[3], v[6];
         world_point(S.frame4[U.z], sp, p);
-        first_reverse_point<ANY>(O, S.Pm, S.G, p, valid, rdil, c, pb);
+        first_reverse_point<ANY, NEAR>(O, S.Pm, S.G, p, valid, rdil, c, pb);
         point_wrench(p, t0, pb, valid, v);
 #pragma unroll
         for (int k = 0; k < 6; ++k) sum[k] += v[k];
@@ -475,7 +529,7 @@ __device__ __forceinline__ void first_reverse_sweep(TstepSmem& S, const ObjDev& 
       const int link = (int)sp.w;
       float p[3], pb[3], v[6];
       world_point(S.frame4[link], sp, p);
-      first_reverse_point<ANY>(O, S.Pm, S.G, p, valid, rdil, c, pb);
+      first_reverse_point<ANY, NEAR>(O, S.Pm, S.G, p, valid, rdil, c, pb);
       point_wrench(p, t0, pb, valid, v);
       link_accumulate(S.lacc[warp], lane, link, valid, v, cur, acc);
     }
@@ -747,7 +801,10 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
         }
         __syncthreads();
         if (t == 0) {               // the adjoint of the initial state is not needed
-          first_reverse_sweep<ANY>(S, O, rdil, lane, warp);
+          if (near_queries(O, mul_(dt, Pm.V)))
+            first_reverse_sweep<ANY, true>(S, O, rdil, lane, warp);
+          else
+            first_reverse_sweep<ANY, false>(S, O, rdil, lane, warp);
           __syncthreads();
           break;
         }

@@ -178,3 +178,24 @@ def test_tstep_ragged_and_large_hands(fg, T, points_per_link):
     _compare(loss.cpu().numpy(), grad.cpu().numpy(), ref, clean)
     l2, g2 = fg.loss_and_grad(case.hand, case.scene, q, params, 0.004)
     assert torch.equal(loss, l2) and torch.equal(grad, g2)
+
+
+@pytest.mark.parametrize("T", [1, 2])
+@pytest.mark.parametrize("nodes,pitch,v_test", [(63, 0.002, 1.0), (126, 0.001003, 1.0), (126, 0.001, 1.0),
+                                                (140, 0.0009, 1.0), (63, 0.002, 0.0), (40, 0.002, 1.0)])
+def test_tstep_pitch_against_the_displacement(fg, T, nodes, pitch, v_test):
+    """The first step's queries lie dt V = 1 mm from the point: below one cell (corners shared by the
+    simulations), at one cell, beyond it, at zero velocity, and on a grid smaller than the hand (clamped axes)."""
+    w = synth.tiny_sphere_workload(n_cand=24)
+    obj = synth.sphere_grid(0.03, nodes, pitch)
+    case = Case(fg, synth.Workload("pitch", w.hand, [obj], w.q0, w.obj_of_cand, w.params, 10))
+    params = dict(w.params, sim_steps=T, v_test=v_test)
+    S = case.oracle(params)
+    q = torch.tensor(w.q0, device=_dev())
+    loss, grad = fg.loss_and_grad(case.hand, case.scene, q, params, 0.012)
+    ref = O.batch_loss_and_grad(S, w.q0, w.obj_of_cand, 0.012)
+    clean = case.clean(S, w.q0, 0.012)
+    if v_test == 0.0:        # a candidate at rest without contacts has no stability gradient: nothing to divide by
+        clean &= ref["N"].reshape(len(clean), -1).sum(axis=1) > 0
+    assert clean.sum() >= 3
+    _compare(loss.cpu().numpy(), grad.cpu().numpy(), ref, clean)
