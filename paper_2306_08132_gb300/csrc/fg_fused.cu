@@ -16,6 +16,24 @@ static const int kCfgPPT[] = {FG_FUSED_CONFIGS(FG_CFG_PPT)};
 static const FusedLaunchFn kLossGradLaunch[] = {FG_FUSED_CONFIGS(FG_CFG_LOSSGRAD)};
 constexpr int kNumCfg = sizeof(kCfgNW) / sizeof(kCfgNW[0]);
 constexpr int kDefaultCfg = 1;   // 4 warps per candidate, >= 5 CTAs per SM, 1 point per thread
+constexpr int kCfg8 = 4;         // 8 warps, >= 3 CTAs per SM
+constexpr int kCfg16 = 11;       // 16 warps, >= 1 CTA per SM
+
+// Warps per candidate of a launch without a selected configuration.  With few
+// candidates the chip is filled by giving each more warps: 152 candidates of 4,352
+// points 0.181 ms with 4 warps, 0.119 with 8, 0.080 with 16; 456: 0.192, 0.136, 0.131;
+// 912: 0.275, 0.208, 0.229; 1,824: 0.360, 0.309, 0.394; 8,192: within 2% with 4 and 8.  A small hand has too few
+// chunks to share (640 points: 304 candidates 0.060, 0.049, 0.058; 1,216: 0.084,
+// 0.087, 0.139).  On a mesh a candidate inside the object costs many times the others, so more
+// warps shorten the end of the launch (2,208 faces: 1,024 candidates 2.57, 1.45, 1.33;
+// 4,096: 6.71, 4.59, 4.36; 8,192: 9.73, 7.56, 8.01).
+static int default_config(const FusedArgs& a) {
+  const long long sms = device_sm_count(), B = a.B;
+  const bool large = a.hand_P >= 2048;
+  if (a.any_mesh) return B <= 32 * sms ? kCfg16 : kCfg8;
+  if (B <= (large ? 3 : 1) * sms) return kCfg16;
+  return B <= (large ? 12 : 4) * sms ? kCfg8 : kDefaultCfg;
+}
 
 static int g_selected[64] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1,
                              -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1,
@@ -42,7 +60,7 @@ void fused_config_select(int i) { selected_slot() = i; }
 cudaError_t launch_fused(int mode, const FusedArgs& a, const fg_hand* h, cudaStream_t st) {
   (void)h;
   if (a.B <= 0) return cudaSuccess;
-  const int cfg = fused_config_current();
+  const int chosen = selected_slot(), cfg = chosen < 0 ? default_config(a) : chosen;
   if (a.any_mesh) {
     switch (mode) {
       case kModeWrench: return launch_wrench_any(a, st);

@@ -790,6 +790,6 @@ cudaError_t launch_fused_cfg(const FusedArgs& a, cudaStream_t st) {
 // warps per candidate, the minimum resident CTAs per SM the register
 // allocation is held to, and points per thread in the adjoint sweep.  The autotuner times them on a workload.
 // (warps per candidate, min CTAs per SM, points per thread per adjoint iteration)
-#define FG_FUSED_CONFIGS(X) X(4, 4, 1) X(4, 5, 1) X(4, 6, 1) X(4, 8, 1) X(8, 3, 1) X(2, 8, 1) X(4, 3, 2) X(4, 4, 2) X(4, 5, 2) X(8, 2, 2) X(4, 7, 1)
+#define FG_FUSED_CONFIGS(X) X(4, 4, 1) X(4, 5, 1) X(4, 6, 1) X(4, 8, 1) X(8, 3, 1) X(2, 8, 1) X(4, 3, 2) X(4, 4, 2) X(4, 5, 2) X(8, 2, 2) X(4, 7, 1) X(16, 1, 1)
 
 }  // namespace fg
