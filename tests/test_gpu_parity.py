@@ -338,3 +338,46 @@ def test_fp32_peak_kernel(fg):
     assert f2 == 2 * f1 and torch.isfinite(out).all()
     with pytest.raises(_lib.FgError):
         fg.fp32_peak_launch(out, False, 0)
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2), (2, 7, 3), (33, 5, 18)])
+def test_query_past_every_face_of_the_grid(fg, dims):
+    """Points inside, below and above the grid on each axis (27 regions) and at its first and last nodes: value and
+    gradient of the clamped interpolant plus the excess distance, in float64 numpy.  An index coordinate below 64
+    rounds by 2e-6; the value changes by at most 2 per cell along an axis (3 axes: 1.2e-5, plus rounding), a
+    derivative by at most 4/h per cell along each other axis (2 axes, h = 1/4: 6.4e-5, plus rounding)."""
+    rng = np.random.default_rng(3)
+    nx, ny, nz = dims
+    h, org = 0.25, np.array([0.5, -1.0, 0.125])                # exact in float32
+    G = rng.uniform(-1, 1, (nz, ny, nx)).astype(np.float32)
+    sdf = fg.Sdf(torch.tensor(G, device="cuda"), org, h, 1.0, 1.0)
+    u, smooth = [], []
+    for _ in range(8):
+        for r in np.ndindex(5, 5, 5):
+            n = np.array(dims) - 1.0
+            x = [(-rng.uniform(0.1, 3), 0.0, rng.integers(0, n[k]) + rng.uniform(0.1, 0.9), n[k], n[k] + rng.uniform(0.1, 3))[r[k]]
+                 for k in range(3)]
+            u.append(x)
+            smooth.append(all(v not in (1, 3) for v in r))
+    p = (org + h * np.array(u)).astype(np.float32)
+    phi, grad = fg.sdf_query(sdf, torch.tensor(p.T.copy(), device="cuda"), 0.0)
+    U = (p.astype(np.float64) - org) / h
+    n = np.array(dims) - 1.0
+    Uc = np.clip(U, 0, n)
+    i = np.minimum(np.floor(Uc), n - 1).astype(int)
+    f = Uc - i
+    c = np.array([[[G[i[:, 2] + dz, i[:, 1] + dy, i[:, 0] + dx] for dx in (0, 1)] for dy in (0, 1)] for dz in (0, 1)],
+                 dtype=np.float64)
+    w = [np.stack([1 - f[:, k], f[:, k]]) for k in range(3)]
+    val = np.einsum("zyxb,zb,yb,xb->b", c, w[2], w[1], w[0])
+    d = np.array([[-1.0], [1.0]]) * np.ones_like(w[0])
+    g = np.stack([np.einsum("zyxb,zb,yb,xb->b", c, w[2], w[1], d), np.einsum("zyxb,zb,yb,xb->b", c, w[2], d, w[0]),
+                  np.einsum("zyxb,zb,yb,xb->b", c, d, w[1], w[0])], 1) / h
+    ex = U - Uc
+    e = np.linalg.norm(ex, axis=1)
+    out = e > 0
+    g[ex != 0] = 0.0
+    g[out] += ex[out] / e[out, None]
+    assert np.abs(phi.cpu().numpy() - (val + h * e)).max() <= 1.5e-5
+    ok = np.array(smooth)
+    assert np.abs(grad.cpu().numpy().T - g)[ok].max() <= 1e-4
