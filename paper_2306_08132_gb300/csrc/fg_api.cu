@@ -331,9 +331,11 @@ fg_status fg_sdf_create(const float* grid, int nx, int ny, int nz, const float* 
   o.inv_h = 1.0f / pitch;
   o.inv_mass = 1.0f / mass;
   o.inv_inertia = 1.0f / inertia;
-  o.uo[0] = -origin[0] * o.inv_h;
-  o.uo[1] = -origin[1] * o.inv_h;
-  o.uo[2] = -origin[2] * o.inv_h;
+  o.axis = make_float4(o.inv_h, -origin[0] * o.inv_h, -origin[1] * o.inv_h, -origin[2] * o.inv_h);
+  o.n_max = make_float4((float)(nx - 1), (float)(ny - 1), (float)(nz - 1), pitch);
+  o.cap = make_int4(nx - 2, ny - 2, nz - 2, ny);
+  o.sy = nx;
+  o.sz = nx * ny;
   int levels = 0;
   const size_t pf = min_pyramid_floats(nx, ny, nz, &levels);
   s->pyr = nullptr;

@@ -48,14 +48,19 @@ constexpr int kMaxCullChunks = 256;
 
 constexpr int kMaxPyrLevels = 12;
 
-struct ObjDev {
+struct alignas(16) ObjDev {
+  // What a lookup reads for every point, as three 16-byte loads (in shared memory a
+  // 4-byte load costs the same wavefront).
+  float4 axis;                   // 1/pitch, then uo = -origin / pitch per axis: index coordinate u = p / pitch + uo
+  float4 n_max;                  // nx - 1, ny - 1, nz - 1 as floats, pitch
+  int4 cap;                      // nx - 2, ny - 2, nz - 2 (last cell), ny
   const float* grid;             // [nz][ny][nx]
+  int sy, sz;                    // strides nx, nx ny
   int nx, ny, nz;
   int pyr_levels;                // levels 1..pyr_levels of the min-pyramid
   float ox, oy, oz;              // origin
   float inv_h, h;                // 1/pitch, pitch
   float inv_mass, inv_inertia;
-  float uo[3];                   // -origin / pitch: index coordinate u = p / pitch + uo
   const float* pyr;              // min-pyramid, level k at pyr + pyr_off[k - 1]
   int pyr_off[kMaxPyrLevels];
   // kind 1: a watertight triangle mesh queried directly (Phong SDF); the grid
@@ -234,21 +239,21 @@ struct AxisIndex {
   bool clamped;
 };
 __device__ __forceinline__ AxisIndex sdf_axis(const ObjDev& O, int k, float x) {
-  const float n_max = (float)((k == 0 ? O.nx : k == 1 ? O.ny : O.nz) - 1);
+  const float4 ax = O.axis, nm = O.n_max;
+  const int4 cp = O.cap;
   AxisIndex a;
-  const float u = fma_(x, O.inv_h, O.uo[k]);
-  const float uc = fminf(fmaxf(u, 0.0f), n_max);        // NaN -> 0
+  const float u = fma_(x, ax.x, k == 0 ? ax.y : k == 1 ? ax.z : ax.w);
+  const float uc = fminf(fmaxf(u, 0.0f), k == 0 ? nm.x : k == 1 ? nm.y : nm.z);        // NaN -> 0
   a.clamped = uc != u;
   a.du = sub_(u, uc);                                   // 0 unless clamped
   const int ii = __float2int_rd(uc);                    // floor (uc >= 0)
-  const int cap = (int)n_max - 1;
-  a.i = ii < cap ? ii : cap;
+  a.i = min(ii, k == 0 ? cp.x : k == 1 ? cp.y : cp.z);
   a.f = sub_(uc, (float)a.i);
   return a;
 }
 // fewer than 2^31 nodes per grid (checked at creation): the index fits 32 bits
 __device__ __forceinline__ const float* sdf_cell(const ObjDev& O, int i, int j, int k) {
-  return O.grid + (unsigned)((k * O.ny + j) * O.nx + i);
+  return O.grid + (unsigned)(k * O.sz + j * O.sy + i);
 }
 
 __device__ __forceinline__ void sdf_index(const ObjDev& O, const float p[3], SdfIndex& ix) {
@@ -265,7 +270,7 @@ __device__ __forceinline__ void sdf_index(const ObjDev& O, const float p[3], Sdf
 }
 
 __device__ __forceinline__ void sdf_gather(const ObjDev& O, const float* G, float c[8]) {
-  const int sy = O.nx, sz = O.nx * O.ny;
+  const int sy = O.sy, sz = O.sz;
   c[0] = __ldg(G);
   c[1] = __ldg(G + 1);
   c[2] = __ldg(G + sy);
@@ -366,18 +371,9 @@ __device__ __forceinline__ void sdf_finish_pair(const ObjDev& O, const SdfIndex&
 // phi(p) >= the block's minimum.
 __device__ __forceinline__ float point_min_bound(const ObjDev& O, const float p[3]) {
   const int lev = O.pyr_levels >= 2 ? 2 : 1;
-  const float n_max[3] = {(float)(O.nx - 1), (float)(O.ny - 1), (float)(O.nz - 1)};
-  const int n[3] = {O.nx, O.ny, O.nz};
-  int b[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const float u = fma_(p[k], O.inv_h, O.uo[k]);
-    const float uc = fminf(fmaxf(u, 0.0f), n_max[k]);      // NaN -> 0
-    const int ii = __float2int_rd(uc);
-    const int cap = n[k] - 2;
-    b[k] = (ii < cap ? ii : cap) >> lev;
-  }
-  const int bx = ((n[0] - 1) + (1 << lev) - 1) >> lev, by = ((n[1] - 1) + (1 << lev) - 1) >> lev;
+  const int4 cp = O.cap;
+  const int b[3] = {sdf_axis(O, 0, p[0]).i >> lev, sdf_axis(O, 1, p[1]).i >> lev, sdf_axis(O, 2, p[2]).i >> lev};
+  const int bx = (cp.x >> lev) + 1, by = (cp.y >> lev) + 1;      // ceil((n - 1) / 2^lev)
   return __ldg(O.pyr + O.pyr_off[lev - 1] + (unsigned)((b[2] * by + b[1]) * bx + b[0]));
 }
 
@@ -1126,38 +1122,46 @@ __device__ __forceinline__ void sim_adjoint(const PointState& ps, int m, float p
 }
 
 // Constants of the simulation adjoint for one candidate step, in shared memory.
-// Scalar table (float index):  0 1/m, 1 1/I, 2 c = dt V, 3 c^2, 4 2c/I, 5 mu,
-// 6 alpha, 7 alpha c, 8 -c, 9 -mu, 10 -alpha c, 11 -w_pen, and for a candidate without
-// contacts, set by sim_constants_free: 12 2 g alpha, 13 -2 g alpha c, 14 -alpha w_pen.
-// The packed table holds each entry twice (a float2 per entry), so that a packed
-// operand is one shared-memory load.
-enum SimConst { kcA = 0, kcB, kcC, kcCC, kcTBC, kcMu, kcAlpha, kcAlphaC, kcMC, kcMMu, kcMAlphaC, kcMWpen, kcCount,
-                kcFree = kcCount, kcFreeN, kcFreePen };
-struct SimConsts {
+// Scalar table (float index), in groups of four read by one 16-byte load each:
+//   0  1/m, 1/I, c^2, 2c/I  (c = dt V)
+//   1  mu; for a candidate without contacts (sim_constants_free): 2 g alpha, -2 g alpha c, -alpha w_pen
+//   2  c, alpha, alpha c, -w_pen
+//   3  -c, -mu, -alpha c
+// The packed table holds each entry twice (a float2 per entry).
+struct alignas(16) SimConsts {
   float s[16];
   float2 p[16];
 };
+template <class V>
+struct SimK4 {
+  V x, y, z, w;
+};
 __device__ __forceinline__ void sim_constants(const ParamsDev& P, const ObjDev& O, SimConsts& K) {
   const float c = P.dt * P.V;
-  const float v[kcCount] = {O.inv_mass, O.inv_inertia, c, c * c, 2.0f * c * O.inv_inertia, P.mu, P.alpha,
-                            P.alpha * c, -c, -P.mu, -P.alpha * c, -P.w_pen};
+  const float v[16] = {O.inv_mass, O.inv_inertia, c * c, 2.0f * c * O.inv_inertia, P.mu, 0.0f, 0.0f, 0.0f,
+                       c, P.alpha, P.alpha * c, -P.w_pen, -c, -P.mu, -P.alpha * c, 0.0f};
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
-    const float x = k < kcCount ? v[k] : 0.0f;
-    K.s[k] = x;
-    K.p[k] = make_float2(x, x);
+    K.s[k] = v[k];
+    K.p[k] = make_float2(v[k], v[k]);
   }
 }
 __device__ __forceinline__ void sim_constants_free(const ParamsDev& P, float g, SimConsts& K) {
   const float v[3] = {2.0f * g * P.alpha, -2.0f * g * P.alpha * (P.dt * P.V), -P.alpha * P.w_pen};
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    K.s[kcFree + k] = v[k];
-    K.p[kcFree + k] = make_float2(v[k], v[k]);
+    K.s[5 + k] = v[k];
+    K.p[5 + k] = make_float2(v[k], v[k]);
   }
 }
-__device__ __forceinline__ float simk(const SimConsts& K, float, int k) { return K.s[k]; }
-__device__ __forceinline__ float2 simk(const SimConsts& K, float2, int k) { return K.p[k]; }
+__device__ __forceinline__ SimK4<float> simk4(const SimConsts& K, float, int j) {
+  const float4 v = reinterpret_cast<const float4*>(K.s)[j];
+  return {v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ SimK4<float2> simk4(const SimConsts& K, float2, int j) {
+  const float4 a = reinterpret_cast<const float4*>(K.p)[2 * j], b = reinterpret_cast<const float4*>(K.p)[2 * j + 1];
+  return {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y), make_float2(b.z, b.w)};
+}
 
 // Wrench adjoint of simulation m, (dL/dW_lin, dL/dW_ang), in shared memory:
 // scalar as (Gl, 0), (Ga, 0); packed with every component twice.
@@ -1238,7 +1242,8 @@ __device__ __forceinline__ void sim_axis_terms(const V n[3], const SimShared<V>&
   x.nkr = vmul(n[k], rr);
   const V Ur = vmul(q.U[k], rr);
   const V UE = vdiff(q.U[j], n[i], q.U[i], n[j]);
-  const V a = simk(K, tag, kcA), b = simk(K, tag, kcB), cc = simk(K, tag, kcCC), tbc = simk(K, tag, kcTBC);
+  const SimK4<V> k0 = simk4(K, tag, 0);
+  const V a = k0.x, b = k0.y, cc = k0.z, tbc = k0.w;
   x.wn0 = vfma(b, vfma(cc, rho2, q.Uu), a);
   x.wn1 = vmul(tbc, UE);
   x.wt0 = vfma(b, vfma(cc, vmul(n[k], n[k]), vfma(Ur, Ur, q.sg2)), a);
@@ -1257,6 +1262,7 @@ template <class V>
 __device__ __forceinline__ void point_sims_adjoint_free(const PointStateT<V>& ps, const SimConsts& K, V& dphi,
                                                         V dn[3]) {
   const V tag{};
+  const SimK4<V> k1 = simk4(K, tag, 1);
   SimShared<V> q;
   sim_shared(ps, q);
   V S = vsplat<V>(0.0f);
@@ -1267,11 +1273,11 @@ __device__ __forceinline__ void point_sims_adjoint_free(const PointStateT<V>& ps
     const V rn = vmap(vmul(vsub(x.wn0, x.wn1), vadd(x.wn0, x.wn1)), rcp_fast);
     const V rt = vmap(vmul(vsub(x.wt0, x.wt1), vadd(x.wt0, x.wt1)), rcp_fast);
     const V an = vmul(ps.n[k], rn);
-    const V at = vmul(vmul(simk(K, tag, kcMu), x.rho), rt);
+    const V at = vmul(vmul(k1.x, x.rho), rt);
     S = vfma(an, x.wn1, vfma(at, x.wt0, S));
-    dn[k] = vmul(simk(K, tag, kcFreeN), vfma(an, x.wn0, vmul(at, x.wt1)));
+    dn[k] = vmul(k1.z, vfma(an, x.wn0, vmul(at, x.wt1)));
   }
-  dphi = vfma(simk(K, tag, kcFree), S, simk(K, tag, kcFreePen));
+  dphi = vfma(k1.y, S, k1.w);
 }
 
 template <class V>
@@ -1282,6 +1288,7 @@ __device__ __forceinline__ void point_sims_adjoint(const PointStateT<V>& ps, con
   const V tag{};
   const V zero = vsplat<V>(0.0f);
   const V* n = ps.n;
+  const SimK4<V> k0 = simk4(K, tag, 0), k1 = simk4(K, tag, 1), k2 = simk4(K, tag, 2), k3 = simk4(K, tag, 3);
   SimShared<V> sh;
   sim_shared(ps, sh);
   unsigned cmask[W];
@@ -1294,9 +1301,9 @@ __device__ __forceinline__ void point_sims_adjoint(const PointStateT<V>& ps, con
     V gl[3], ga[3];
     get_sim_adjoint(G, 0, gl, ga);
     const V gfn = dot6(gl, n, ga, sh.U);
-    const V rw = vmap(vfma(simk(K, tag, kcB), sh.Uu, simk(K, tag, kcA)), rcp_fast);
-    const V q = vfma(gfn, rw, simk(K, tag, kcMWpen));
-    dphi = vfma(simk(K, tag, kcAlpha), vsel(kap, zero, q), dphi);
+    const V rw = vmap(vfma(k0.y, sh.Uu, k0.x), rcp_fast);
+    const V q = vfma(gfn, rw, k2.w);
+    dphi = vfma(k2.y, vsel(kap, zero, q), dphi);
   }
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -1309,7 +1316,7 @@ __device__ __forceinline__ void point_sims_adjoint(const PointStateT<V>& ps, con
       const int m = 1 + 2 * k + h;
       V gl[3], ga[3];
       get_sim_adjoint(G, m, gl, ga);
-      const V msc = simk(K, tag, h == 0 ? kcMC : kcC);               // -s c
+      const V msc = h == 0 ? k3.x : k2.x;               // -s c
       const V hi = vfma(ga[j], ps.p[k], vfnma(ga[k], ps.p[j], gl[i]));
       const V hj = vfma(ga[k], ps.p[i], vfnma(ga[i], ps.p[k], gl[j]));
       const V hk = vfma(ga[i], ps.p[j], vfnma(ga[j], ps.p[i], gl[k]));
@@ -1322,10 +1329,10 @@ __device__ __forceinline__ void point_sims_adjoint(const PointStateT<V>& ps, con
       // dph = -alpha dC,  dC = -(gf.n)/w_n - mu s (gf.tau)/w_t,  w = w0 - s w1
       const V rwn = vmap(h == 0 ? vsub(x.wn0, x.wn1) : vadd(x.wn0, x.wn1), rcp_fast);
       const V rwt = vmap(h == 0 ? vsub(x.wt0, x.wt1) : vadd(x.wt0, x.wt1), rcp_fast);
-      const V q = vfma(simk(K, tag, h == 0 ? kcMu : kcMMu), vmul(gdt, rwt), vmul(gdn, rwn));
+      const V q = vfma(h == 0 ? k1.x : k3.y, vmul(gdt, rwt), vmul(gdn, rwn));
       const V qa = vsel(kap, zero, q);
-      dphi = vfma(simk(K, tag, kcAlpha), qa, dphi);
-      dn[k] = vfma(simk(K, tag, h == 0 ? kcMAlphaC : kcAlphaC), qa, dn[k]);
+      dphi = vfma(k2.y, qa, dphi);
+      dn[k] = vfma(h == 0 ? k3.z : k2.z, qa, dn[k]);
     }
   }
   // simulations in which some lane of the warp is in contact: general adjoint,
