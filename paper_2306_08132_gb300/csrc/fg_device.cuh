@@ -232,12 +232,16 @@ struct SdfIndex {
   const float* cell;   // corner (i0, j0, k0)
 };
 
-// Index along one axis: the clamped cell, the fraction in it and the excess u - u_c.
+// Index along one axis: the cell, the fraction in it and the excess u - u_c.  Where u is
+// clamped, i is the boundary node itself (0 or n - 1) and f = 0: the value there does
+// not depend on the cell's other plane.
 struct AxisIndex {
   float f, du;
   int i;
   bool clamped;
 };
+// kNode = false: the last cell (f = 1) instead, for reads of whole cells.
+template <bool kNode = true>
 __device__ __forceinline__ AxisIndex sdf_axis(const ObjDev& O, int k, float x) {
   const float4 ax = O.axis, nm = O.n_max;
   const int4 cp = O.cap;
@@ -247,7 +251,8 @@ __device__ __forceinline__ AxisIndex sdf_axis(const ObjDev& O, int k, float x) {
   a.clamped = uc != u;
   a.du = sub_(u, uc);                                   // 0 unless clamped
   const int ii = __float2int_rd(uc);                    // floor (uc >= 0)
-  a.i = min(ii, k == 0 ? cp.x : k == 1 ? cp.y : cp.z);
+  const int cap = k == 0 ? cp.x : k == 1 ? cp.y : cp.z;
+  a.i = ii > cap && !(kNode && a.clamped) ? cap : ii;
   a.f = sub_(uc, (float)a.i);
   return a;
 }
@@ -260,7 +265,7 @@ __device__ __forceinline__ void sdf_index(const ObjDev& O, const float p[3], Sdf
   int i0[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const AxisIndex a = sdf_axis(O, k, p[k]);
+    const AxisIndex a = sdf_axis<true>(O, k, p[k]);
     ix.clamped[k] = a.clamped;
     ix.du[k] = a.du;
     ix.f[k] = a.f;
@@ -269,16 +274,28 @@ __device__ __forceinline__ void sdf_index(const ObjDev& O, const float p[3], Sdf
   ix.cell = sdf_cell(O, i0[0], i0[1], i0[2]);
 }
 
-__device__ __forceinline__ void sdf_gather(const ObjDev& O, const float* G, float c[8]) {
+// The corners of the planes that count (hi[k]: the upper plane of axis k does).  On a
+// clamped axis the upper plane has weight f = 0 in the value, its differences reach
+// only derivatives along that axis, which are zero there, and it may lie outside the
+// grid: its corners are not read and stand as 0.  Most hand points are outside the
+// grid, and the lanes of a warp mostly past the same face, so this removes whole loads.
+// Sweep of 256 objects 10.15 -> 9.79 ms, standalone lookups 0.273 -> 0.244 ms with points and wrenches.
+__device__ __forceinline__ void sdf_gather(const ObjDev& O, const float* G, const bool hi[3], float c[8]) {
   const int sy = O.sy, sz = O.sz;
+#pragma unroll
+  for (int e = 1; e < 8; ++e) c[e] = 0.0f;
   c[0] = __ldg(G);
-  c[1] = __ldg(G + 1);
-  c[2] = __ldg(G + sy);
-  c[3] = __ldg(G + sy + 1);
-  c[4] = __ldg(G + sz);
-  c[5] = __ldg(G + sz + 1);
-  c[6] = __ldg(G + sz + sy);
-  c[7] = __ldg(G + sz + sy + 1);
+  if (hi[0]) c[1] = __ldg(G + 1);
+  if (hi[1]) c[2] = __ldg(G + sy);
+  if (hi[0] && hi[1]) c[3] = __ldg(G + sy + 1);
+  if (hi[2]) c[4] = __ldg(G + sz);
+  if (hi[0] && hi[2]) c[5] = __ldg(G + sz + 1);
+  if (hi[1] && hi[2]) c[6] = __ldg(G + sz + sy);
+  if (hi[0] && hi[1] && hi[2]) c[7] = __ldg(G + sz + sy + 1);
+}
+__device__ __forceinline__ void sdf_gather(const ObjDev& O, const SdfIndex& ix, float c[8]) {
+  const bool hi[3] = {!ix.clamped[0], !ix.clamped[1], !ix.clamped[2]};
+  sdf_gather(O, ix.cell, hi, c);
 }
 
 __device__ __forceinline__ float rsqrt_or_zero(float x) { return x > 0.0f ? rsqrtf(x) : 0.0f; }
@@ -366,13 +383,14 @@ __device__ __forceinline__ void sdf_finish_pair(const ObjDev& O, const SdfIndex&
 
 // Lower bound of the interpolated SDF at p from one entry of the min-pyramid: the
 // block of 2^lev cells (level 2 when the grid has it) holding p's cell, the cell
-// sdf_index picks.  The interpolant in a cell is a convex combination of its
+// sdf_index picks (the last cell at the upper boundary).  The interpolant in a cell is a convex combination of its
 // corners and the excess distance outside the grid is non-negative, so
 // phi(p) >= the block's minimum.
 __device__ __forceinline__ float point_min_bound(const ObjDev& O, const float p[3]) {
   const int lev = O.pyr_levels >= 2 ? 2 : 1;
   const int4 cp = O.cap;
-  const int b[3] = {sdf_axis(O, 0, p[0]).i >> lev, sdf_axis(O, 1, p[1]).i >> lev, sdf_axis(O, 2, p[2]).i >> lev};
+  const int b[3] = {sdf_axis<false>(O, 0, p[0]).i >> lev, sdf_axis<false>(O, 1, p[1]).i >> lev,
+                    sdf_axis<false>(O, 2, p[2]).i >> lev};
   const int bx = (cp.x >> lev) + 1, by = (cp.y >> lev) + 1;      // ceil((n - 1) / 2^lev)
   return __ldg(O.pyr + O.pyr_off[lev - 1] + (unsigned)((b[2] * by + b[1]) * bx + b[0]));
 }
@@ -914,7 +932,7 @@ __device__ __forceinline__ void sdf_lookup(const ObjDev& O, const float p[3], Sd
   SdfIndex ix;
   sdf_index(O, p, ix);
   float c[8];
-  sdf_gather(O, ix.cell, c);
+  sdf_gather(O, ix, c);
   sdf_finish<kHess>(O, ix, c, s);
 }
 

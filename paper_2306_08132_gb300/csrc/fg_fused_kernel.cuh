@@ -203,8 +203,8 @@ __device__ __forceinline__ void point_adjoint_pair(const HandDev& H, const float
     sdf_index(O, pa, xa);
     sdf_index(O, pb, xb);
     float ca[8], cb[8];
-    sdf_gather(O, xa.cell, ca);
-    sdf_gather(O, xb.cell, cb);
+    sdf_gather(O, xa, ca);
+    sdf_gather(O, xb, cb);
     sdf_finish_pair(O, xa, xb, ca, cb, smp);
   }
   const float2 p[3] = {make_float2(pa[0], pb[0]), make_float2(pa[1], pb[1]), make_float2(pa[2], pb[2])};

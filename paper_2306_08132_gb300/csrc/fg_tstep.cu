@@ -380,14 +380,15 @@ __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const Param
   if constexpr (NEAR) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const AxisIndex a = sdf_axis(O, k, p[k]);
+      const AxisIndex a = sdf_axis<false>(O, k, p[k]);
       ix.f[k] = a.f;
       ix.du[k] = a.du;
       ix.clamped[k] = a.clamped;
       cell[k] = a.i;
     }
     ix.cell = sdf_cell(O, cell[0], cell[1], cell[2]);
-    sdf_gather(O, ix.cell, c0);
+    const bool all[3] = {true, true, true};        // whole cells: a plane that is skipped costs more tests here than it saves
+    sdf_gather(O, ix.cell, all, c0);
   }
 #pragma unroll
   for (int m = 0; m < kSims; ++m) {
@@ -403,7 +404,7 @@ __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const Param
         // the query moves against the velocity: down for m odd, up for m even
         const int k = sim_axis(m);
         const bool down = m & 1;
-        const AxisIndex a = sdf_axis(O, k, r[k]);
+        const AxisIndex a = sdf_axis<false>(O, k, r[k]);
         q.f[k] = a.f;
         q.du[k] = a.du;
         q.clamped[k] = a.clamped;
@@ -841,7 +842,7 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
               touch = sub_(msmp.phi, rdil) < 0.0f;
             } else {
               sdf_index(O, r, ix);
-              sdf_gather(O, ix.cell, corner);
+              sdf_gather(O, ix, corner);
               touch = query_in_contact(O, ix, corner, rdil);
             }
             float pb[3];
