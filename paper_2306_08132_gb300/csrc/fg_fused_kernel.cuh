@@ -46,6 +46,7 @@ struct FusedSmem {
   unsigned long long wfix[kSims][8];  // forward sums in fixed point: W (6), N (integer), pen
   float lacc[NW][kMaxLinks][6];    // per warp, per link: sum g, sum (p - t) x g (fixed ranges)
   float uacc[kMaxUnits][6];        // per work unit: sum g, sum (p - t) x g
+  float lsum[kMaxLinks][6];        // per link: sum g, sum (p - t) x g
   float Wtot[kSims][8];
   float loss;
   int cand;                        // the candidate claimed by this CTA
@@ -133,17 +134,15 @@ __device__ __forceinline__ float sphere_bound(const ObjDev& O, const float4* f4,
   return mn - (1e-6f + 1e-5f * fabsf(mn));
 }
 
-// Adjoint of one hand point (index i, link frames in smem): dL/dp through the 7
+// Adjoint of one hand point (index i, record sp of link `link`, link frames in smem): dL/dp through the 7
 // simulations, the normal and the SDF lookup.  v = (g, (p - t0) x g).  FREE: a
 // candidate without contacts (point_sims_adjoint_free).  faces: the points' closest
 // faces (mesh objects), or nullptr to search for them.
 template <bool ANY, bool FREE>
-__device__ __forceinline__ void point_adjoint(const HandDev& H, const float4 (*frame4)[3], const SimAdjoints& G,
+__device__ __forceinline__ void point_adjoint(const float4 (*frame4)[3], const SimAdjoints& G,
                                               const SimConsts& K, const ObjDev& O,
                                               const ParamsDev& Pm, float r, const float t0[3], const int* faces,
-                                              int i, bool valid, float v[6], int& link) {
-  const float4 sp = __ldg(H.pts + i);
-  link = (int)sp.w;
+                                              int i, const float4& sp, int link, bool valid, float v[6]) {
   float p[3];
   world_point(frame4[link], sp, p);
   SdfSample smp;
@@ -343,9 +342,10 @@ __device__ __forceinline__ void adjoint_sweep(FusedSmem<NW>& S, const ObjDev& O,
       return __shfl_sync(kFull, j, 0);
     };
     int u = claim();
+    int4 U = __ldg(H.units + min(u, H.nunits - 1));      // first point, count, link
     while (u < H.nunits) {
       const int nu = claim();
-      const int4 U = __ldg(H.units + u);      // first point, count, link
+      const int4 nU = __ldg(H.units + min(nu, H.nunits - 1));
       float sum[6];
       if (PPT == 2) {
         // one point of each half of the unit per lane, packed arithmetic
@@ -359,17 +359,24 @@ __device__ __forceinline__ void adjoint_sweep(FusedSmem<NW>& S, const ObjDev& O,
       } else {
 #pragma unroll
         for (int k = 0; k < 6; ++k) sum[k] = 0.0f;
+        // the next half's record is read before this half is computed
+        int i = lane < U.y ? U.x + lane : U.x;
+        float4 sp = __ldg(H.pts + i);
+#pragma unroll 1
         for (int h = 0; h < U.y; h += 32) {
+          const int ni = h + 32 + lane < U.y ? U.x + h + 32 + lane : U.x;
+          const float4 nsp = __ldg(H.pts + ni);
           float v[6];
-          int link;
-          const bool valid = h + lane < U.y;
-          point_adjoint<ANY, FREE>(H, S.frame4, S.G, S.K, O, Pm, r, t0, faces, valid ? U.x + h + lane : U.x, valid, v, link);
+          point_adjoint<ANY, FREE>(S.frame4, S.G, S.K, O, Pm, r, t0, faces, i, sp, U.z, h + lane < U.y, v);
 #pragma unroll
           for (int k = 0; k < 6; ++k) sum[k] += v[k];
+          i = ni;
+          sp = nsp;
         }
       }
       unit_reduce_store(sum, lane, S.uacc[u]);
       u = nu;
+      U = nU;
     }
   } else {
     // fixed, contiguous 32-aligned point ranges per warp
@@ -379,10 +386,11 @@ __device__ __forceinline__ void adjoint_sweep(FusedSmem<NW>& S, const ObjDev& O,
     const int pb = warp * span, pe = min(P, pb + span);
     for (int base = pb; base < pe; base += 32) {
       float v[6];
-      int link;
       const int i = base + lane;
       const bool valid = i < pe;
-      point_adjoint<ANY, FREE>(H, S.frame4, S.G, S.K, O, Pm, r, t0, faces, valid ? i : base, valid, v, link);
+      const float4 sp = __ldg(H.pts + (valid ? i : base));
+      const int link = (int)sp.w;
+      point_adjoint<ANY, FREE>(S.frame4, S.G, S.K, O, Pm, r, t0, faces, valid ? i : base, sp, link, valid, v);
       link_accumulate(S.lacc[warp], lane, link, valid, v, cur, acc);
     }
     if (cur >= 0) {
@@ -654,7 +662,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
           if (lane == 0) S.loss = Ls + Pm.w_range * rn + Pm.w_limit * lims + Pm.w_pen * S.Wtot[0][7];
         }
       }
-      for (int idx = tid; idx < NW * kMaxLinks * 6; idx += NW * 32) (&S.lacc[0][0][0])[idx] = 0.0f;
+      if (H.nunits > kMaxUnits)
+        for (int idx = tid; idx < NW * kMaxLinks * 6; idx += NW * 32) (&S.lacc[0][0][0])[idx] = 0.0f;
       if (tid == 0) S.next_unit = 0;
       __syncthreads();
       if (MODE == kModeLossGrad && a.grad == nullptr) {    // loss only: no adjoint
@@ -679,20 +688,25 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
       __syncthreads();
 
       // ------------------------------------------------------------------ tree
+      // per-link sums, one thread per link and component
+      for (int idx = tid; idx < L * 6; idx += NW * 32) {
+        const int l = idx / 6, k = idx - 6 * l;
+        float x = 0.0f;
+        if (H.nunits <= kMaxUnits) {
+          for (int u = H.unit_begin[l]; u < H.unit_begin[l + 1]; ++u) x += S.uacc[u][k];
+        } else {
+#pragma unroll
+          for (int w = 0; w < NW; ++w) x += S.lacc[w][l][k];
+        }
+        S.lsum[l][k] = x;
+      }
+      __syncthreads();
       if (warp == 0) {
-        // per-link sums over warps, inclusive prefix over preorder links
+        // inclusive prefix over preorder links
         float pre[6];
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-          float x = 0.0f;
-          if (lane < L) {
-            if (H.nunits <= kMaxUnits) {
-              for (int u = H.unit_begin[lane]; u < H.unit_begin[lane + 1]; ++u) x += S.uacc[u][k];
-            } else {
-#pragma unroll
-              for (int w = 0; w < NW; ++w) x += S.lacc[w][lane][k];
-            }
-          }
+          float x = lane < L ? S.lsum[lane][k] : 0.0f;
 #pragma unroll
           for (int o = 1; o < 32; o <<= 1) {
             const float y = __shfl_up_sync(kFull, x, o);
