@@ -210,14 +210,15 @@ __device__ __forceinline__ void transform_point(const float* R, const float* o, 
 // Result of one grid lookup (V = float: one point; float2: two points).  g is
 // the gradient of the undilated SDF; hxy, hxz, hyz the mixed second derivatives
 // of the trilinear part (zero on clamped axes); when the point lies outside the
-// grid, eh = (u - u_c)/|u - u_c| and e the excess distance.
+// grid, eh = (u - u_c)/|u - u_c| and re the reciprocal of the excess distance (the curvature
+// of the distance to the grid's box); both are 0 inside.
 template <class V>
 struct SdfSampleT {
   V phi;
   V g[3];
   V hxy, hxz, hyz;
   V eh[3];
-  V e;
+  V re;
   V curv;          // mesh objects: s / |p - r*_rho| (curvature of the Phong SDF about r*_rho); 0 for grids
   mask_t<V> outside;
 };
@@ -298,8 +299,15 @@ __device__ __forceinline__ void sdf_gather(const ObjDev& O, const SdfIndex& ix, 
   sdf_gather(O, ix.cell, hi, c);
 }
 
-__device__ __forceinline__ float rsqrt_or_zero(float x) { return x > 0.0f ? rsqrtf(x) : 0.0f; }
-__device__ __forceinline__ float rcp_or_zero(float x) { return x > 0.0f ? __fdividef(1.0f, x) : 0.0f; }
+// 1/sqrt(x) of a normal float: the hardware approximation, one instruction (rsqrtf adds the
+// scaling of subnormal arguments, three more).
+__device__ __forceinline__ float rsqrt_fast(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// 0 where x is not a positive normal float (zero, subnormal, NaN).
+__device__ __forceinline__ float rsqrt_or_zero(float x) { return x >= 1.17549435e-38f ? rsqrt_fast(x) : 0.0f; }
 // Reciprocal of a positive, normal float (the effective inverse masses w_n, w_t
 // >= 1/m of the simulation adjoint): the hardware approximation, one instruction.
 __device__ __forceinline__ float rcp_fast(float x) {
@@ -329,12 +337,12 @@ __device__ __forceinline__ void sdf_finish_v(const ObjDev& O, const V f[3], cons
   const V ddy = vsub(dy1, dy0);
   const V gy = vfma(f[2], ddy, dy0);            // d/dfy
   const V gz = dz;                              // d/dfz
-  const V zero = vsplat<V>(0.0f), ih = vsplat<V>(O.inv_h);
+  const V zero = vsplat<V>(0.0f), ih = vsplat<V>(O.axis.x);
   s.g[0] = vsel(cl[0], zero, vmul(gx, ih));
   s.g[1] = vsel(cl[1], zero, vmul(gy, ih));
   s.g[2] = vsel(cl[2], zero, vmul(gz, ih));
   if (kHess) {
-    const V ih2 = vsplat<V>(mul_(O.inv_h, O.inv_h));
+    const V ih2 = vsplat<V>(mul_(O.axis.x, O.axis.x));
     const V hxy = vfma(f[2], vsub(ey1, ey0), ey0);
     s.hxy = vsel(mor(cl[0], cl[1]), zero, vmul(hxy, ih2));
     s.hxz = vsel(mor(cl[0], cl[2]), zero, vmul(dax, ih2));
@@ -342,21 +350,21 @@ __device__ __forceinline__ void sdf_finish_v(const ObjDev& O, const V f[3], cons
   }
   s.outside = mor(mor(cl[0], cl[1]), cl[2]);
   s.curv = zero;
-  s.e = zero;
+  s.re = zero;
   s.eh[0] = s.eh[1] = s.eh[2] = zero;
+  s.phi = val;
   if (many(s.outside)) {
-    // du is exactly 0 on unclamped axes, so points inside the grid get eh = 0, e = 0
+    // du is exactly 0 on unclamped axes, so points inside the grid get eh = 0, re = 0
     const V dn2 = vfma(du[0], du[0], vfma(du[1], du[1], vmul(du[2], du[2])));
     const V r = vmap(dn2, rsqrt_or_zero);
-    const V dn = vmul(dn2, r);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       s.eh[k] = vmul(du[k], r);
-      s.g[k] = vsel(s.outside, vadd(s.g[k], s.eh[k]), s.g[k]);
+      s.g[k] = vadd(s.g[k], s.eh[k]);
     }
-    s.e = vmul(vsplat<V>(O.h), dn);
+    s.re = vmul(r, ih);
+    s.phi = vadd(val, vmul(vsplat<V>(O.n_max.w), vmul(dn2, r)));
   }
-  s.phi = vadd(val, s.e);
 }
 
 template <bool kHess>
@@ -862,7 +870,7 @@ static __device__ __noinline__ int mesh_find(const ObjDev& O, const float p[3]) 
 static __device__ __noinline__ void mesh_eval(const ObjDev& O, const float p[3], int f, SdfSample& s) {
   if (f < 0) {                                  // p not finite: no face compares closer
     const float nan = __int_as_float(0x7fc00000);
-    s.phi = s.curv = s.e = nan;
+    s.phi = s.curv = s.re = nan;
     s.g[0] = s.g[1] = s.g[2] = nan;
     s.eh[0] = s.eh[1] = s.eh[2] = 0.0f;
     s.hxy = s.hxz = s.hyz = 0.0f;
@@ -909,7 +917,7 @@ static __device__ __noinline__ void mesh_eval(const ObjDev& O, const float p[3],
     s.eh[k] = 0.0f;
   }
   s.hxy = s.hxz = s.hyz = 0.0f;
-  s.e = 0.0f;
+  s.re = 0.0f;
   s.curv = sgn * inv;
   s.outside = false;
 }
@@ -1141,7 +1149,7 @@ __device__ __forceinline__ void sim_adjoint(const PointState& ps, int m, float p
 
 // Constants of the simulation adjoint for one candidate step, in shared memory.
 // Scalar table (float index), in groups of four read by one 16-byte load each:
-//   0  1/m, 1/I, c^2, 2c/I  (c = dt V)
+//   0  1/m, 1/I, c^2/I, 2c/I  (c = dt V)
 //   1  mu; for a candidate without contacts (sim_constants_free): 2 g alpha, -2 g alpha c, -alpha w_pen
 //   2  c, alpha, alpha c, -w_pen
 //   3  -c, -mu, -alpha c
@@ -1156,7 +1164,7 @@ struct SimK4 {
 };
 __device__ __forceinline__ void sim_constants(const ParamsDev& P, const ObjDev& O, SimConsts& K) {
   const float c = P.dt * P.V;
-  const float v[16] = {O.inv_mass, O.inv_inertia, c * c, 2.0f * c * O.inv_inertia, P.mu, 0.0f, 0.0f, 0.0f,
+  const float v[16] = {O.inv_mass, O.inv_inertia, c * c * O.inv_inertia, 2.0f * c * O.inv_inertia, P.mu, 0.0f, 0.0f, 0.0f,
                        c, P.alpha, P.alpha * c, -P.w_pen, -c, -P.mu, -P.alpha * c, 0.0f};
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
@@ -1232,40 +1240,41 @@ __device__ __forceinline__ V dot6(const V gl[3], const V a[3], const V ga[3], co
 // 14 multiply-adds a simulation instead of the 20 of two 6-term dot products, and
 // no vector products of tau: 0.26 of the adjoint's instructions on the
 // 8-superquadric batch.
+// The inverse masses as base + c^2/I (...) need the squares n_k^2 and two bases once a point.
 template <class V>
 struct SimShared {
-  V U[3], Uu, sg, sg2;
+  V U[3], Uu, sg, nn[3], wn, wt, tsg;      // wn = 1/m + |U|^2/I, wt = 1/m + sg^2/I, tsg = 2c/I sg
 };
 template <class V>
-__device__ __forceinline__ void sim_shared(const PointStateT<V>& ps, SimShared<V>& q) {
+__device__ __forceinline__ void sim_shared(const PointStateT<V>& ps, const SimK4<V>& k0, SimShared<V>& q) {
   vcross(ps.p, ps.n, q.U);
   q.Uu = vdot(q.U, q.U);
   q.sg = vdot(ps.p, ps.n);
-  q.sg2 = vmul(q.sg, q.sg);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) q.nn[k] = vmul(ps.n[k], ps.n[k]);
+  q.wn = vfma(k0.y, q.Uu, k0.x);
+  q.wt = vfma(k0.y, vmul(q.sg, q.sg), k0.x);
+  q.tsg = vmul(k0.w, q.sg);
 }
-// Per axis k: rho, n_k/rho (0 when n is parallel to e_k) and the inverse masses
-// w = w0 - s w1 of the normal and tangential corrections.
+// Per axis k: rho^2, 1/rho (rho bounded away from 0: n parallel to e_k gives rho = 0,
+// U_k = 0, n_k/rho times zero) and the inverse masses w = w0 - s w1 of the normal and tangential
+// corrections.
 template <class V>
 struct SimAxis {
-  V rho, nkr, wn0, wn1, wt0, wt1;
+  V rho2, rr, wn0, wn1, wt0, wt1;
 };
+__device__ __forceinline__ float rsqrt_bounded(float x) { return rsqrt_fast(fmaxf(x, 1e-30f)); }
 template <class V>
-__device__ __forceinline__ void sim_axis_terms(const V n[3], const SimShared<V>& q, const SimConsts& K, int k,
+__device__ __forceinline__ void sim_axis_terms(const V n[3], const SimShared<V>& q, const SimK4<V>& k0, int k,
                                                SimAxis<V>& x) {
-  const V tag{};
   const int i = (k + 1) % 3, j = (k + 2) % 3;
-  const V rho2 = vfma(n[i], n[i], vmul(n[j], n[j]));
-  const V rr = vmap(rho2, rsqrt_or_zero);
-  x.rho = vmul(rho2, rr);
-  x.nkr = vmul(n[k], rr);
-  const V Ur = vmul(q.U[k], rr);
-  const V UE = vdiff(q.U[j], n[i], q.U[i], n[j]);
-  const SimK4<V> k0 = simk4(K, tag, 0);
-  const V a = k0.x, b = k0.y, cc = k0.z, tbc = k0.w;
-  x.wn0 = vfma(b, vfma(cc, rho2, q.Uu), a);
-  x.wn1 = vmul(tbc, UE);
-  x.wt0 = vfma(b, vfma(cc, vmul(n[k], n[k]), vfma(Ur, Ur, q.sg2)), a);
-  x.wt1 = vmul(tbc, vmul(q.sg, n[k]));
+  x.rho2 = vadd(q.nn[i], q.nn[j]);
+  x.rr = vmap(x.rho2, rsqrt_bounded);
+  const V Ur = vmul(q.U[k], x.rr);
+  x.wn0 = vfma(k0.z, x.rho2, q.wn);
+  x.wn1 = vmul(k0.w, vdiff(q.U[j], n[i], q.U[i], n[j]));
+  x.wt0 = vfma(vmul(k0.y, Ur), Ur, vfma(k0.z, q.nn[k], q.wt));
+  x.wt1 = vmul(q.tsg, n[k]);
 }
 
 // The adjoint of a candidate without any contact (no simulation moved the object):
@@ -1275,27 +1284,29 @@ __device__ __forceinline__ void sim_axis_terms(const V n[3], const SimShared<V>&
 //   q+ - q- = 2 g (n_k w_n0 / (w_n0^2 - w_n1^2) + mu rho w_t1 / (w_t0^2 - w_t1^2)),
 // dphi = alpha sum (q+ + q-) - alpha w_pen, dn_k = -alpha c (q+ - q-): 2 reciprocals an
 // axis and no wrench adjoint to read.  Three quarters of the benchmark's
-// candidates touch nothing.
+// candidates touch nothing.  The factor of dn is left to 1/|grad|, which multiplies
+// it next (ps.rg becomes that product).
 template <class V>
-__device__ __forceinline__ void point_sims_adjoint_free(const PointStateT<V>& ps, const SimConsts& K, V& dphi,
-                                                        V dn[3]) {
+__device__ __forceinline__ void point_sims_adjoint_free(PointStateT<V>& ps, const SimConsts& K, V& dphi, V dn[3]) {
   const V tag{};
-  const SimK4<V> k1 = simk4(K, tag, 1);
+  const SimK4<V> k0 = simk4(K, tag, 0), k1 = simk4(K, tag, 1);
   SimShared<V> q;
-  sim_shared(ps, q);
+  sim_shared(ps, k0, q);
   V S = vsplat<V>(0.0f);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     SimAxis<V> x;
-    sim_axis_terms(ps.n, q, K, k, x);
+    sim_axis_terms(ps.n, q, k0, k, x);
     const V rn = vmap(vmul(vsub(x.wn0, x.wn1), vadd(x.wn0, x.wn1)), rcp_fast);
     const V rt = vmap(vmul(vsub(x.wt0, x.wt1), vadd(x.wt0, x.wt1)), rcp_fast);
     const V an = vmul(ps.n[k], rn);
-    const V at = vmul(vmul(k1.x, x.rho), rt);
-    S = vfma(an, x.wn1, vfma(at, x.wt0, S));
-    dn[k] = vmul(k1.z, vfma(an, x.wn0, vmul(at, x.wt1)));
+    const V at = vmul(vmul(vmul(k1.x, x.rho2), x.rr), rt);
+    const V St = k == 0 ? vmul(at, x.wt0) : vfma(at, x.wt0, S);
+    S = vfma(an, x.wn1, St);
+    dn[k] = vfma(an, x.wn0, vmul(at, x.wt1));
   }
   dphi = vfma(k1.y, S, k1.w);
+  ps.rg = vmul(ps.rg, k1.z);
 }
 
 template <class V>
@@ -1308,7 +1319,7 @@ __device__ __forceinline__ void point_sims_adjoint(const PointStateT<V>& ps, con
   const V* n = ps.n;
   const SimK4<V> k0 = simk4(K, tag, 0), k1 = simk4(K, tag, 1), k2 = simk4(K, tag, 2), k3 = simk4(K, tag, 3);
   SimShared<V> sh;
-  sim_shared(ps, sh);
+  sim_shared(ps, k0, sh);
   unsigned cmask[W];
 #pragma unroll
   for (int l = 0; l < W; ++l) cmask[l] = 0u;
@@ -1319,7 +1330,7 @@ __device__ __forceinline__ void point_sims_adjoint(const PointStateT<V>& ps, con
     V gl[3], ga[3];
     get_sim_adjoint(G, 0, gl, ga);
     const V gfn = dot6(gl, n, ga, sh.U);
-    const V rw = vmap(vfma(k0.y, sh.Uu, k0.x), rcp_fast);
+    const V rw = vmap(sh.wn, rcp_fast);
     const V q = vfma(gfn, rw, k2.w);
     dphi = vfma(k2.y, vsel(kap, zero, q), dphi);
   }
@@ -1328,7 +1339,8 @@ __device__ __forceinline__ void point_sims_adjoint(const PointStateT<V>& ps, con
     const int i = (k + 1) % 3, j = (k + 2) % 3;
     const V ni = n[i], nj = n[j], nk = n[k];
     SimAxis<V> x;
-    sim_axis_terms(n, sh, K, k, x);
+    sim_axis_terms(n, sh, k0, k, x);
+    const V rho = vmul(x.rho2, x.rr), nkr = vmul(nk, x.rr);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int m = 1 + 2 * k + h;
@@ -1340,7 +1352,7 @@ __device__ __forceinline__ void point_sims_adjoint(const PointStateT<V>& ps, con
       const V hk = vfma(ga[i], ps.p[j], vfnma(ga[j], ps.p[i], gl[k]));
       const V A = vfma(msc, vdiff(ga[j], ni, ga[i], nj), vfma(ni, hi, vmul(nj, hj)));
       const V gdn = vfma(nk, hk, A);
-      const V gdt = vdiff(x.rho, hk, x.nkr, A);
+      const V gdt = vdiff(rho, hk, nkr, A);
       const mask_t<V> kap = vlt(sim_phi(ps, m, P.dt * P.V), zero);
 #pragma unroll
       for (int l = 0; l < W; ++l) cmask[l] |= mlane(kap, l) ? (1u << m) : 0u;
@@ -1391,27 +1403,33 @@ __device__ __forceinline__ void point_sims_adjoint(const PointStateT<V>& ps, con
 // direct dL/dp, returns the total dL/dp.  n = g/|g|, g = grad phi(p), and the
 // Hessian of phi is the trilinear mixed part plus, outside the grid, the
 // curvature (I - eh eh^T)/e of the excess distance on the clamped axes.
-template <class V>
+// kMesh: the sample may be a mesh's (curv); kDirect: dp holds a direct part (otherwise
+// it is only written).
+template <bool kMesh = true, bool kDirect = true, class V>
 __device__ __forceinline__ void sdf_adjoint(const SdfSampleT<V>& s, const PointStateT<V>& ps, V d_phi_hat,
                                             const V dn[3], V dp[3]) {
   const V ndn = vdot(ps.n, dn);
   V dg[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) dg[k] = vmul(vfnma(ndn, ps.n[k], dn[k]), ps.rg);
-  dp[0] = vadd(dp[0], vfma(d_phi_hat, s.g[0], vfma(s.hxy, dg[1], vfma(s.hxz, dg[2], vmul(s.curv, dg[0])))));
-  dp[1] = vadd(dp[1], vfma(d_phi_hat, s.g[1], vfma(s.hxy, dg[0], vfma(s.hyz, dg[2], vmul(s.curv, dg[1])))));
-  dp[2] = vadd(dp[2], vfma(d_phi_hat, s.g[2], vfma(s.hxz, dg[0], vfma(s.hyz, dg[1], vmul(s.curv, dg[2])))));
+  const V h[3][2] = {{s.hxy, s.hxz}, {s.hxy, s.hyz}, {s.hxz, s.hyz}};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const V d0 = dg[k == 0 ? 1 : 0], d1 = dg[k == 2 ? 1 : 2];
+    const V t = kMesh ? vfma(h[k][1], d1, vmul(s.curv, dg[k])) : vmul(h[k][1], d1);
+    const V x = vfma(d_phi_hat, s.g[k], vfma(h[k][0], d0, t));
+    dp[k] = kDirect ? vadd(dp[k], x) : x;
+  }
   if (many(s.outside)) {
-    // eh is zero on unclamped axes (and for points inside the grid, where e = 0
+    // eh is zero on unclamped axes (and for points inside the grid, where re = 0
     // and the term vanishes), so (I - eh eh^T) restricted to clamped axes is
     // D_c - eh eh^T with D_c the mask of axes where eh != 0.
-    const V zero = vsplat<V>(0.0f), one = vsplat<V>(1.0f);
-    const V re = vmap(s.e, rcp_or_zero);
+    const V zero = vsplat<V>(0.0f);
     const V ehdg = vdot(s.eh, dg);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const V ck = vsel(vne(s.eh[k], zero), one, zero);
-      dp[k] = vfma(vfnma(s.eh[k], ehdg, vmul(ck, dg[k])), re, dp[k]);
+      const V t = vsel(vne(s.eh[k], zero), vfnma(s.eh[k], ehdg, dg[k]), zero);
+      dp[k] = vfma(t, s.re, dp[k]);
     }
   }
 }

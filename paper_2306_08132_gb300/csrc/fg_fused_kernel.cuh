@@ -157,17 +157,12 @@ __device__ __forceinline__ void point_adjoint(const float4 (*frame4)[3], const S
     point_sims_adjoint_free(ps, K, dphi, dn);
   else
     point_sims_adjoint(ps, G, K, Pm, O, dphi, dn, dp);
-  sdf_adjoint(smp, ps, dphi, dn, dp);
-  if (valid) {
-    const float rel[3] = {p[0] - t0[0], p[1] - t0[1], p[2] - t0[2]};
-    float tq[3];
-    cross3(rel, dp, tq);
-    v[0] = dp[0]; v[1] = dp[1]; v[2] = dp[2];
-    v[3] = tq[0]; v[4] = tq[1]; v[5] = tq[2];
-  } else {
+  sdf_adjoint<ANY, !FREE>(smp, ps, dphi, dn, dp);
+  // a lane without a point holds a copy of another one (finite or not, as that one is): zero force, zero torque
+  const float rel[3] = {p[0] - t0[0], p[1] - t0[1], p[2] - t0[2]};
 #pragma unroll
-    for (int k = 0; k < 6; ++k) v[k] = 0.0f;
-  }
+  for (int k = 0; k < 3; ++k) v[k] = valid ? dp[k] : 0.0f;
+  cross3(rel, v, v + 3);
 }
 
 // The same for two points (a, b) at once, in packed f32x2 arithmetic: positions
@@ -189,7 +184,7 @@ __device__ __forceinline__ void point_adjoint_pair(const HandDev& H, const float
     mesh_eval(O, pa, faces != nullptr ? faces[ia] : mesh_find(O, pa), sa);
     mesh_eval(O, pb, faces != nullptr ? faces[ib] : mesh_find(O, pb), sb);
     smp.phi = make_float2(sa.phi, sb.phi);
-    smp.hxy = smp.hxz = smp.hyz = smp.e = make_float2(0.0f, 0.0f);
+    smp.hxy = smp.hxz = smp.hyz = smp.re = make_float2(0.0f, 0.0f);
     smp.curv = make_float2(sa.curv, sb.curv);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -215,7 +210,7 @@ __device__ __forceinline__ void point_adjoint_pair(const HandDev& H, const float
     point_sims_adjoint_free(ps, K, dphi, dn);
   else
     point_sims_adjoint(ps, G, K, Pm, O, dphi, dn, dp);
-  sdf_adjoint(smp, ps, dphi, dn, dp);
+  sdf_adjoint<ANY, !FREE>(smp, ps, dphi, dn, dp);
   const float2 rel[3] = {vsub(p[0], vsplat<float2>(t0[0])), vsub(p[1], vsplat<float2>(t0[1])),
                          vsub(p[2], vsplat<float2>(t0[2]))};
   float2 tq[3];

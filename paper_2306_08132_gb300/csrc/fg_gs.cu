@@ -785,7 +785,7 @@ __global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_ke
             for (int k = 0; k < 6; ++k) st0[k] = sn[k];
             gs_chunk_reverse(ps, xt, st0, av, mask, m, lane, Pm, O, smine, amine, dphi, dn, dp);
             if (!((mask >> lane) & 1u)) gs_leaky(ps, xt, smine, amine, m == 0 ? Pm.w_pen : 0.0f, Pm, O, dphi, dn, dp);
-            sdf_adjoint(smp, ps, dphi, dn, dp);
+            sdf_adjoint<ANY>(smp, ps, dphi, dn, dp);
             float v[6];
             if (valid) {
               const float rel[3] = {p[0] - t0[0], p[1] - t0[1], p[2] - t0[2]};
@@ -854,7 +854,7 @@ __global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_ke
               }
             }
           }
-          sdf_adjoint(smp, ps, dphi, dn, dp);
+          sdf_adjoint<ANY>(smp, ps, dphi, dn, dp);
           float v[6];
           if (valid) {
             const float rel[3] = {p[0] - t0[0], p[1] - t0[1], p[2] - t0[2]};

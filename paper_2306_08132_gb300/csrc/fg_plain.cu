@@ -20,7 +20,7 @@ namespace fg {
 
 namespace {
 
-constexpr int kSampleFloats = 11;   // phi, g[3], hxy, hxz, hyz, eh[3], e
+constexpr int kSampleFloats = 11;   // phi, g[3], hxy, hxz, hyz, eh[3], re
 constexpr size_t kAlign = 256;
 
 struct Workspace {
@@ -120,7 +120,7 @@ __global__ void sdf_stage_kernel(const HandDev* __restrict__ Hp, const ObjDev* _
     float p[3] = {pts[idx], pts[BP + idx], pts[2 * BP + idx]};
     SdfSample s;
     sdf_lookup<true, false>(O, p, s);   // the per-stage form takes grid objects only
-    float v[kSampleFloats] = {s.phi, s.g[0], s.g[1], s.g[2], s.hxy, s.hxz, s.hyz, s.eh[0], s.eh[1], s.eh[2], s.e};
+    float v[kSampleFloats] = {s.phi, s.g[0], s.g[1], s.g[2], s.hxy, s.hxz, s.hyz, s.eh[0], s.eh[1], s.eh[2], s.re};
 #pragma unroll
     for (int k = 0; k < kSampleFloats; ++k) smp[k * BP + idx] = v[k];
   }
@@ -137,8 +137,8 @@ __device__ __forceinline__ void load_sample(const float* smp, size_t BP, size_t 
   s.eh[0] = smp[7 * BP + idx];
   s.eh[1] = smp[8 * BP + idx];
   s.eh[2] = smp[9 * BP + idx];
-  s.e = smp[10 * BP + idx];
-  s.outside = s.e > 0.0f || s.eh[0] != 0.0f || s.eh[1] != 0.0f || s.eh[2] != 0.0f;
+  s.re = smp[10 * BP + idx];
+  s.outside = s.re > 0.0f || s.eh[0] != 0.0f || s.eh[1] != 0.0f || s.eh[2] != 0.0f;
 }
 
 // 4: contact forward, one CTA (256 threads) per candidate.
@@ -251,7 +251,7 @@ __global__ void contact_adj_kernel(const HandDev* __restrict__ Hp, const ObjDev*
       const float Ga[3] = {Gb[m * 6 + 3], Gb[m * 6 + 4], Gb[m * 6 + 5]};
       sim_adjoint(ps, m, phm, phm < 0.0f, Gl, Ga, Pm, O, m == 0 ? Pm.w_pen : 0.0f, dphi, dn, dp);
     }
-    sdf_adjoint(s, ps, dphi, dn, dp);
+    sdf_adjoint<false>(s, ps, dphi, dn, dp);
     dpo[idx] = dp[0];
     dpo[BP + idx] = dp[1];
     dpo[2 * BP + idx] = dp[2];

@@ -359,7 +359,7 @@ __device__ __forceinline__ void first_forward_chunk(const ObjDev& O, const Param
 // Reverse of one point in every simulation: pb = dL/dp.  A point out of contact
 // (C = 0) passes only dphi_hat = -alpha dC to the query, through the gradient of the
 // SDF; with U = d x n, sg = d . n, t = s (e_k - n_k n)/rho:
-//   |d x t|^2 = sg^2 + (U_k/rho)^2,   gf . t = s (gf_k - n_k (gf . n))/rho
+//   |d x t|^2 = sg^2 + (U_k/rho)^2,   gf . t = s (rho^2 gf_k - n_k (gf_i n_i + gf_j n_j))/rho
 // (gf = Gl + Ga x d).  Simulations in which some lane of the warp is in contact go
 // through the general adjoint afterwards, for those lanes.
 //
@@ -432,14 +432,14 @@ __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const Param
     const float* g = G[m];
     const float gf[3] = {g[0] + g[4] * r[2] - g[5] * r[1], g[1] + g[5] * r[0] - g[3] * r[2],
                          g[2] + g[3] * r[1] - g[4] * r[0]};
-    const float gn = gf[0] * n[0] + gf[1] * n[1] + gf[2] * n[2];
-    float dC = gn * rcp_fast(fma_(O.inv_inertia, dot3(U, U), O.inv_mass));     // -dC
+    const int k = m > 0 ? sim_axis(m) : 0, i = (k + 1) % 3, j = (k + 2) % 3;
+    const float A = gf[i] * n[i] + gf[j] * n[j];
+    float dC = (A + gf[k] * n[k]) * rcp_fast(fma_(O.inv_inertia, dot3(U, U), O.inv_mass));     // -dC
     if (m > 0) {
-      const int k = sim_axis(m), i = (k + 1) % 3, j = (k + 2) % 3;
-      const float rr = rsqrt_or_zero(n[i] * n[i] + n[j] * n[j]);
+      const float rho2 = n[i] * n[i] + n[j] * n[j], rr = rsqrt_bounded(rho2);
       const float Ur = U[k] * rr;
       const float rwt = rcp_fast(fma_(O.inv_inertia, fma_(Ur, Ur, sg * sg), O.inv_mass));
-      const float gt = (gf[k] - n[k] * gn) * rr;
+      const float gt = (rho2 * gf[k] - n[k] * A) * rr;
       dC += (sim_sign(m) * mu) * gt * rwt;
     } else {
       dC -= Pm.w_pen;                            // L_pen on the first step at rest
@@ -448,7 +448,7 @@ __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const Param
     touch |= kap ? 1u << m : 0u;
     const float dphi = kap ? 0.0f : Pm.alpha * dC;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) pb[k] = fmaf(dphi, smp.g[k], pb[k]);
+    for (int e = 0; e < 3; ++e) pb[e] = fmaf(dphi, smp.g[e], pb[e]);
   }
   unsigned wmask = __reduce_or_sync(kFull, valid ? touch : 0u);
   while (wmask) {
@@ -464,7 +464,7 @@ __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const Param
       float dphi, dn[3], dd[3], dsr[3];
       contact_adjoint(r, ps.n, sr, ps.phi_hat, true, G[m], G[m] + 3, Pm, O, m == 0 ? Pm.w_pen : 0.0f, dphi, dn, dd,
                       dsr);
-      sdf_adjoint(smp, ps, dphi, dn, dd);        // adds the lookup's adjoint; dsr does not reach p (sr is constant)
+      sdf_adjoint<ANY>(smp, ps, dphi, dn, dd);        // adds the lookup's adjoint; dsr does not reach p (sr is constant)
 #pragma unroll
       for (int k = 0; k < 3; ++k) pb[k] += dd[k];
     }
@@ -895,7 +895,7 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
               float dno[3], rtb[3];
               mat_t_vec(st.Rt, dn, dno);
               cross3(n, dn, rtb);
-              sdf_adjoint(smp, ps, dphi, dno, rb);          // adds the lookup's adjoint to rb
+              sdf_adjoint<ANY>(smp, ps, dphi, dno, rb);          // adds the lookup's adjoint to rb
               // r = R~^T d
               float Rrb[3], tmp[3];
               matvec3(st.Rt, rb, Rrb);
