@@ -34,7 +34,7 @@ namespace {
 constexpr int kQW = 8;                       // warps per candidate
 constexpr int kQBatchChunks = 32;            // chunks per contact batch (<= 1024 contacts)
 constexpr int kQBatch = 32 * kQBatchChunks;
-constexpr int kQD = 4;                       // directions per thread per pass over the contacts
+constexpr int kQD = 2;                       // directions per thread per pass over the contacts
 
 struct QualitySmem {
   HandDev H;
@@ -154,57 +154,64 @@ __global__ void __launch_bounds__(kQW * 32) measure_kernel(FusedArgs a, const fl
   work_done(a.work);
 }
 
-// Contact record in the batch: point p, outward normal n, tangent basis t1, t2.
-struct ContactRec {
-  float4 a;   // p.x p.y p.z n.x
-  float4 b;   // n.y n.z t1.x t1.y
-  float4 c;   // t1.z t2.x t2.y t2.z
+// Two contacts of the batch, value by value (x: the even one, y: the odd one): point p,
+// outward normal n, tangent basis t1, t2.
+struct ContactPair {
+  float2 p[3], n[3], t1[3], t2[3];
 };
 
 // max over the k cone edges of cos_e x + sin_e y, from the edges that can attain it.
 // The edges are symmetric under y -> -y, for even k under x -> -x and for k a
 // multiple of 4 under x <-> y, so after the matching reflections the angle of (x, y)
 // lies in [0, pi], [0, pi/2] or [0, pi/4] and only edges 0 .. last = k/2, k/4 or k/8 (rounded down)
-// can be the nearest.  Edge 0 is (1, 0).  LAST = 1 (k = 8, 12: two edges) is compiled
-// without the loop: of the 24 multiply-adds and maxima of 8 edges 6 remain.
+// can be the nearest.  Edge 0 is (1, 0).  EIGHT (k = 8) needs no order of |x| and |y|:
+// max(|x|, |y|, (|x| + |y|)/sqrt 2), 3 operations instead of 24.
 enum ConeSymmetry { kConeOdd = 0, kConeEven = 1, kConeQuad = 2 };
 __device__ __forceinline__ int cone_symmetry(int k) { return (k & 1) ? kConeOdd : (k & 3) ? kConeEven : kConeQuad; }
 __device__ __forceinline__ int cone_last_edge(int k) { return (k & 1) ? k / 2 : (k & 3) ? k / 4 : k / 8; }
 
-// Running maxima h of kQD directions (uf, ut) over contacts j0, j0 + stride, ...
-template <int LAST>
-__device__ __forceinline__ void fold_contacts(const ContactRec* rec, int nc, int j0, int stride, const float* ce,
+template <bool EIGHT>
+__device__ __forceinline__ float cone_max(float a1, float a2, const float* ce, const float* se, int sym, int last) {
+  if (EIGHT) return fmaxf(fmaxf(fabsf(a1), fabsf(a2)), ce[1] * (fabsf(a1) + fabsf(a2)));
+  float y = fabsf(a2), x = sym == kConeOdd ? a1 : fabsf(a1);
+  if (sym == kConeQuad) {
+    const float t = fmaxf(x, y);
+    y = fminf(x, y);
+    x = t;
+  }
+  float best = x;
+  for (int e = 1; e <= last; ++e) best = fmaxf(best, ce[e] * x + se[e] * y);
+  return best;
+}
+
+// Running maxima h of kQD directions over the contact pairs j0, j0 + stride, ...: the dot
+// products of both contacts of a pair in packed f32x2 arithmetic, every value of a
+// direction twice in a register pair.
+template <bool EIGHT>
+__device__ __forceinline__ void fold_contacts(const ContactPair* rec, int np, int j0, int stride, const float* ce,
                                               const float* se, int sym, int last, float mu,
                                               const float (&uf)[kQD][3], const float (&ut)[kQD][3], float (&h)[kQD]) {
-  const float c1 = ce[1], s1 = se[1];
-  for (int jc = j0; jc < nc; jc += stride) {
-    const float4 ra = rec[jc].a, rb = rec[jc].b, rc = rec[jc].c;
+  float2 f2[kQD][3], t2[kQD][3], m2[kQD][3];
+#pragma unroll
+  for (int d = 0; d < kQD; ++d)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      f2[d][k] = make_float2(uf[d][k], uf[d][k]);
+      t2[d][k] = make_float2(ut[d][k], ut[d][k]);
+      m2[d][k] = make_float2(-ut[d][k], -ut[d][k]);
+    }
+  for (int jp = j0; jp < np; jp += stride) {
+    const ContactPair c = rec[jp];
 #pragma unroll
     for (int d = 0; d < kQD; ++d) {
       // a = u_f + s (u_t x p)
-      const float ax = uf[d][0] + (ut[d][1] * ra.z - ut[d][2] * ra.y);
-      const float ay = uf[d][1] + (ut[d][2] * ra.x - ut[d][0] * ra.z);
-      const float az = uf[d][2] + (ut[d][0] * ra.y - ut[d][1] * ra.x);
-      const float an = ax * ra.w + ay * rb.x + az * rb.y;
-      const float a1 = ax * rb.z + ay * rb.w + az * rc.x;
-      const float a2 = ax * rc.y + ay * rc.z + az * rc.w;
-      float x, y, best;
-      if (LAST == 1) {
-        x = fmaxf(fabsf(a1), fabsf(a2));
-        y = fminf(fabsf(a1), fabsf(a2));
-        best = fmaxf(x, c1 * x + s1 * y);
-      } else {
-        y = fabsf(a2);
-        x = sym == kConeOdd ? a1 : fabsf(a1);
-        if (sym == kConeQuad) {
-          const float t = fmaxf(x, y);
-          y = fminf(x, y);
-          x = t;
-        }
-        best = x;
-        for (int e = 1; e <= last; ++e) best = fmaxf(best, ce[e] * x + se[e] * y);
-      }
-      h[d] = fmaxf(h[d], mu * best - an);
+      const float2 a[3] = {vfma(m2[d][2], c.p[1], vfma(t2[d][1], c.p[2], f2[d][0])),
+                           vfma(m2[d][0], c.p[2], vfma(t2[d][2], c.p[0], f2[d][1])),
+                           vfma(m2[d][1], c.p[0], vfma(t2[d][0], c.p[1], f2[d][2]))};
+      const float2 an = vdot(a, c.n), a1 = vdot(a, c.t1), a2 = vdot(a, c.t2);
+      const float vx = mu * cone_max<EIGHT>(a1.x, a2.x, ce, se, sym, last) - an.x;
+      const float vy = mu * cone_max<EIGHT>(a1.y, a2.y, ce, se, sym, last) - an.y;
+      h[d] = fmaxf(h[d], fmaxf(vx, vy));
     }
   }
 }
@@ -216,9 +223,9 @@ __device__ __forceinline__ int float_order(float x) {
 }
 __device__ __forceinline__ float order_float(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
-// Bound: the FP32 pipe in the fold, 22 instructions a (direction, contact) pair.
-// 8,192 candidates, 76 contacts each, 1,024 directions, 8 edges: 2.02 -> 0.74 ms (FMA
-// pipe 50% while the SMs are busy, 38% over the launch: candidates with over a
+// Bound: issue in the fold, 13 instructions a (direction, contact) pair with 8 edges.
+// 8,192 candidates, 76 contacts each, 1,024 directions, 8 edges: 2.02 -> 0.67 ms (FMA
+// pipe 33%; the SMs are busy 73% of the launch: candidates with over a
 // thousand contacts end last).
 template <bool ANY>
 __global__ void __launch_bounds__(kQW * 32) epsilon_kernel(FusedArgs a, float tau, float mu, int k_edges,
@@ -227,8 +234,8 @@ __global__ void __launch_bounds__(kQW * 32) epsilon_kernel(FusedArgs a, float ta
   __shared__ QualitySmem S;
   __shared__ unsigned short list[kQBatchChunks];
   extern __shared__ float4 dyn4[];
-  ContactRec* rec = reinterpret_cast<ContactRec*>(dyn4);        // [kQBatch]
-  int* hmax = reinterpret_cast<int*>(rec + kQBatch);            // [K], float_order
+  ContactPair* rec = reinterpret_cast<ContactPair*>(dyn4);      // [kQBatch / 2]
+  int* hmax = reinterpret_cast<int*>(rec + kQBatch / 2);        // [K], float_order
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NT = kQW * 32;
   if (tid == 0) S.hand_loaded = nullptr;
@@ -294,14 +301,26 @@ __global__ void __launch_bounds__(kQW * 32) epsilon_kernel(FusedArgs a, float ta
           const float bb = nr[0] * nr[1] * aa;
           const float t1[3] = {1.0f + sg * nr[0] * nr[0] * aa, sg * bb, -sg * nr[0]};
           const float t2[3] = {bb, sg + nr[1] * nr[1] * aa, -nr[1]};
-          ContactRec& r = rec[base + __popc(bal & ((1u << lane) - 1u))];
-          r.a = make_float4(p[0], p[1], p[2], nr[0]);
-          r.b = make_float4(nr[1], nr[2], t1[0], t1[1]);
-          r.c = make_float4(t1[2], t2[0], t2[1], t2[2]);
+          const int slot = base + __popc(bal & ((1u << lane) - 1u));
+          float* w = reinterpret_cast<float*>(rec + (slot >> 1)) + (slot & 1);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            w[2 * k] = p[k];
+            w[2 * (3 + k)] = nr[k];
+            w[2 * (6 + k)] = t1[k];
+            w[2 * (9 + k)] = t2[k];
+          }
         }
       }
       __syncthreads();
-      const int nc = S.count;
+      const int nc = S.count, np = (nc + 1) >> 1;
+      if (nc & 1) {                                     // the last contact stands twice
+        if (tid < 12) {
+          float* w = reinterpret_cast<float*>(rec + np - 1) + 2 * tid;
+          w[1] = w[0];
+        }
+        __syncthreads();
+      }
       // kQD directions per thread per pass: each contact record read from shared
       // memory serves all of them
       for (int w0 = tid; w0 < groups * ways && nc > 0; w0 += NT) {
@@ -318,10 +337,10 @@ __global__ void __launch_bounds__(kQW * 32) epsilon_kernel(FusedArgs a, float ta
           }
           h[d] = -INFINITY;
         }
-        if (sym == kConeQuad && last == 1)
-          fold_contacts<1>(rec, nc, way, ways, S.ce, S.se, sym, last, mu, uf, ut, h);
+        if (k_edges == 8)
+          fold_contacts<true>(rec, np, way, ways, S.ce, S.se, sym, last, mu, uf, ut, h);
         else
-          fold_contacts<0>(rec, nc, way, ways, S.ce, S.se, sym, last, mu, uf, ut, h);
+          fold_contacts<false>(rec, np, way, ways, S.ce, S.se, sym, last, mu, uf, ut, h);
 #pragma unroll
         for (int d = 0; d < kQD; ++d)
           if (k0 + d * groups < K) atomicMax(hmax + k0 + d * groups, float_order(h[d]));
@@ -379,7 +398,7 @@ cudaError_t launch_contact_measure(const FusedArgs& a0, const float* weights, fl
   return cudaGetLastError();
 }
 
-size_t epsilon_smem_bytes(int K) { return sizeof(ContactRec) * kQBatch + sizeof(float) * (size_t)K; }
+size_t epsilon_smem_bytes(int K) { return sizeof(ContactPair) * (kQBatch / 2) + sizeof(float) * (size_t)K; }
 
 cudaError_t launch_grasp_epsilon(const FusedArgs& a0, float tau, float mu, int k_edges, float tscale,
                                  const float* dirs, int K, float* eps, int* ncontact, cudaStream_t st) {
