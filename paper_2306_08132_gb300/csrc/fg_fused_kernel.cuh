@@ -276,6 +276,86 @@ __device__ __forceinline__ void unit_reduce_add_fixed(const float a[6], int lane
   if ((lane & 3) == 0 && k < 6) atomicAdd(slot + k, to_fixed(w));
 }
 
+// Forces and torques of a warp's 32 points in every simulation, added to the sums
+// wfix[m] (6 values and the count; the penetration of simulation 0 in its slot 7);
+// flags(m, word) takes the contact flags.  With the shared terms of the adjoint
+// (point_sims_adjoint), lambda_t = min(sigma, mu C)/w_t and sigma = c rho,
+//   f = A n + B e_k,              B = -s lambda_t/rho,  A = -lambda_n - B n_k
+//   d x f = A (U - s c E_k) + B p x e_k
+// so a simulation takes about 20 operations and 2 reciprocals where its own lever, cross
+// products and selects of the axis took about 110.  One axis at a time, the components
+// rotated so that it comes first: one copy of the code.  FORCE_FIGURES
+template <class F>
+__device__ __forceinline__ void chunk_forces(const PointState& ps, const SimConsts& K, bool valid, float c, float w_pen,
+                                             int lane, unsigned long long (*wfix)[8], F flags) {
+  const SimK4<float> k0 = simk4(K, 0.0f, 0);
+  const float mu = K.s[4];
+  SimShared<float> q;
+  sim_shared(ps, k0, q);
+  const int rank = lane >> 2;                      // unit_reduce: lane 4 rank holds value rank
+  const bool holds = (lane & 3) == 0 && rank < 6;
+  {
+    const bool kap = valid && ps.phi_hat < 0.0f;
+    const unsigned bal = __ballot_sync(kFull, kap);
+    flags(0, bal);
+    if (bal != 0u) {
+      const float al = kap ? ps.phi_hat * rcp_fast(q.wn) : 0.0f;       // -C/w_n
+      const float v[6] = {al * ps.n[0], al * ps.n[1], al * ps.n[2], al * q.U[0], al * q.U[1], al * q.U[2]};
+      const float w = unit_reduce(v, lane);
+      if (holds) atomicAdd(&wfix[0][rank], to_fixed(w));
+      if (lane == 0) atomicAdd(&wfix[0][6], (unsigned long long)__popc(bal));
+      if (w_pen != 0.0f) {
+        const float pen = warp_sum(kap ? -ps.phi_hat : 0.0f);
+        if (lane == 0) atomicAdd(&wfix[0][7], to_fixed(pen));
+      }
+    }
+  }
+  float n[3] = {ps.n[0], ps.n[1], ps.n[2]}, nn[3] = {q.nn[0], q.nn[1], q.nn[2]};
+  float p1 = ps.p[1], p2 = ps.p[2], p0 = ps.p[0], U0 = q.U[0], U1 = q.U[1], U2 = q.U[2];
+  int slot = rank < 3 ? rank : rank - 3;           // axis of the lane's value
+#pragma unroll 1
+  for (int k = 0; k < 3; ++k) {
+    const float rho2 = nn[1] + nn[2], rr = rsqrt_bounded(rho2), Ur = U0 * rr;
+    const float sigma = c * (rho2 * rr);
+    const float wn0 = fmaf(k0.z, rho2, q.wn), wn1 = k0.w * (U2 * n[1] - U1 * n[2]);
+    const float wt0 = fmaf(k0.y * Ur, Ur, fmaf(k0.z, nn[0], q.wt)), wt1 = q.tsg * n[0];
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      const float s = h == 0 ? 1.0f : -1.0f;
+      const float phm = fma_(-s * c, n[0], ps.phi_hat);                // sim_phi
+      const bool kap = valid && phm < 0.0f;
+      const unsigned bal = __ballot_sync(kFull, kap);
+      const int m = 1 + 2 * k + h;
+      flags(m, bal);
+      if (bal == 0u) continue;
+      float v[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+      if (kap) {
+        const float C = -phm;
+        const float lam_t = fminf(sigma, mu * C) * rcp_fast(fmaf(-s, wt1, wt0));
+        const float B = -s * lam_t * rr;
+        const float A = -fmaf(C, rcp_fast(fmaf(-s, wn1, wn0)), B * n[0]);
+        const float scA = s * c * A;
+        v[0] = fmaf(A, n[0], B);
+        v[1] = A * n[1];
+        v[2] = A * n[2];
+        // E_k = e_k x n = (0, -n_2, n_1) and p x e_k = (0, p_2, -p_1) in the rotated axes
+        v[3] = A * U0;
+        v[4] = fmaf(B, p2, fmaf(scA, n[2], A * U1));
+        v[5] = fmaf(-B, p1, fmaf(-scA, n[1], A * U2));
+      }
+      const float w = unit_reduce(v, lane);
+      if (holds) atomicAdd(&wfix[m][rank < 3 ? slot : 3 + slot], to_fixed(w));
+      if (lane == 0) atomicAdd(&wfix[m][6], (unsigned long long)__popc(bal));
+    }
+    // the next axis first
+    float t = n[0]; n[0] = n[1]; n[1] = n[2]; n[2] = t;
+    t = nn[0]; nn[0] = nn[1]; nn[1] = nn[2]; nn[2] = t;
+    t = U0; U0 = U1; U1 = U2; U2 = t;
+    t = p0; p0 = p1; p1 = p2; p2 = t;
+    slot = slot == 2 ? 0 : slot + 1;
+  }
+}
+
 // Adds 32 points' (g, r x g) to the warp's per-link sums.  Runs of points of one
 // link accumulate in registers (acc, for link cur) and are reduced when the link
 // changes; a group of 32 that straddles links is reduced link by link.
@@ -572,29 +652,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
           }
           PointState ps;
           point_state(smp, p, r, ps);
-#pragma unroll 1
-          for (int m = 0; m < kSims; ++m) {
-            const float phm = sim_phi(ps, m, dtV);
-            const bool kap = valid && phm < 0.0f;
-            const unsigned bal = __ballot_sync(kFull, kap);
+          chunk_forces(ps, S.K, valid, dtV, Pm.w_pen, lane, S.wfix, [&](int m, unsigned bal) {
             if (MODE == kModeWrench && lane == 0 && a.bits)
               a.bits[((size_t)c * kSims + m) * nwords + (base >> 5)] = bal;
-            if (bal == 0u) continue;
-            float v[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-            if (kap) {
-              float f[3], d[3], tq[3];
-              contact_force(ps, m, -phm, Pm, O, f, d);
-              cross3(d, f, tq);
-              v[0] = f[0]; v[1] = f[1]; v[2] = f[2];
-              v[3] = tq[0]; v[4] = tq[1]; v[5] = tq[2];
-            }
-            unit_reduce_add_fixed(v, lane, S.wfix[m]);
-            if (lane == 0) atomicAdd(&S.wfix[m][6], (unsigned long long)__popc(bal));
-            if (m == 0 && Pm.w_pen != 0.0f) {
-              const float pen = warp_sum(kap ? -phm : 0.0f);
-              if (lane == 0) atomicAdd(&S.wfix[0][7], to_fixed(pen));
-            }
-          }
+          });
           idx = nidx;
         }
       }
