@@ -128,29 +128,41 @@ __device__ __forceinline__ float gs_tangent(const float n[3], const float D[3], 
   return sig;
 }
 
-// Correction of one projected point (C = -phi > 0): force f = -(lambda_n n +
-// lambda_t t) with lambda_n = C / w_n (Eq. 1) and Coulomb friction on the
-// tangential displacement (static when sigma <= mu C), torque d x f.
-__device__ __forceinline__ void gs_force(const PointState& ps, const float d[3], const float D[3], float C,
+// What a point keeps while the state changes: un = d x n, 1/w_n, s_d = d . n and
+// w_t's constant part.  With t normal to n, |d x t|^2 = s_d^2 + (un . t)^2.
+struct GsPoint {
+  float d[3], un[3], rwn, wt0;
+};
+__device__ __forceinline__ void gs_point(const PointState& ps, const float xt[3], const ObjDev& O, GsPoint& g) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) g.d[k] = sub_(ps.p[k], xt[k]);
+  cross3(g.d, ps.n, g.un);
+  g.rwn = rcp_fast(fma_(O.inv_inertia, dot3(g.un, g.un), O.inv_mass));
+  const float sd = dot3(g.d, ps.n);
+  g.wt0 = fma_(O.inv_inertia, mul_(sd, sd), O.inv_mass);
+}
+
+// Correction of one projected point (phi < 0): force f = -(lambda_n n + lambda_t t) with
+// lambda_n = C / w_n (Eq. 1) and Coulomb friction on the tangential displacement s =
+// D - (D . n) n (static when |s| <= mu C), torque d x f.  Every lane of the warp
+// computes its own from the common state (a branch for the projected lane and the terms
+// that do not depend on the state would lengthen the chain of projections).  With the
+// reverse's chain cut to gs_passage, 8 objects x 256 candidates: 0.98 -> 0.80 ms.
+__device__ __forceinline__ void gs_force(const PointState& ps, const GsPoint& g, const float D[3], float phi,
                                          const ParamsDev& P, const ObjDev& O, float f[3], float tq[3]) {
-  float un[3];
-  cross3(d, ps.n, un);
-  const float wn = fma_(O.inv_inertia, dot3(un, un), O.inv_mass);
-  const float lam_n = mul_(C, rcp_fast(wn));
+  const float lam = mul_(-phi, g.rwn), sn = dot3(ps.n, D);
+  float s[3], ds[3];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) f[k] = -mul_(lam_n, ps.n[k]);
-  float t[3], sn;
-  const float sig = gs_tangent(ps.n, D, t, sn);
-  if (sig > 0.0f) {
-    float ut[3];
-    cross3(d, t, ut);
-    const float wt = fma_(O.inv_inertia, dot3(ut, ut), O.inv_mass);
-    const float muC = mul_(P.mu, C);
-    const float lam_t = mul_(sig <= muC ? sig : muC, rcp_fast(wt));
+  for (int k = 0; k < 3; ++k) s[k] = fma_(-sn, ps.n[k], D[k]);
+  const float s2 = dot3(s, s), rs = rsqrt_or_zero(s2), us = mul_(dot3(g.un, s), rs);
+  const float bound = fminf(mul_(s2, rs), mul_(P.mu, -phi));
+  const float kt = mul_(mul_(bound, rs), rcp_fast(fma_(O.inv_inertia, mul_(us, us), g.wt0)));   // lambda_t / |s|
+  cross3(g.d, s, ds);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) f[k] = fma_(-lam_t, t[k], f[k]);
+  for (int k = 0; k < 3; ++k) {
+    f[k] = -fma_(kt, s[k], mul_(lam, ps.n[k]));
+    tq[k] = -fma_(kt, ds[k], mul_(lam, g.un[k]));
   }
-  cross3(d, f, tq);
 }
 
 // s += (f / m, (d x f) / I), the correction of lane j broadcast to the warp.
@@ -262,13 +274,11 @@ __device__ __forceinline__ void gs_leaky_rec(const PointState& ps, const float U
 }
 
 // General adjoint of a projected point: a is the adjoint of the state after
-// it, st the state before it.  Adds dL/dphi_hat, dL/dn, dL/dp and returns the
-// adjoint of the state before it minus a in ds (the correction's dependence on
-// the state through D).
+// it, st the state before it.  Adds dL/dphi_hat, dL/dn and dL/dp (the state's own
+// adjoint: gs_passage).
 __device__ __forceinline__ void gs_contact_adjoint(const PointState& ps, const float xt[3], const float st[6],
                                                    const float a[6], float extra_dC, const ParamsDev& P,
-                                                   const ObjDev& O, float& dphi, float dn[3], float dp[3],
-                                                   float ds[6]) {
+                                                   const ObjDev& O, float& dphi, float dn[3], float dp[3]) {
   float d[3], D[3];
   const float phi = gs_phi(ps, xt, st, d, D);
   const float C = -phi;
@@ -357,15 +367,39 @@ __device__ __forceinline__ void gs_contact_adjoint(const PointState& ps, const f
     dn[k] += nb[k];
   }
   // D = x~ + dx + dth x d
-  float dthb[3], ddb[3];
-  cross3(d, Db, dthb);                                   // d(Db . (dth x d))/ddth = d x Db
-  cross3(Db, st + 3, ddb);                               // ... /dd = Db x dth
+  float ddb[3];
+  cross3(Db, st + 3, ddb);                               // d(Db . (dth x d))/dd = Db x dth
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    ds[k] = Db[k];
-    ds[3 + k] = dthb[k];
-    dp[k] += dd[k] + ddb[k];
-  }
+  for (int k = 0; k < 3; ++k) dp[k] += dd[k] + ddb[k];
+}
+
+// What the state adjoint's passage through a projected point needs, from the state before
+// it: with gf = a_x/m + (a_th x d)/I, gn = gf . n, gt = gf . t and L = gf . f,
+//   dL/dC = -(gn/w_n + [kinetic] mu gt/w_t),
+//   dL/ds = -k1 (gf - gn n - [kinetic] gt t) + k2 gt (un - us t),
+//   k1 = lambda_t/|s|,  k2 = 2 lambda_t us/(I w_t |s|)
+// and dL/dD = dL/dC n + dL/ds, so that only these few operations stand in the chain of
+// projections; a point's own dL/dphi, dL/dn and dL/dp follow for all lanes at once.
+struct GsPassage {
+  float t[3], mr, k1, kt, k2;      // mr = [kinetic] mu/w_t, kt = [kinetic] k1 - k2 us
+};
+__device__ __forceinline__ void gs_passage(const PointState& ps, const GsPoint& g, const float xt[3],
+                                           const float st[6], const ParamsDev& P, const ObjDev& O, GsPassage& q) {
+  float d[3], D[3];
+  const float phi = gs_phi(ps, xt, st, d, D), sn = dot3(ps.n, D), muC = mul_(P.mu, -phi);
+  float s[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) s[k] = fma_(-sn, ps.n[k], D[k]);
+  const float s2 = dot3(s, s), rs = rsqrt_or_zero(s2), us = dot3(g.un, s) * rs, sig = s2 * rs;
+  const float rwt = rcp_fast(fmaf(O.inv_inertia, us * us, g.wt0));
+  const bool kin = sig > muC;
+  const float lam = (kin ? muC : sig) * rwt;
+  q.mr = kin ? P.mu * rwt : 0.0f;
+  q.k1 = kin ? lam * rs : (s2 > 0.0f ? rwt : 0.0f);
+  q.k2 = 2.0f * O.inv_inertia * lam * rwt * us * rs;
+  q.kt = (kin ? q.k1 : 0.0f) - q.k2 * us;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) q.t[k] = s[k] * rs;
 }
 
 // One chunk of simulation m in reverse: from the state st0 at its start, the
@@ -378,22 +412,24 @@ __device__ __forceinline__ void gs_chunk_reverse(const PointState& ps, const flo
                                                  const ObjDev& O, float smine[6], float amine[6], float& dphi,
                                                  float dn[3], float dp[3]) {
   float st[6];
+  GsPoint g;
+  gs_point(ps, xt, O, g);
 #pragma unroll
   for (int k = 0; k < 6; ++k) st[k] = smine[k] = st0[k];
   for (unsigned rest = mask; rest; rest &= rest - 1u) {   // forward re-run, lanes in order
     const int j = __ffs(rest) - 1;
-    float f[3] = {0.0f, 0.0f, 0.0f}, tq[3] = {0.0f, 0.0f, 0.0f};
-    if (lane == j) {
-      float d[3], D[3];
-      const float phi = gs_phi(ps, xt, st, d, D);
-      gs_force(ps, d, D, -phi, P, O, f, tq);
-    }
+    float d[3], D[3], f[3], tq[3];
+    const float phi = gs_phi(ps, xt, st, d, D);
+    gs_force(ps, g, D, phi, P, O, f, tq);
     gs_apply(st, f, tq, O, j);
     if (lane > j) {
 #pragma unroll
       for (int k = 0; k < 6; ++k) smine[k] = st[k];
     }
   }
+  GsPassage q;
+  gs_passage(ps, g, xt, smine, P, O, q);
+  const float extra = m == 0 ? P.w_pen : 0.0f;
   int hi = 32;
   for (unsigned rest = mask; rest;) {                     // events in reverse
     const int j = 31 - __clz(rest);
@@ -402,16 +438,28 @@ __device__ __forceinline__ void gs_chunk_reverse(const PointState& ps, const flo
 #pragma unroll
       for (int k = 0; k < 6; ++k) amine[k] = a[k];
     }
-    float ds[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    if (lane == j) gs_contact_adjoint(ps, xt, smine, a, m == 0 ? P.w_pen : 0.0f, P, O, dphi, dn, dp, ds);
+    float gf[3], Db[3], w[3];
+    cross3(a + 3, g.d, gf);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) a[k] += __shfl_sync(kFull, ds[k], j);
+    for (int k = 0; k < 3; ++k) gf[k] = fmaf(O.inv_inertia, gf[k], O.inv_mass * a[k]);
+    const float gn = dot3(gf, ps.n), gt = dot3(gf, q.t);
+    const float cn = extra - fmaf(q.mr, gt, gn * g.rwn) + q.k1 * gn, ct = q.kt * gt, cu = q.k2 * gt;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      Db[k] = fmaf(cn, ps.n[k], fmaf(-q.k1, gf[k], fmaf(ct, q.t[k], cu * g.un[k])));
+    cross3(g.d, Db, w);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      a[k] += __shfl_sync(kFull, Db[k], j);
+      a[3 + k] += __shfl_sync(kFull, w[k], j);
+    }
     hi = j;
   }
   if (lane < hi) {
 #pragma unroll
     for (int k = 0; k < 6; ++k) amine[k] = a[k];
   }
+  if ((mask >> lane) & 1u) gs_contact_adjoint(ps, xt, smine, amine, extra, P, O, dphi, dn, dp);
 }
 
 // Lookup of point i: from its closest face when the faces are kept (mesh objects).
@@ -617,6 +665,8 @@ __global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_ke
             gs_lookup<false, ANY>(O, p, faces, valid ? i : 32 * jn, smp);
             PointState ps;
             point_state(smp, p, r, ps);
+            GsPoint g;
+            gs_point(ps, xt, O, g);
             int last = -1;
             for (;;) {
               float d[3], Dd[3];
@@ -624,9 +674,9 @@ __global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_ke
               const unsigned cand = __ballot_sync(kFull, valid && lane > last && phi < 0.0f);
               if (!cand) break;
               const int jl = __ffs(cand) - 1;
-              float f[3] = {0.0f, 0.0f, 0.0f}, tq[3] = {0.0f, 0.0f, 0.0f};
+              float f[3], tq[3];
+              gs_force(ps, g, Dd, phi, Pm, O, f, tq);
               if (lane == jl) {
-                gs_force(ps, d, Dd, -phi, Pm, O, f, tq);
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                   Wl[k] += f[k];
