@@ -617,8 +617,10 @@ static __device__ __noinline__ int mesh_closest_warp(const ObjDev& O, const floa
   int stack[kBvhStack];
   int sp = 0, node = 0, best = done ? -1 : init;
   float best_d2 = done ? -1.0f : (init >= 0 ? init_d2 : 3.0e38f);
+  // a node's box comes with the test that leads to it: one trip to memory a level
+  // (mesh batch of 8 x 128 candidates 1.41 -> 1.36 ms)
+  float4 lo = __ldg(O.bvh), hi = __ldg(O.bvh + 1);
   for (;;) {
-    const float4 lo = __ldg(O.bvh + 2 * node), hi = __ldg(O.bvh + 2 * node + 1);
     const int count = __float_as_int(hi.w);
     if (count > 0) {
       // the leaf's faces whose plane is near enough for some lane (their loads overlap)
@@ -645,8 +647,9 @@ static __device__ __noinline__ int mesh_closest_warp(const ObjDev& O, const floa
       }
     } else {
       const int l = node + 1, r = __float_as_int(lo.w);
-      const float dl = box_dist2(p, __ldg(O.bvh + 2 * l), __ldg(O.bvh + 2 * l + 1));
-      const float dr = box_dist2(p, __ldg(O.bvh + 2 * r), __ldg(O.bvh + 2 * r + 1));
+      const float4 llo = __ldg(O.bvh + 2 * l), lhi = __ldg(O.bvh + 2 * l + 1);
+      const float4 rlo = __ldg(O.bvh + 2 * r), rhi = __ldg(O.bvh + 2 * r + 1);
+      const float dl = box_dist2(p, llo, lhi), dr = box_dist2(p, rlo, rhi);
       const bool need_l = __any_sync(0xffffffffu, dl < best_d2);
       const bool need_r = __any_sync(0xffffffffu, dr < best_d2);
       // nearer child first: the one nearer for most lanes
@@ -654,19 +657,20 @@ static __device__ __noinline__ int mesh_closest_warp(const ObjDev& O, const floa
       const int nearc = left_first ? l : r, farc = left_first ? r : l;
       const bool need_near = left_first ? need_l : need_r, need_far = left_first ? need_r : need_l;
       if (need_near && need_far && sp < kBvhStack) stack[sp++] = farc;
-      if (need_near) {
-        node = nearc;
-        continue;
-      }
-      if (need_far) {
-        node = farc;
+      if (need_near || need_far) {
+        const bool left = need_near == left_first;       // the near one, or the far one alone
+        node = need_near ? nearc : farc;
+        lo = left ? llo : rlo;
+        hi = left ? lhi : rhi;
         continue;
       }
     }
     bool found = false;
     while (sp > 0) {
       const int cand = stack[--sp];
-      if (__any_sync(0xffffffffu, box_dist2(p, __ldg(O.bvh + 2 * cand), __ldg(O.bvh + 2 * cand + 1)) < best_d2)) {
+      lo = __ldg(O.bvh + 2 * cand);
+      hi = __ldg(O.bvh + 2 * cand + 1);
+      if (__any_sync(0xffffffffu, box_dist2(p, lo, hi) < best_d2)) {
         node = cand;
         found = true;
         break;

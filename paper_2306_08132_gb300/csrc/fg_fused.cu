@@ -20,13 +20,13 @@ constexpr int kCfg8 = 4;         // 8 warps, >= 3 CTAs per SM
 constexpr int kCfg16 = 11;       // 16 warps, >= 1 CTA per SM
 
 // Warps per candidate of a launch without a selected configuration.  With few
-// candidates the chip is filled by giving each more warps: 152 candidates of 4,352
-// points 0.181 ms with 4 warps, 0.119 with 8, 0.080 with 16; 456: 0.192, 0.136, 0.131;
-// 912: 0.275, 0.208, 0.229; 1,824: 0.360, 0.309, 0.394; 8,192: within 2% with 4 and 8.  A small hand has too few
-// chunks to share (640 points: 304 candidates 0.060, 0.049, 0.058; 1,216: 0.084,
-// 0.087, 0.139).  On a mesh a candidate inside the object costs many times the others, so more
-// warps shorten the end of the launch (2,208 faces: 1,024 candidates 2.57, 1.45, 1.33;
-// 4,096: 6.71, 4.59, 4.36; 8,192: 9.73, 7.56, 8.01).
+// candidates the chip is filled by giving each more warps (ms with 4, 8, 16 warps;
+// 4,352 points): 152 candidates 0.100, 0.069, 0.049; 456: 0.145, 0.102, 0.099; 912: 0.189,
+// 0.150, 0.166; 1,824: 0.251, 0.225, 0.297; 4,096: 0.433, 0.445, 0.626.  A small hand has too
+// few chunks to share (640 points: 152 candidates 0.041, 0.033, 0.028; 304: 0.044, 0.037,
+// 0.044; 912: 0.058, 0.059, 0.092).  On a mesh a candidate inside the object costs many
+// times the others, so more warps shorten the end of the launch (2,208 faces: 1,024
+// candidates 2.11, 1.40, 1.29; 4,096: 6.03, 4.49, 4.08; 8,192: 9.19, 7.65, 7.55).
 static int default_config(const FusedArgs& a) {
   const long long sms = device_sm_count(), B = a.B;
   const bool large = a.hand_P >= 2048;
