@@ -54,9 +54,9 @@ sys.path.insert(0, ROOT)
 # the oracle's counting instantiation (oracle/flop_count.py); the same for the
 # 4- and 5-finger hands.
 FLOPS_PER_POINT_STEP = 2092
-# The fused kernel's own minimal count for a point out of contact (forward once +
-# leaky adjoint once, FMA = 2), reported beside it.
-KERNEL_MIN_FLOPS_PER_POINT_STEP = 599
+# The fused kernel's own minimal count for a point of a candidate without contacts (its
+# chunk culled from the forward sweep, the adjoint's closed form once, FMA = 2), reported beside it.
+KERNEL_MIN_FLOPS_PER_POINT_STEP = 250
 # The same count for the Gauss-Seidel form (oracle counting instantiation, this workload).
 GS_FLOPS_PER_POINT_STEP = 2540
 # The T-step form, by the number of simulation steps T (same counter, same workload).
@@ -513,8 +513,8 @@ def roofline_of(w, S_in, kern_ms, peak, hbm_gbs, hbm_basis, prof):
                                   "forward pass + reverse mode, both arms of every select)"},
         "kernel_minimal": {"flops_per_point_step": KERNEL_MIN_FLOPS_PER_POINT_STEP,
                            "frac": KERNEL_MIN_FLOPS_PER_POINT_STEP * units / kern_s / 1e12 / P,
-                           "basis": "the fused kernel's own operation count for a point out of contact "
-                                    "(forward once + leaky adjoint once, FMA = 2); contacts add work"},
+                           "basis": "the fused kernel's own operation count for a point of a candidate without contacts "
+                                    "(culled forward + closed-form adjoint, FMA = 2); contacts add work"},
         "executed_fp32": None,
     }
     if prof and "executed_fp32_flops_per_point_step" in prof:
