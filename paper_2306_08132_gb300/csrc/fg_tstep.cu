@@ -3,7 +3,7 @@
 // SDF at each simulation's predicted object pose, and the gradient is the
 // hand-written adjoint of the whole chain, reversed step by step.
 //
-// One CTA of 4 warps per candidate (persistent over candidates and optimisation
+// One CTA of 4 or 8 warps per candidate (persistent over candidates and optimisation
 // steps).  Per optimisation step:
 //
 //   FK            warp 0 (as in the one-step kernel)
@@ -17,8 +17,8 @@
 //                 object-state adjoint; lanes 0..6 carry it to the previous step
 //   tree, update  as in the one-step kernel
 //
-// Work is assigned to warps in a fixed pattern (chunk j to warp j mod 4) and
-// every reduction has a fixed order, so results are bit-reproducible.
+// Work is assigned to eight slots of partial sums in a fixed pattern (chunk j to slot j
+// mod 8) and every reduction has a fixed order, so results are bit-reproducible.
 #include <cuda_runtime.h>
 
 #include "fg_fused_kernel.cuh"
@@ -28,7 +28,10 @@ namespace fg {
 
 namespace {
 
-constexpr int kTW = 4;                        // warps per candidate
+constexpr int kTSlots = 8;                    // partial sums of a candidate, in a fixed order
+// Warps per candidate: 4, or 8 for few candidates.  Work is dealt to the 8 slots, warp w
+// taking slots w, w + TW, ..., so the sums do not depend on the number of warps.
+constexpr int kTWarps = 4, kTWide = 8;
 constexpr int kTSteps = FG_MAX_SIM_STEPS;
 
 // One simulation step as the forward computed it; the reverse reads it back.
@@ -54,8 +57,8 @@ struct TstepSmem {
   float x[kSims][3], Rc[kSims][9], v[kSims][3], w[kSims][3];   // current object state
   float G[kSims][6];          // dL/dW_lin, dL/dW_ang of the step being reversed
   float ab[kSims][12];        // adjoint of a state: x, R (world-frame rotation vector), v, w
-  float red[kTW][kSims][12];  // per-warp partial sums
-  float lacc[kTW][kMaxLinks][6];
+  float red[kTSlots][kSims][12];  // per-slot partial sums
+  float lacc[kTSlots][kMaxLinks][6];
   float uacc[kMaxUnits][6];   // first step's reverse: per work unit, sum g, sum (p - t) x g
   int next_unit;              // its next unclaimed work unit
   unsigned act[kSims][kMaxCullChunks / 32];   // forward: chunks that may touch the object, per simulation
@@ -578,7 +581,7 @@ __device__ __forceinline__ void point_wrench(const float p[3], const float t0[3]
 // The first step's reverse sweep: per-link sums of (g, (p - t0) x g), by work units
 // claimed from a counter (as in the one-step kernel), or by fixed ranges of points for
 // hands with more units than uacc holds.
-template <bool ANY, bool NEAR>
+template <bool ANY, bool NEAR, int TW>
 __device__ __forceinline__ void first_reverse_sweep(TstepSmem& S, const ObjDev& O, float rdil, int lane, int warp) {
   const HandDev& H = S.H;
   const float c = mul_(S.Pm.dt, S.Pm.V);
@@ -605,28 +608,30 @@ __device__ __forceinline__ void first_reverse_sweep(TstepSmem& S, const ObjDev& 
       unit_reduce_store(sum, lane, S.uacc[u]);
     }
   } else {
-    int cur = -1;
-    float acc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    const int span = (H.nchunks + kTW - 1) / kTW, jb = warp * span, je = min(H.nchunks, jb + span);
-    for (int j = jb; j < je; ++j) {
-      const int i = 32 * j + lane;
-      const bool valid = i < H.P;
-      const float4 sp = __ldg(H.pts + (valid ? i : 32 * j));
-      const int link = (int)sp.w;
-      float p[3], pb[3], v[6];
-      world_point(S.frame4[link], sp, p);
-      first_reverse_point<ANY, NEAR>(O, S.Pm, S.G, p, valid, rdil, c, pb);
-      point_wrench(p, t0, pb, valid, v);
-      link_accumulate(S.lacc[warp], lane, link, valid, v, cur, acc);
+    for (int slot = warp; slot < kTSlots; slot += TW) {
+      int cur = -1;
+      float acc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+      const int span = (H.nchunks + kTSlots - 1) / kTSlots, jb = slot * span, je = min(H.nchunks, jb + span);
+      for (int j = jb; j < je; ++j) {
+        const int i = 32 * j + lane;
+        const bool valid = i < H.P;
+        const float4 sp = __ldg(H.pts + (valid ? i : 32 * j));
+        const int link = (int)sp.w;
+        float p[3], pb[3], v[6];
+        world_point(S.frame4[link], sp, p);
+        first_reverse_point<ANY, NEAR>(O, S.Pm, S.G, p, valid, rdil, c, pb);
+        point_wrench(p, t0, pb, valid, v);
+        link_accumulate(S.lacc[slot], lane, link, valid, v, cur, acc);
+      }
+      __syncwarp();
+      if (cur >= 0) unit_reduce_add(acc, lane, S.lacc[slot][cur]);
     }
-    __syncwarp();
-    if (cur >= 0) unit_reduce_add(acc, lane, S.lacc[warp][cur]);
   }
 }
 
 // ANY = false: grid objects only; true: grids and meshes (the lookup dispatches on the kind).
-template <int MODE, bool ANY>
-__global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
+template <int MODE, bool ANY, int TW>
+__global__ void __launch_bounds__(TW * 32, 16 / TW) tstep_kernel(FusedArgs a) {
   __shared__ TstepSmem S;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) S.hand_loaded = nullptr;
@@ -646,7 +651,7 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
     if (a.hand != S.hand_loaded) {
       const int* src = reinterpret_cast<const int*>(a.hand);
       int* dst = reinterpret_cast<int*>(&S.H);
-      for (int k = tid; k < (int)(sizeof(HandDev) / sizeof(int)); k += kTW * 32) dst[k] = src[k];
+      for (int k = tid; k < (int)(sizeof(HandDev) / sizeof(int)); k += TW * 32) dst[k] = src[k];
       __syncthreads();
       if (tid == 0) S.hand_loaded = a.hand;
     }
@@ -677,7 +682,7 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
 #pragma unroll
         for (int k = 0; k < 9; ++k) S.Rc[m][k] = (k % 4 == 0) ? 1.0f : 0.0f;
       }
-      for (int idx = tid; idx < kTW * kMaxLinks * 6; idx += kTW * 32) (&S.lacc[0][0][0])[idx] = 0.0f;
+      for (int idx = tid; idx < kTSlots * kMaxLinks * 6; idx += TW * 32) (&S.lacc[0][0][0])[idx] = 0.0f;
       __syncthreads();
 
       // ------------------------------------------------------------- forward
@@ -703,7 +708,7 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
           // one test per chunk for all simulations: their queries lie within dt V of the points
           const float c = mul_(dt, Pm.V);
           if (cull) {
-            for (int j0 = warp * 32; j0 < H.nchunks; j0 += kTW * 32) {
+            for (int j0 = warp * 32; j0 < H.nchunks; j0 += TW * 32) {
               const int j = j0 + lane;
               bool active = j < H.nchunks;
               if (active) {
@@ -718,21 +723,22 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
               if (lane == 0) S.act[0][j0 >> 5] = word;
             }
           }
-          for (int idx = tid; idx < kTW * kSims * 12; idx += kTW * 32) (&S.red[0][0][0])[idx] = 0.0f;
+          for (int idx = tid; idx < kTSlots * kSims * 12; idx += TW * 32) (&S.red[0][0][0])[idx] = 0.0f;
           __syncthreads();
-          for (int j = warp; j < H.nchunks; j += kTW) {
-            if (cull && !((S.act[0][j >> 5] >> (j & 31)) & 1u)) continue;
-            const int i = 32 * j + lane;
-            const bool valid = i < P;
-            const float4 sp = __ldg(H.pts + (valid ? i : 32 * j));
-            float p[3];
-            world_point(S.frame4[(int)sp.w], sp, p);
-            first_forward_chunk<ANY>(O, Pm, p, valid, rdil, c, lane, S.red[warp]);
-          }
+          for (int slot = warp; slot < kTSlots; slot += TW)
+            for (int j = slot; j < H.nchunks; j += kTSlots) {
+              if (cull && !((S.act[0][j >> 5] >> (j & 31)) & 1u)) continue;
+              const int i = 32 * j + lane;
+              const bool valid = i < P;
+              const float4 sp = __ldg(H.pts + (valid ? i : 32 * j));
+              float p[3];
+              world_point(S.frame4[(int)sp.w], sp, p);
+              first_forward_chunk<ANY>(O, Pm, p, valid, rdil, c, lane, S.red[slot]);
+            }
         } else {
         if (cull) {
           const int span = ((H.nchunks + 31) >> 5) * 32;
-          for (int e = tid; e < kSims * span; e += kTW * 32) {      // a warp's 32 entries share m
+          for (int e = tid; e < kSims * span; e += TW * 32) {      // a warp's 32 entries share m
             const int m = e / span, j = e - m * span;
             bool active = false;
             if (j < H.nchunks) {
@@ -752,42 +758,44 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
         }
         for (int m = 0; m < kSims; ++m) {
           const SimStep st = S.st[t][m];          // registers: the sweep also writes shared memory
-          float W[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, cnt = 0.0f;
-          for (int j = warp; j < H.nchunks; j += kTW) {
-            if (cull && !((S.act[m][j >> 5] >> (j & 31)) & 1u)) continue;   // no contact possible
-            const int base = 32 * j, i = base + lane;
-            const bool valid = i < P;
-            const float4 sp = __ldg(H.pts + (valid ? i : base));
-            float p[3], d[3], r[3];
-            world_point(S.frame4[(int)sp.w], sp, p);
-            step_query(st, p, d, r);
-            if (!(ANY && O.kind == kObjMesh)) {
-              // point by point (one pyramid entry each): phi_hat(r) >= min - rdil
-              const float mn = point_min_bound(O, r);
-              if (__all_sync(kFull, !valid || mn - rdil - (1e-6f + 1e-5f * fabsf(mn)) > 0.0f)) continue;
+          for (int slot = warp; slot < kTSlots; slot += TW) {
+            float W[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, cnt = 0.0f;
+            for (int j = slot; j < H.nchunks; j += kTSlots) {
+              if (cull && !((S.act[m][j >> 5] >> (j & 31)) & 1u)) continue;   // no contact possible
+              const int base = 32 * j, i = base + lane;
+              const bool valid = i < P;
+              const float4 sp = __ldg(H.pts + (valid ? i : base));
+              float p[3], d[3], r[3];
+              world_point(S.frame4[(int)sp.w], sp, p);
+              step_query(st, p, d, r);
+              if (!(ANY && O.kind == kObjMesh)) {
+                // point by point (one pyramid entry each): phi_hat(r) >= min - rdil
+                const float mn = point_min_bound(O, r);
+                if (__all_sync(kFull, !valid || mn - rdil - (1e-6f + 1e-5f * fabsf(mn)) > 0.0f)) continue;
+              }
+              SdfSample smp;
+              sdf_lookup<false, ANY>(O, r, smp);
+              PointState ps;
+              point_state(smp, r, rdil, ps);
+              const bool kap = valid && ps.phi_hat < 0.0f;
+              cnt += (float)__popc(__ballot_sync(kFull, kap));
+              if (kap) {
+                float n[3], sr[3], f[3], tq[3];
+                matvec3(st.Rt, ps.n, n);
+                material_displacement(st, d, sr);
+                force_general(d, n, sr, -ps.phi_hat, Pm, O, f);
+                cross3(d, f, tq);
+                W[0] += f[0]; W[1] += f[1]; W[2] += f[2];
+                W[3] += tq[0]; W[4] += tq[1]; W[5] += tq[2];
+              }
             }
-            SdfSample smp;
-            sdf_lookup<false, ANY>(O, r, smp);
-            PointState ps;
-            point_state(smp, r, rdil, ps);
-            const bool kap = valid && ps.phi_hat < 0.0f;
-            cnt += (float)__popc(__ballot_sync(kFull, kap));
-            if (kap) {
-              float n[3], sr[3], f[3], tq[3];
-              matvec3(st.Rt, ps.n, n);
-              material_displacement(st, d, sr);
-              force_general(d, n, sr, -ps.phi_hat, Pm, O, f);
-              cross3(d, f, tq);
-              W[0] += f[0]; W[1] += f[1]; W[2] += f[2];
-              W[3] += tq[0]; W[4] += tq[1]; W[5] += tq[2];
-            }
-          }
 #pragma unroll
-          for (int k = 0; k < 6; ++k) {
-            const float v = warp_sum(W[k]);
-            if (lane == 0) S.red[warp][m][k] = v;
+            for (int k = 0; k < 6; ++k) {
+              const float v = warp_sum(W[k]);
+              if (lane == 0) S.red[slot][m][k] = v;
+            }
+            if (lane == 0) S.red[slot][m][6] = cnt;
           }
-          if (lane == 0) S.red[warp][m][6] = cnt;
         }
         }
         __syncthreads();
@@ -799,7 +807,7 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
           for (int k = 0; k < 7; ++k) {
             float v = 0.0f;
 #pragma unroll
-            for (int w = 0; w < kTW; ++w) v += S.red[w][m][k];
+            for (int w = 0; w < kTSlots; ++w) v += S.red[w][m][k];
             Wt[k] = v;
           }
           const float Nc = fmaxf(Wt[6], 1.0f);
@@ -888,9 +896,9 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
         __syncthreads();
         if (t == 0) {               // the adjoint of the initial state is not needed
           if (near_queries(O, mul_(dt, Pm.V)))
-            first_reverse_sweep<ANY, true>(S, O, rdil, lane, warp);
+            first_reverse_sweep<ANY, true, TW>(S, O, rdil, lane, warp);
           else
-            first_reverse_sweep<ANY, false>(S, O, rdil, lane, warp);
+            first_reverse_sweep<ANY, false, TW>(S, O, rdil, lane, warp);
           __syncthreads();
           break;
         }
@@ -899,135 +907,137 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
           const float Gl[3] = {S.G[m][0], S.G[m][1], S.G[m][2]};
           const float Ga[3] = {S.G[m][3], S.G[m][4], S.G[m][5]};
           const float t0[3] = {S.q[0], S.q[1], S.q[2]};
-          float accS[12];
+          for (int slot = warp; slot < kTSlots; slot += TW) {
+            float accS[12];
 #pragma unroll
-          for (int k = 0; k < 12; ++k) accS[k] = 0.0f;
-          int cur = -1;
-          float accL[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-          // contiguous chunks per warp: a warp meets each link in one run
-          const int span = (H.nchunks + kTW - 1) / kTW, jb = warp * span, je = min(H.nchunks, jb + span);
-          for (int j = jb; j < je; ++j) {
-            const int base = 32 * j, i = base + lane;
-            const bool valid = i < P;
-            const float4 sp = __ldg(H.pts + (valid ? i : base));
-            const int link = (int)sp.w;
-            float p[3], d[3], r[3];
-            world_point(S.frame4[link], sp, p);
-            step_query(st, p, d, r);
-            // A warp with no point in contact in this simulation and step takes the
-            // leaky-only adjoint: C = 0 there, so the force direction (normal,
-            // tangent) carries no gradient and only dphi_hat = -alpha dC reaches
-            // the query, through the gradient of the SDF (no curvature term).
-            SdfIndex ix;
-            float corner[8];
-            SdfSample msmp;              // mesh objects: the whole lookup (value, gradient, curvature) at once
-            bool touch;
-            if (ANY && O.kind == kObjMesh) {
-              mesh_lookup(O, r, msmp);
-              touch = sub_(msmp.phi, rdil) < 0.0f;
-            } else {
-              sdf_index(O, r, ix);
-              sdf_gather(O, ix, corner);
-              touch = query_in_contact(O, ix, corner, rdil);
-            }
-            float pb[3];
-            if (!__any_sync(kFull, valid && touch)) {
-              SdfSample smp;
-              if (ANY && O.kind == kObjMesh)
-                smp = msmp;
-              else
-                sdf_finish<false>(O, ix, corner, smp);
-              PointState ps;
-              point_state(smp, r, rdil, ps);
-              float n[3], sr[3];
-              matvec3(st.Rt, ps.n, n);
-              material_displacement(st, d, sr);
-              const float dphi = leaky_adjoint(d, n, sr, Gl, Ga, Pm, O);
-              float rb[3], Rrb[3], rtb[3];
+            for (int k = 0; k < 12; ++k) accS[k] = 0.0f;
+            int cur = -1;
+            float accL[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+            // contiguous chunks per slot: a warp meets each link in one run
+            const int span = (H.nchunks + kTSlots - 1) / kTSlots, jb = slot * span, je = min(H.nchunks, jb + span);
+            for (int j = jb; j < je; ++j) {
+              const int base = 32 * j, i = base + lane;
+              const bool valid = i < P;
+              const float4 sp = __ldg(H.pts + (valid ? i : base));
+              const int link = (int)sp.w;
+              float p[3], d[3], r[3];
+              world_point(S.frame4[link], sp, p);
+              step_query(st, p, d, r);
+              // A warp with no point in contact in this simulation and step takes the
+              // leaky-only adjoint: C = 0 there, so the force direction (normal,
+              // tangent) carries no gradient and only dphi_hat = -alpha dC reaches
+              // the query, through the gradient of the SDF (no curvature term).
+              SdfIndex ix;
+              float corner[8];
+              SdfSample msmp;              // mesh objects: the whole lookup (value, gradient, curvature) at once
+              bool touch;
+              if (ANY && O.kind == kObjMesh) {
+                mesh_lookup(O, r, msmp);
+                touch = sub_(msmp.phi, rdil) < 0.0f;
+              } else {
+                sdf_index(O, r, ix);
+                sdf_gather(O, ix, corner);
+                touch = query_in_contact(O, ix, corner, rdil);
+              }
+              float pb[3];
+              if (!__any_sync(kFull, valid && touch)) {
+                SdfSample smp;
+                if (ANY && O.kind == kObjMesh)
+                  smp = msmp;
+                else
+                  sdf_finish<false>(O, ix, corner, smp);
+                PointState ps;
+                point_state(smp, r, rdil, ps);
+                float n[3], sr[3];
+                matvec3(st.Rt, ps.n, n);
+                material_displacement(st, d, sr);
+                const float dphi = leaky_adjoint(d, n, sr, Gl, Ga, Pm, O);
+                float rb[3], Rrb[3], rtb[3];
 #pragma unroll
-              for (int k = 0; k < 3; ++k) rb[k] = dphi * smp.g[k];
-              matvec3(st.Rt, rb, Rrb);
-              cross3(Rrb, d, rtb);
+                for (int k = 0; k < 3; ++k) rb[k] = dphi * smp.g[k];
+                matvec3(st.Rt, rb, Rrb);
+                cross3(Rrb, d, rtb);
 #pragma unroll
-              for (int k = 0; k < 3; ++k) pb[k] = Rrb[k];
-              if (valid) {
+                for (int k = 0; k < 3; ++k) pb[k] = Rrb[k];
+                if (valid) {
+#pragma unroll
+                  for (int k = 0; k < 3; ++k) {
+                    accS[k] -= Rrb[k];         // x~
+                    accS[3 + k] += rtb[k];     // R~
+                  }
+                }
+              } else {
+                SdfSample smp;
+                if (ANY && O.kind == kObjMesh)
+                  smp = msmp;
+                else
+                  sdf_finish<true>(O, ix, corner, smp);
+                PointState ps;
+                point_state(smp, r, rdil, ps);
+                const bool kap = ps.phi_hat < 0.0f;
+                float n[3], sr[3];
+                matvec3(st.Rt, ps.n, n);
+                material_displacement(st, d, sr);
+                float dphi, dn[3], dd[3], dsr[3];
+                contact_adjoint(d, n, sr, ps.phi_hat, kap, Gl, Ga, Pm, O, 0.0f, dphi, dn, dd, dsr);
+                // sr = p - x - R r: r gets -R^T dsr, with R^T = R~^T Exp(wdt)
+                float e[3], rb[3];
+                exp_apply(st.wdt, st.c1, st.c2, 1.0f, dsr, e);
+                mat_t_vec(st.Rt, e, rb);
+                rb[0] = -rb[0]; rb[1] = -rb[1]; rb[2] = -rb[2];
+                // n = R~ n_obj
+                float dno[3], rtb[3];
+                mat_t_vec(st.Rt, dn, dno);
+                cross3(n, dn, rtb);
+                sdf_adjoint<ANY>(smp, ps, dphi, dno, rb);          // adds the lookup's adjoint to rb
+                // r = R~^T d
+                float Rrb[3], tmp[3];
+                matvec3(st.Rt, rb, Rrb);
+                cross3(Rrb, d, tmp);
+                float Rr[3], rRb[3];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                  accS[k] -= Rrb[k];         // x~
-                  accS[3 + k] += rtb[k];     // R~
+                  dd[k] += Rrb[k];
+                  rtb[k] += tmp[k];
+                  pb[k] = dd[k] + dsr[k];
+                  Rr[k] = d[k] + st.dtv[k] - sr[k];           // R r = p - x - sr
+                }
+                cross3(dsr, Rr, rRb);
+                if (valid) {
+#pragma unroll
+                  for (int k = 0; k < 3; ++k) {
+                    accS[k] -= dd[k];          // x~
+                    accS[3 + k] += rtb[k];     // R~
+                    accS[6 + k] -= dsr[k];     // x (through sr)
+                    accS[9 + k] += rRb[k];     // R (through sr)
+                  }
                 }
               }
-            } else {
-              SdfSample smp;
-              if (ANY && O.kind == kObjMesh)
-                smp = msmp;
-              else
-                sdf_finish<true>(O, ix, corner, smp);
-              PointState ps;
-              point_state(smp, r, rdil, ps);
-              const bool kap = ps.phi_hat < 0.0f;
-              float n[3], sr[3];
-              matvec3(st.Rt, ps.n, n);
-              material_displacement(st, d, sr);
-              float dphi, dn[3], dd[3], dsr[3];
-              contact_adjoint(d, n, sr, ps.phi_hat, kap, Gl, Ga, Pm, O, 0.0f, dphi, dn, dd, dsr);
-              // sr = p - x - R r: r gets -R^T dsr, with R^T = R~^T Exp(wdt)
-              float e[3], rb[3];
-              exp_apply(st.wdt, st.c1, st.c2, 1.0f, dsr, e);
-              mat_t_vec(st.Rt, e, rb);
-              rb[0] = -rb[0]; rb[1] = -rb[1]; rb[2] = -rb[2];
-              // n = R~ n_obj
-              float dno[3], rtb[3];
-              mat_t_vec(st.Rt, dn, dno);
-              cross3(n, dn, rtb);
-              sdf_adjoint<ANY>(smp, ps, dphi, dno, rb);          // adds the lookup's adjoint to rb
-              // r = R~^T d
-              float Rrb[3], tmp[3];
-              matvec3(st.Rt, rb, Rrb);
-              cross3(Rrb, d, tmp);
-              float Rr[3], rRb[3];
-#pragma unroll
-              for (int k = 0; k < 3; ++k) {
-                dd[k] += Rrb[k];
-                rtb[k] += tmp[k];
-                pb[k] = dd[k] + dsr[k];
-                Rr[k] = d[k] + st.dtv[k] - sr[k];           // R r = p - x - sr
-              }
-              cross3(dsr, Rr, rRb);
+              float vL[6];
               if (valid) {
+                const float rel[3] = {p[0] - t0[0], p[1] - t0[1], p[2] - t0[2]};
+                float tq[3];
+                cross3(rel, pb, tq);
+                vL[0] = pb[0]; vL[1] = pb[1]; vL[2] = pb[2];
+                vL[3] = tq[0]; vL[4] = tq[1]; vL[5] = tq[2];
+              } else {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                  accS[k] -= dd[k];          // x~
-                  accS[3 + k] += rtb[k];     // R~
-                  accS[6 + k] -= dsr[k];     // x (through sr)
-                  accS[9 + k] += rRb[k];     // R (through sr)
-                }
+                for (int k = 0; k < 6; ++k) vL[k] = 0.0f;
+              }
+              link_accumulate(S.lacc[slot], lane, link, valid, vL, cur, accL);
+            }
+            if (cur >= 0) {
+#pragma unroll
+              for (int k = 0; k < 6; ++k) {
+                const float sum = warp_sum(accL[k]);
+                if (lane == 0) S.lacc[slot][cur][k] += sum;
               }
             }
-            float vL[6];
-            if (valid) {
-              const float rel[3] = {p[0] - t0[0], p[1] - t0[1], p[2] - t0[2]};
-              float tq[3];
-              cross3(rel, pb, tq);
-              vL[0] = pb[0]; vL[1] = pb[1]; vL[2] = pb[2];
-              vL[3] = tq[0]; vL[4] = tq[1]; vL[5] = tq[2];
-            } else {
 #pragma unroll
-              for (int k = 0; k < 6; ++k) vL[k] = 0.0f;
+            for (int k = 0; k < 12; ++k) {
+              const float v = warp_sum(accS[k]);
+              if (lane == 0) S.red[slot][m][k] = v;
             }
-            link_accumulate(S.lacc[warp], lane, link, valid, vL, cur, accL);
-          }
-          if (cur >= 0) {
-#pragma unroll
-            for (int k = 0; k < 6; ++k) {
-              const float sum = warp_sum(accL[k]);
-              if (lane == 0) S.lacc[warp][cur][k] += sum;
-            }
-          }
-#pragma unroll
-          for (int k = 0; k < 12; ++k) {
-            const float v = warp_sum(accS[k]);
-            if (lane == 0) S.red[warp][m][k] = v;
           }
         }
         __syncthreads();
@@ -1039,7 +1049,7 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
           for (int k = 0; k < 3; ++k) {
             float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
 #pragma unroll
-            for (int w = 0; w < kTW; ++w) {
+            for (int w = 0; w < kTSlots; ++w) {
               s0 += S.red[w][m][k];
               s1 += S.red[w][m][3 + k];
               s2 += S.red[w][m][6 + k];
@@ -1074,7 +1084,7 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
           float x = 0.0f;
           if (lane < L) {
 #pragma unroll
-            for (int w = 0; w < kTW; ++w) x += S.lacc[w][lane][k];
+            for (int w = 0; w < kTSlots; ++w) x += S.lacc[w][lane][k];
             if (H.nunits <= kMaxUnits)
               for (int u = H.unit_begin[lane]; u < H.unit_begin[lane + 1]; ++u) x += S.uacc[u][k];
           }
@@ -1134,14 +1144,14 @@ __global__ void __launch_bounds__(kTW * 32, 4) tstep_kernel(FusedArgs a) {
   work_done(a.work);
 }
 
-template <int MODE, bool ANY>
+template <int MODE, bool ANY, int TW>
 cudaError_t launch_tstep_mode(const FusedArgs& a, cudaStream_t st) {
   static int blocks_per_sm[64] = {0};
   int dev = 0;
   cudaGetDevice(&dev);
   int& bps = blocks_per_sm[dev & 63];
   if (bps <= 0) {
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, tstep_kernel<MODE, ANY>, kTW * 32, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, tstep_kernel<MODE, ANY, TW>, TW * 32, 0);
     if (e != cudaSuccess) return e;
     if (bps < 1) bps = 1;
   }
@@ -1151,8 +1161,17 @@ cudaError_t launch_tstep_mode(const FusedArgs& a, cudaStream_t st) {
   FusedArgs b = a;
   cudaError_t e = work_pair(&b.work, st);
   if (e != cudaSuccess) return e;
-  tstep_kernel<MODE, ANY><<<(int)grid, kTW * 32, 0, st>>>(b);
+  tstep_kernel<MODE, ANY, TW><<<(int)grid, TW * 32, 0, st>>>(b);
   return cudaGetLastError();
+}
+
+template <int TW>
+cudaError_t launch_tstep_warps(int mode, const FusedArgs& a, cudaStream_t st) {
+  if (a.any_mesh)
+    return mode == kModeLossGrad ? launch_tstep_mode<kModeLossGrad, true, TW>(a, st)
+                                 : launch_tstep_mode<kModeOptimize, true, TW>(a, st);
+  return mode == kModeLossGrad ? launch_tstep_mode<kModeLossGrad, false, TW>(a, st)
+                               : launch_tstep_mode<kModeOptimize, false, TW>(a, st);
 }
 
 }  // namespace
@@ -1160,11 +1179,13 @@ cudaError_t launch_tstep_mode(const FusedArgs& a, cudaStream_t st) {
 cudaError_t launch_tstep(int mode, const FusedArgs& a, cudaStream_t st) {
   if (a.B <= 0) return cudaSuccess;
   if (a.P.sim_steps < 1 || a.P.sim_steps > kTSteps) return cudaErrorInvalidValue;
-  if (a.any_mesh)
-    return mode == kModeLossGrad ? launch_tstep_mode<kModeLossGrad, true>(a, st)
-                                 : launch_tstep_mode<kModeOptimize, true>(a, st);
-  return mode == kModeLossGrad ? launch_tstep_mode<kModeLossGrad, false>(a, st)
-                               : launch_tstep_mode<kModeOptimize, false>(a, st);
+  // Eight warps a candidate shorten its phases and fill the chip with few candidates (4,352
+  // points, T = 1: 152 candidates 0.217 -> 0.136 ms, 912: 0.444 -> 0.364, 2,048: 0.693 -> 0.663,
+  // 4,096: 1.197 -> 1.235; 640 points: 304 candidates 0.082 -> 0.065, 608: 0.085 -> 0.092), and the sweeps
+  // of the later steps balance better over them at any number (T = 2: 152 candidates 0.589 -> 0.354,
+  // 4,096: 4.18 -> 3.89; 640 points, 4,096: 1.25 -> 1.13).
+  const bool wide = a.P.sim_steps >= 2 || a.B <= (a.hand_P >= 2048 ? 12LL : 3LL) * device_sm_count();
+  return wide ? launch_tstep_warps<kTWide>(mode, a, st) : launch_tstep_warps<kTWarps>(mode, a, st);
 }
 
 }  // namespace fg
