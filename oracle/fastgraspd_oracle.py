@@ -534,6 +534,26 @@ class GSDecisions:
     below: torch.Tensor = None
 
 
+GS_RUN = 256          # most points evaluate_gs takes at once
+
+
+def _gs_run_end(p, nrm, phi_hat, x_pred, dx, dth, a: int, force: dict | None) -> int:
+    """End of the run of points from a on that evaluate_gs takes at once: a single point where one
+    is in contact in some simulation (or has a forced decision), otherwise the points up to the next such
+    one, at most GS_RUN.  A point without contact has C = 0 in value and leaves the state as it is,
+    so the points of a run see the state the sweep reaches the first one with."""
+    with torch.no_grad():
+        e = min(a + GS_RUN, p.shape[1])
+        d = p[:, a:e, None, :] - x_pred
+        D = x_pred + dx[:, None] + _cross(dth[:, None].expand_as(d), d)
+        stop = (phi_hat[:, a:e, None] - _dot(nrm[:, a:e, None, :].expand_as(D), D) < 0).any(-1).any(0)
+        for key in ("kappa", "static") if force else ():
+            if key in force:
+                stop = stop | force[key][0][:, a:e].any(-1).any(0)
+        first = torch.nonzero(stop).flatten()
+        return e if len(first) == 0 else max(a + int(first[0]), a + 1)
+
+
 def evaluate_gs(hand: Hand, obj: Obj, q: torch.Tensor, r: float, prm: Params,
                 dec: GSDecisions | None = None, anchor_mode: bool = False, force: dict | None = None) -> dict:
     """The one-step grasp metric with the constraints projected by a Gauss-Seidel
@@ -590,50 +610,53 @@ def evaluate_gs(hand: Hand, obj: Obj, q: torch.Tensor, r: float, prm: Params,
     dth = torch.zeros(B, M_SIMS, 3, dtype=F64)
     Wsum = torch.zeros(B, M_SIMS, 6, dtype=F64)
     phi_ms, Cs, sigs = [], [], []
-    # per-point views (unbind: the reverse pass gathers their gradients once)
-    p_i, n_i, ph_i = p.unbind(1), nrm.unbind(1), phi_hat.unbind(1)
-    for i in range(P):
-        n_ = n_i[i][:, None, :].expand(B, M_SIMS, 3)
-        d = p_i[i][:, None, :] - x_pred                               # [B,M,3]
-        Dsp = x_pred + dx + _cross(dth, d)                            # material point's displacement
-        phi_m = ph_i[i][:, None] - _dot(n_, Dsp)                      # [B,M]
+    a = 0
+    while a < P:
+        # points a .. b-1 see the same state: one point, or a run of points without contact
+        b = a + 1 if anchor_mode or not take else _gs_run_end(p, nrm, phi_hat, x_pred, dx, dth, a, force)
+        n_ = nrm[:, a:b, None, :].expand(B, b - a, M_SIMS, 3)
+        d = p[:, a:b, None, :] - x_pred                               # [B,n,M,3]
+        x_, th_ = dx[:, None], dth[:, None].expand(B, b - a, M_SIMS, 3)
+        Dsp = x_pred + x_ + _cross(th_, d)                            # material point's displacement
+        phi_m = phi_hat[:, a:b, None] - _dot(n_, Dsp)                 # [B,n,M]
         if take:
-            dec.state[:, i] = torch.cat([dx, dth], -1).detach()
-            dec.kappa[:, i] = _forced(phi_m.detach() < 0, force, "kappa", i)
+            dec.state[:, a:b] = torch.cat([dx, dth], -1).detach()[:, None]
+            dec.kappa[:, a:b] = _forced(phi_m.detach() < 0, force, "kappa", slice(a, b))
         if anchor_mode:
-            st = dec.state[:, i].clone()
+            st = dec.state[:, a:b].clone()
             dx_c, dth_c = st[..., :3], st[..., 3:]
         else:
-            dx_c, dth_c = dx.detach(), dth.detach()
-        phi_p = ph_i[i][:, None] - _dot(n_, x_pred + dx_c + _cross(dth_c, d))
+            dx_c, dth_c = x_.detach(), th_.detach()
+        phi_p = phi_hat[:, a:b, None] - _dot(n_, x_pred + dx_c + _cross(dth_c, d))
         if take:
-            dec.anchor[:, i] = phi_p.detach()
-        anchor = dec.anchor[:, i].clone() if anchor_mode else phi_p.detach()
-        kap = dec.kappa[:, i].clone()           # copies: the decision tables are filled in place
+            dec.anchor[:, a:b] = phi_p.detach()
+        anchor = dec.anchor[:, a:b].clone() if anchor_mode else phi_p.detach()
+        kap = dec.kappa[:, a:b].clone()         # copies: the decision tables are filled in place
         C = torch.where(kap, -phi_m, -alpha * (phi_p - anchor))
         u_n = _cross(d, n_)
         w_n = obj.inv_mass + obj.inv_inertia * _dot(u_n, u_n)
         lam_n = C / w_n
         s = Dsp - _dot(Dsp, n_)[..., None] * n_                       # tangential displacement
         if take:
-            dec.has_t[:, i] = (s.detach() * s.detach()).sum(-1) > 0
-        ht = dec.has_t[:, i].clone()
+            dec.has_t[:, a:b] = (s.detach() * s.detach()).sum(-1) > 0
+        ht = dec.has_t[:, a:b].clone()
         sig = _safe_norm(s, ht)
         t_hat = s / torch.where(ht, sig, torch.ones_like(sig))[..., None]
         u_t = _cross(d, t_hat)
         w_t = obj.inv_mass + obj.inv_inertia * _dot(u_t, u_t)
         if take:
-            dec.static[:, i] = _forced(sig.detach() <= prm.mu * C.detach(), force, "static", i)
-        stat = dec.static[:, i].clone()
+            dec.static[:, a:b] = _forced(sig.detach() <= prm.mu * C.detach(), force, "static", slice(a, b))
+        stat = dec.static[:, a:b].clone()
         lam_t = torch.where(ht, torch.where(stat, sig, prm.mu * C) / w_t, torch.zeros_like(sig))
-        f = -(lam_n[..., None] * n_ + lam_t[..., None] * t_hat)       # [B,M,3]
+        f = -(lam_n[..., None] * n_ + lam_t[..., None] * t_hat)       # [B,n,M,3]
         tq = _cross(d, f)
-        dx = dx + obj.inv_mass * f
-        dth = dth + obj.inv_inertia * tq
-        Wsum = Wsum + torch.cat([f, tq], -1)
+        dx = dx + obj.inv_mass * f.sum(1)
+        dth = dth + obj.inv_inertia * tq.sum(1)
+        Wsum = Wsum + torch.cat([f, tq], -1).sum(1)
         phi_ms.append(phi_m)
         Cs.append(C)
         sigs.append(sig)
+        a = b
     xdot = V[None] + dx / prm.dt
     thdot = dth / prm.dt
     if take:
@@ -641,13 +664,13 @@ def evaluate_gs(hand: Hand, obj: Obj, q: torch.Tensor, r: float, prm: Params,
         dec.w_nz = (thdot.detach() ** 2).sum(-1) > 0
     L_stable = (_safe_norm(xdot, dec.v_nz) + _safe_norm(thdot, dec.w_nz)).sum(-1) / M_SIMS   # Eq. (2)
     L_range, L_limit = _joint_losses(hand, q, dec)
-    C = torch.stack(Cs, 1)                                            # [B,P,M]
+    C = torch.cat(Cs, 1)                                              # [B,P,M]
     L_pen = C[..., 0].sum(-1)
     L = L_stable + prm.w_range * L_range + prm.w_limit * L_limit + prm.w_pen * L_pen
     return {"L": L, "L_stable": L_stable, "L_range": L_range, "L_limit": L_limit, "L_pen": L_pen,
             "W": Wsum, "N": dec.kappa.sum(1).to(F64), "kappa": dec.kappa, "dx": dx, "dth": dth,
-            "points": p, "phi_hat": phi_hat, "grad_phi": grad, "phi_m": torch.stack(phi_ms, 1), "C": C,
-            "sigma": torch.stack(sigs, 1), "dec": dec}
+            "points": p, "phi_hat": phi_hat, "grad_phi": grad, "phi_m": torch.cat(phi_ms, 1), "C": C,
+            "sigma": torch.cat(sigs, 1), "dec": dec}
 
 
 def evaluate_any(hand: Hand, obj: Obj, q: torch.Tensor, r: float, prm: Params, dec=None,

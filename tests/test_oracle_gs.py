@@ -256,3 +256,24 @@ def test_repeated_sweeps_converge_to_a_feasible_state(plane):
     assert v[1] > 1e-4
     assert 0 < v[3] < 0.1 * v[1]
     assert v[60] < 1e-12
+
+
+@pytest.mark.parametrize("w_pen", [0.0, 2.0])
+def test_gs_runs_of_points_equal_one_point_at_a_time(monkeypatch, w_pen):
+    """Points without contact are evaluated in runs that share the state: the same results, bit for bit, as a
+    sweep that takes the points one at a time."""
+    w = synth.tiny_sphere_workload(n_cand=6)
+    S = O.Setup(w.hand, w.objects, dict(w.params, gauss_seidel=1, w_pen=w_pen))
+    runs = O.loss_and_grad(S.hand, S.objs[0], w.q0, 0.004, S.prm)
+    band = O.decision_band(S.hand, S.objs[0], w.q0, 0.004, S.prm, phi_tol=1e-5)
+    assert runs["kappa"].any() and sum(len(b["L"]) for b in band["branches"]) > len(w.q0)
+    monkeypatch.setattr(O, "GS_RUN", 1)
+    single = O.loss_and_grad(S.hand, S.objs[0], w.q0, 0.004, S.prm)
+    band1 = O.decision_band(S.hand, S.objs[0], w.q0, 0.004, S.prm, phi_tol=1e-5)
+    for name in ("L", "grad", "W", "N", "kappa", "dx", "dth", "phi_m", "C", "sigma"):
+        assert torch.equal(runs[name], single[name]), name
+    for name in ("kappa", "has_t", "static", "anchor", "state"):
+        assert torch.equal(getattr(runs["dec"], name), getattr(single["dec"], name)), name
+    for a, b in zip(band["branches"], band1["branches"]):
+        for name in ("L", "grad", "W"):
+            np.testing.assert_array_equal(a[name], b[name])
