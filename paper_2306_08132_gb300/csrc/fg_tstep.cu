@@ -342,9 +342,12 @@ __device__ __forceinline__ void rotate_from(int k, const float o[3], float v[3])
 
 // A contact of the first step with lever d and normal n (components rotated, the
 // velocity's axis first; s its sign, 0 at rest): U = d x n, s_d = d . n and the inverse
-// masses, |d x t|^2 = s_d^2 + (U_0/rho)^2 (t normal to n).
+// masses, |d x t|^2 = s_d^2 + (U_0/rho)^2 (t normal to n).  Where the gradient is zero
+// (flat: n = 0) the whole displacement is tangential: t = s e_0, rho = 1,
+// |d x t|^2 = d_1^2 + d_2^2.
 struct FirstContact {
   float U[3], sd, rho2, rr, rwn, rwt;
+  bool flat;
 };
 __device__ __forceinline__ void first_contact(const float d[3], const float n[3], const ObjDev& O, FirstContact& q) {
   cross3(d, n, q.U);
@@ -352,8 +355,14 @@ __device__ __forceinline__ void first_contact(const float d[3], const float n[3]
   q.rho2 = n[1] * n[1] + n[2] * n[2];
   q.rr = rsqrt_bounded(q.rho2);
   const float Ur = q.U[0] * q.rr;
+  float ut2 = fmaf(Ur, Ur, q.sd * q.sd);
+  q.flat = q.rho2 == 0.0f && n[0] == 0.0f;
+  if (q.flat) {
+    q.rho2 = q.rr = 1.0f;
+    ut2 = d[1] * d[1] + d[2] * d[2];
+  }
   q.rwn = rcp_fast(fmaf(O.inv_inertia, dot3(q.U, q.U), O.inv_mass));
-  q.rwt = rcp_fast(fmaf(O.inv_inertia, fmaf(Ur, Ur, q.sd * q.sd), O.inv_mass));
+  q.rwt = rcp_fast(fmaf(O.inv_inertia, ut2, O.inv_mass));
 }
 // Its force f = A n + B e_0 and torque A U + B d x e_0, with lambda_t = min(c rho, mu C)/w_t,
 // B = -s lambda_t/rho, A = -C/w_n - B n_0.
@@ -393,9 +402,10 @@ __device__ __forceinline__ void first_contact_adjoint(const float d[3], const fl
   const float f[3] = {fmaf(A, n[0], B), A * n[1], A * n[2]};
   float fg_[3];
   cross3(f, ga, fg_);
+  const float k12 = q.flat ? kt : kn;              // flat: kn = 0, and w_t hangs on d_1^2 + d_2^2
   dd[0] = fmaf(kn, d[0], fmaf(w, n[0], fg_[0]));
-  dd[1] = fmaf(kn, d[1], fmaf(w, n[1], fmaf(ku, n[2], fg_[1])));
-  dd[2] = fmaf(kn, d[2], fmaf(w, n[2], fmaf(-ku, n[1], fg_[2])));
+  dd[1] = fmaf(k12, d[1], fmaf(w, n[1], fmaf(ku, n[2], fg_[1])));
+  dd[2] = fmaf(k12, d[2], fmaf(w, n[2], fmaf(-ku, n[1], fg_[2])));
   dn[0] = fmaf(A, gf[0], fmaf(w, d[0], -B * gn));
   dn[1] = fmaf(A, gf[1], fmaf(w, d[1], fmaf(e, n[1], -ku * d[2])));
   dn[2] = fmaf(A, gf[2], fmaf(w, d[2], fmaf(e, n[2], ku * d[1])));
