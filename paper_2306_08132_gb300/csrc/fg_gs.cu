@@ -129,10 +129,15 @@ __device__ __forceinline__ float gs_tangent(const float n[3], const float D[3], 
 }
 
 // What a point keeps while the state changes: un = d x n, 1/w_n, s_d = d . n and
-// w_t's constant part.  With t normal to n, |d x t|^2 = s_d^2 + (un . t)^2.
+// w_t's constant part.  With t normal to n, |d x t|^2 = s_d^2 + (un . t)^2.  Where the
+// gradient is zero, n = 0 and all of D is tangential, so |d x t|^2 is formed from the
+// vectors, behind a branch that the warp takes only when some lane has such a point.
 struct GsPoint {
   float d[3], un[3], rwn, wt0;
+  bool some_flat;
 };
+__device__ __forceinline__ bool flat_normal(const float n[3]) { return n[0] == 0.0f && n[1] == 0.0f && n[2] == 0.0f; }
+// Every lane of the warp must call it.
 __device__ __forceinline__ void gs_point(const PointState& ps, const float xt[3], const ObjDev& O, GsPoint& g) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) g.d[k] = sub_(ps.p[k], xt[k]);
@@ -140,6 +145,7 @@ __device__ __forceinline__ void gs_point(const PointState& ps, const float xt[3]
   g.rwn = rcp_fast(fma_(O.inv_inertia, dot3(g.un, g.un), O.inv_mass));
   const float sd = dot3(g.d, ps.n);
   g.wt0 = fma_(O.inv_inertia, mul_(sd, sd), O.inv_mass);
+  g.some_flat = __any_sync(kFull, flat_normal(ps.n));
 }
 
 // Correction of one projected point (phi < 0): force f = -(lambda_n n + lambda_t t) with
@@ -156,8 +162,10 @@ __device__ __forceinline__ void gs_force(const PointState& ps, const GsPoint& g,
   for (int k = 0; k < 3; ++k) s[k] = fma_(-sn, ps.n[k], D[k]);
   const float s2 = dot3(s, s), rs = rsqrt_or_zero(s2), us = mul_(dot3(g.un, s), rs);
   const float bound = fminf(mul_(s2, rs), mul_(P.mu, -phi));
-  const float kt = mul_(mul_(bound, rs), rcp_fast(fma_(O.inv_inertia, mul_(us, us), g.wt0)));   // lambda_t / |s|
   cross3(g.d, s, ds);
+  float ut2 = mul_(us, us);
+  if (g.some_flat && flat_normal(ps.n)) ut2 = mul_(dot3(ds, ds), mul_(rs, rs));
+  const float kt = mul_(mul_(bound, rs), rcp_fast(fma_(O.inv_inertia, ut2, g.wt0)));   // lambda_t / |s|
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     f[k] = -fma_(kt, s[k], mul_(lam, ps.n[k]));
@@ -380,23 +388,34 @@ __device__ __forceinline__ void gs_contact_adjoint(const PointState& ps, const f
 //   k1 = lambda_t/|s|,  k2 = 2 lambda_t us/(I w_t |s|)
 // and dL/dD = dL/dC n + dL/ds, so that only these few operations stand in the chain of
 // projections; a point's own dL/dphi, dL/dn and dL/dp follow for all lanes at once.
+// Where n = 0, |d x t|^2 = |d|^2 - (d . t)^2: d and d . t stand in the places of un and us, and k2 changes sign.
 struct GsPassage {
   float t[3], mr, k1, kt, k2;      // mr = [kinetic] mu/w_t, kt = [kinetic] k1 - k2 us
 };
-__device__ __forceinline__ void gs_passage(const PointState& ps, const GsPoint& g, const float xt[3],
+__device__ __forceinline__ void gs_passage(const PointState& ps, GsPoint& g, const float xt[3],
                                            const float st[6], const ParamsDev& P, const ObjDev& O, GsPassage& q) {
   float d[3], D[3];
   const float phi = gs_phi(ps, xt, st, d, D), sn = dot3(ps.n, D), muC = mul_(P.mu, -phi);
   float s[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) s[k] = fma_(-sn, ps.n[k], D[k]);
-  const float s2 = dot3(s, s), rs = rsqrt_or_zero(s2), us = dot3(g.un, s) * rs, sig = s2 * rs;
-  const float rwt = rcp_fast(fmaf(O.inv_inertia, us * us, g.wt0));
+  const float s2 = dot3(s, s), rs = rsqrt_or_zero(s2), sig = s2 * rs;
+  float us = dot3(g.un, s) * rs, ut2 = us * us, sgn = 1.0f;
+  if (g.some_flat && flat_normal(ps.n)) {
+    float ds[3];
+    cross3(g.d, s, ds);
+    ut2 = dot3(ds, ds) * (rs * rs);
+    us = dot3(g.d, s) * rs;
+    sgn = -1.0f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) g.un[k] = g.d[k];
+  }
+  const float rwt = rcp_fast(fmaf(O.inv_inertia, ut2, g.wt0));
   const bool kin = sig > muC;
   const float lam = (kin ? muC : sig) * rwt;
   q.mr = kin ? P.mu * rwt : 0.0f;
   q.k1 = kin ? lam * rs : (s2 > 0.0f ? rwt : 0.0f);
-  q.k2 = 2.0f * O.inv_inertia * lam * rwt * us * rs;
+  q.k2 = sgn * (2.0f * O.inv_inertia * lam * rwt * us * rs);
   q.kt = (kin ? q.k1 : 0.0f) - q.k2 * us;
 #pragma unroll
   for (int k = 0; k < 3; ++k) q.t[k] = s[k] * rs;

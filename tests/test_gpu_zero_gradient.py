@@ -64,6 +64,13 @@ def _check(loss, grad, ref, idx):
     assert grel.max() < GRAD_TOL, (idx[np.argmax(grel)], grel.max())
 
 
+def _check_wrench(W, N, ref, idx):
+    assert np.array_equal(N.cpu().numpy()[idx], ref["N"][idx].astype(np.int32))
+    a, b = W.cpu().numpy().astype(np.float64)[idx].reshape(len(idx), -1), ref["W"][idx].reshape(len(idx), -1)
+    rel = np.linalg.norm(a - b, axis=1) / np.maximum(np.linalg.norm(b, axis=1), 1e-9)
+    assert rel.max() < GRAD_TOL, (idx[np.argmax(rel)], rel.max())
+
+
 @pytest.mark.parametrize("mu", [0.5, 0.05])
 @pytest.mark.parametrize("T", [1, 2])
 def test_zero_gradient_contacts_tstep(fg, case, T, mu):
@@ -71,3 +78,13 @@ def test_zero_gradient_contacts_tstep(fg, case, T, mu):
     ref, idx = case.reference(params)
     loss, grad = fg.loss_and_grad(case.hand, case.scene, case.q, params, R)
     _check(loss, grad, ref, idx)
+
+
+@pytest.mark.parametrize("mu", [0.5, 0.05])
+def test_zero_gradient_contacts_gauss_seidel(fg, case, mu):
+    params = dict(case.w.params, gauss_seidel=1, mu=mu)
+    ref, idx = case.reference(params)
+    loss, grad = fg.loss_and_grad(case.hand, case.scene, case.q, params, R)
+    _check(loss, grad, ref, idx)
+    W, N, _ = fg.contact_wrench(case.hand, case.scene, case.q, params, R)
+    _check_wrench(W, N, ref, idx)
