@@ -30,8 +30,8 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// Work units whose adjoint sums fit in shared memory (hands up to ~12,000 points);
-// larger hands use fixed per-warp point ranges.
+// Work units whose adjoint sums fit in shared memory (~12,000 points); larger hands are swept in as
+// many parts.
 constexpr int kMaxUnits = 192;
 
 template <int NW>
@@ -44,7 +44,6 @@ struct FusedSmem {
   float q[64];
   float grad[64];
   unsigned long long wfix[kSims][8];  // forward sums in fixed point: W (6), N (integer), pen
-  float lacc[NW][kMaxLinks][6];    // per warp, per link: sum g, sum (p - t) x g (fixed ranges)
   float uacc[kMaxUnits][6];        // per work unit: sum g, sum (p - t) x g
   float lsum[kMaxLinks][6];        // per link: sum g, sum (p - t) x g
   float Wtot[kSims][8];
@@ -399,83 +398,59 @@ __device__ __forceinline__ void link_accumulate(float (*lacc)[6], int lane, int 
   for (int k = 0; k < 6; ++k) acc[k] = 0.0f;
 }
 
-// Sweep 2 of one candidate: the adjoint of every point, reduced per link.
+// Sweep 2 of one candidate: the adjoint of the points of work units [u0, u1), at most
+// kMaxUnits, each unit's sums into its own slot of uacc.  Warps claim units
+// (<= 64 points of one link) from a shared counter, so a warp that meets contacts
+// (general adjoint) does not hold the others at the barrier, and the result does not
+// depend on which warp ran a unit, nor on the number of warps.  The next claim is issued before the
+// current unit so that its latency is hidden.
 template <int NW, int PPT, bool ANY, bool FREE>
-__device__ __forceinline__ void adjoint_sweep(FusedSmem<NW>& S, const ObjDev& O, float r, const int* faces, int lane, int warp) {
+__device__ __forceinline__ void adjoint_sweep(FusedSmem<NW>& S, const ObjDev& O, float r, const int* faces, int u0, int u1,
+                                              int lane) {
   const HandDev& H = S.H;
   const ParamsDev& Pm = S.Pm;
-  const int P = H.P;
   const float t0[3] = {S.q[0], S.q[1], S.q[2]};
-  if (H.nunits <= kMaxUnits) {
-    // Warps claim work units (<= 64 points of one link) from a shared
-    // counter, so a warp that meets contacts (general adjoint) does not hold
-    // the others at the barrier; each unit's sums go to its own slot, so the
-    // result does not depend on which warp ran it.  The next claim is issued
-    // before the current unit so that its latency is hidden.
-    auto claim = [&]() {
-      int j = 0;
-      if (lane == 0) j = atomicAdd(&S.next_unit, 1);
-      return __shfl_sync(kFull, j, 0);
-    };
-    int u = claim();
-    int4 U = __ldg(H.units + min(u, H.nunits - 1));      // first point, count, link
-    while (u < H.nunits) {
-      const int nu = claim();
-      const int4 nU = __ldg(H.units + min(nu, H.nunits - 1));
-      float sum[6];
-      if (PPT == 2) {
-        // one point of each half of the unit per lane, packed arithmetic
-        float v[2][6];
-        int link[2];
-        const bool va = lane < U.y, vb = lane + 32 < U.y;
-        point_adjoint_pair<ANY, FREE>(H, S.frame4, S.G, S.K, O, Pm, r, t0, faces, va ? U.x + lane : U.x,
-                                      vb ? U.x + 32 + lane : U.x, va, vb, v, link);
+  auto claim = [&]() {
+    int j = 0;
+    if (lane == 0) j = atomicAdd(&S.next_unit, 1);
+    return __shfl_sync(kFull, j, 0);
+  };
+  int u = claim();
+  int4 U = __ldg(H.units + min(u, u1 - 1));      // first point, count, link
+  while (u < u1) {
+    const int nu = claim();
+    const int4 nU = __ldg(H.units + min(nu, u1 - 1));
+    float sum[6];
+    if (PPT == 2) {
+      // one point of each half of the unit per lane, packed arithmetic
+      float v[2][6];
+      int link[2];
+      const bool va = lane < U.y, vb = lane + 32 < U.y;
+      point_adjoint_pair<ANY, FREE>(H, S.frame4, S.G, S.K, O, Pm, r, t0, faces, va ? U.x + lane : U.x,
+                                    vb ? U.x + 32 + lane : U.x, va, vb, v, link);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) sum[k] = v[0][k] + v[1][k];
-      } else {
+      for (int k = 0; k < 6; ++k) sum[k] = v[0][k] + v[1][k];
+    } else {
 #pragma unroll
-        for (int k = 0; k < 6; ++k) sum[k] = 0.0f;
-        // the next half's record is read before this half is computed
-        int i = lane < U.y ? U.x + lane : U.x;
-        float4 sp = __ldg(H.pts + i);
+      for (int k = 0; k < 6; ++k) sum[k] = 0.0f;
+      // the next half's record is read before this half is computed
+      int i = lane < U.y ? U.x + lane : U.x;
+      float4 sp = __ldg(H.pts + i);
 #pragma unroll 1
-        for (int h = 0; h < U.y; h += 32) {
-          const int ni = h + 32 + lane < U.y ? U.x + h + 32 + lane : U.x;
-          const float4 nsp = __ldg(H.pts + ni);
-          float v[6];
-          point_adjoint<ANY, FREE>(S.frame4, S.G, S.K, O, Pm, r, t0, faces, i, sp, U.z, h + lane < U.y, v);
+      for (int h = 0; h < U.y; h += 32) {
+        const int ni = h + 32 + lane < U.y ? U.x + h + 32 + lane : U.x;
+        const float4 nsp = __ldg(H.pts + ni);
+        float v[6];
+        point_adjoint<ANY, FREE>(S.frame4, S.G, S.K, O, Pm, r, t0, faces, i, sp, U.z, h + lane < U.y, v);
 #pragma unroll
-          for (int k = 0; k < 6; ++k) sum[k] += v[k];
-          i = ni;
-          sp = nsp;
-        }
-      }
-      unit_reduce_store(sum, lane, S.uacc[u]);
-      u = nu;
-      U = nU;
-    }
-  } else {
-    // fixed, contiguous 32-aligned point ranges per warp
-    int cur = -1;
-    float acc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    const int span = ((P + 32 * NW - 1) / (32 * NW)) * 32;
-    const int pb = warp * span, pe = min(P, pb + span);
-    for (int base = pb; base < pe; base += 32) {
-      float v[6];
-      const int i = base + lane;
-      const bool valid = i < pe;
-      const float4 sp = __ldg(H.pts + (valid ? i : base));
-      const int link = (int)sp.w;
-      point_adjoint<ANY, FREE>(S.frame4, S.G, S.K, O, Pm, r, t0, faces, valid ? i : base, sp, link, valid, v);
-      link_accumulate(S.lacc[warp], lane, link, valid, v, cur, acc);
-    }
-    if (cur >= 0) {
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        const float sum = warp_sum(acc[k]);
-        if (lane == 0) S.lacc[warp][cur][k] += sum;
+        for (int k = 0; k < 6; ++k) sum[k] += v[k];
+        i = ni;
+        sp = nsp;
       }
     }
+    unit_reduce_store(sum, lane, S.uacc[u - u0]);
+    u = nu;
+    U = nU;
   }
 }
 
@@ -719,8 +694,6 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
           if (lane == 0) S.loss = Ls + Pm.w_range * rn + Pm.w_limit * lims + Pm.w_pen * S.Wtot[0][7];
         }
       }
-      if (H.nunits > kMaxUnits)
-        for (int idx = tid; idx < NW * kMaxLinks * 6; idx += NW * 32) (&S.lacc[0][0][0])[idx] = 0.0f;
       if (tid == 0) S.next_unit = 0;
       __syncthreads();
       if (MODE == kModeLossGrad && a.grad == nullptr) {    // loss only: no adjoint
@@ -737,27 +710,27 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
       }
 
       // ---------------------------------------------------------------- sweep 2
-      // The whole CTA takes the short form when its candidate has no contact.
-      if (S.free)
-        adjoint_sweep<NW, PPT, ANY, true>(S, O, r, faces, lane, warp);
-      else
-        adjoint_sweep<NW, PPT, ANY, false>(S, O, r, faces, lane, warp);
-      __syncthreads();
+      // The whole CTA takes the short form when its candidate has no contact.  Hands of more than
+      // kMaxUnits units go in several parts; a link's sums add its units in their order in any case.
+      for (int u0 = 0; u0 < H.nunits; u0 += kMaxUnits) {
+        const int u1 = min(H.nunits, u0 + kMaxUnits);
+        if (S.free)
+          adjoint_sweep<NW, PPT, ANY, true>(S, O, r, faces, u0, u1, lane);
+        else
+          adjoint_sweep<NW, PPT, ANY, false>(S, O, r, faces, u0, u1, lane);
+        __syncthreads();
+        // per-link sums, one thread per link and component
+        for (int idx = tid; idx < L * 6; idx += NW * 32) {
+          const int l = idx / 6, k = idx - 6 * l;
+          float x = u0 == 0 ? 0.0f : S.lsum[l][k];
+          for (int u = max(H.unit_begin[l], u0); u < min(H.unit_begin[l + 1], u1); ++u) x += S.uacc[u - u0][k];
+          S.lsum[l][k] = x;
+        }
+        if (tid == 0) S.next_unit = u1;
+        __syncthreads();
+      }
 
       // ------------------------------------------------------------------ tree
-      // per-link sums, one thread per link and component
-      for (int idx = tid; idx < L * 6; idx += NW * 32) {
-        const int l = idx / 6, k = idx - 6 * l;
-        float x = 0.0f;
-        if (H.nunits <= kMaxUnits) {
-          for (int u = H.unit_begin[l]; u < H.unit_begin[l + 1]; ++u) x += S.uacc[u][k];
-        } else {
-#pragma unroll
-          for (int w = 0; w < NW; ++w) x += S.lacc[w][l][k];
-        }
-        S.lsum[l][k] = x;
-      }
-      __syncthreads();
       if (warp == 0) {
         // inclusive prefix over preorder links
         float pre[6];

@@ -12,6 +12,7 @@ import pytest
 import torch
 
 import synth
+import synth.meshes
 from oracle import fastgraspd_oracle as O
 
 pytestmark = pytest.mark.gpu
@@ -381,3 +382,44 @@ def test_query_past_every_face_of_the_grid(fg, dims):
     assert np.abs(phi.cpu().numpy() - (val + h * e)).max() <= 1.5e-5
     ok = np.array(smooth)
     assert np.abs(grad.cpu().numpy().T - g)[ok].max() <= 1e-4
+
+
+def test_large_hand_results_do_not_depend_on_the_batch(fg):
+    """A hand of 13,000 points (more work units than one part of the adjoint sweep takes): a candidate's results are
+    the same bits at every batch size (16, 8 and 4 warps a candidate), in every one-point configuration and in the
+    request queue, on a grid and on a mesh; and they match the oracle."""
+    h = synth.make_hand(3, 1300)
+    w = synth.tiny_sphere_workload(n_cand=12)
+    q = torch.tensor(synth.sample_candidates(np.random.default_rng(7), h, 2400, 0.095), device=_dev())
+    hand, sdf = fg.Hand.from_synth(h), fg.Sdf.from_synth(w.objects[0])
+    scene = fg.Scene([sdf])
+    first = q[:12].contiguous()
+    l0, g0 = fg.loss_and_grad(hand, scene, first, w.params, 0.004)
+    for B in (600, 2400):
+        l, g = fg.loss_and_grad(hand, scene, q[:B].contiguous(), w.params, 0.004)
+        assert torch.equal(l[:12], l0) and torch.equal(g[:12], g0), B
+    mesh = fg.Scene([fg.Sdf.from_synth(synth.meshes.icosphere(0.04, 2))])
+    lm, gm = fg.loss_and_grad(hand, mesh, first, w.params, 0.004)
+    try:
+        for i, (_, _, ppt) in enumerate(fg.fused_configs()):
+            if ppt == 1:
+                fg.fused_config_select(i)
+                for sc, lr, gr in ((scene, l0, g0), (mesh, lm, gm)):
+                    l, g = fg.loss_and_grad(hand, sc, first, w.params, 0.004)
+                    assert torch.equal(l, lr) and torch.equal(g, gr), i
+    finally:
+        fg.fused_config_select(-1)
+    q1 = first.clone()
+    fg.optimize_step(hand, scene, q1, w.params, 0, 10, 1)
+    queue = fg.Queue(1 << 30)
+    try:
+        rid = queue.submit(hand, sdf, first.cpu().numpy(), 1, w.params)
+        queue.wait(rid, 120000)
+        np.testing.assert_array_equal(queue.result(rid)[0], q1.cpu().numpy())
+    finally:
+        queue.close()
+    case = Case(fg, synth.Workload("large", h, w.objects, q[:12].cpu().numpy(), np.zeros(12, dtype=np.int32), w.params, 10))
+    ref = O.batch_loss_and_grad(case.S, case.w.q0, case.w.obj_of_cand, 0.004)
+    clean = case.clean(case.w.q0, 0.004)
+    assert clean.sum() >= 1
+    _compare_loss_grad(l0.cpu().numpy(), g0.cpu().numpy(), ref, clean)
