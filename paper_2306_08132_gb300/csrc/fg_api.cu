@@ -339,8 +339,8 @@ fg_status fg_sdf_create(const float* grid, int nx, int ny, int nz, const float* 
   int levels = 0;
   const size_t pf = min_pyramid_floats(nx, ny, nz, &levels);
   s->pyr = nullptr;
-  e = cudaMalloc(&s->pyr, sizeof(float) * pf);
-  if (e == cudaSuccess) e = build_min_pyramid(s->grid, nx, ny, nz, s->pyr, levels, o.pyr_off);
+  e = cudaMalloc(&s->pyr, sizeof(float) * (pf + 1));
+  if (e == cudaSuccess) e = build_min_pyramid(s->grid, nx, ny, nz, s->pyr, levels, o.pyr_off, &o.flat_min);
   if (e != cudaSuccess) {
     cudaFree(s->pyr);
     cudaFree(s->grid);
@@ -350,7 +350,7 @@ fg_status fg_sdf_create(const float* grid, int nx, int ny, int nz, const float* 
   o.pyr = s->pyr;
   o.pyr_levels = levels;
   o.kind = kObjGrid;
-  s->pyr_bytes = sizeof(float) * pf;
+  s->pyr_bytes = sizeof(float) * (pf + 1);
   s->mesh = nullptr;
   *out = s;
   return FG_OK;
@@ -377,7 +377,11 @@ fg_status fg_scene_create(const fg_sdf* const* sdfs, int n, fg_scene** out) {
   if (!sc) return FG_ERR_OOM;
   sc->n = n;
   sc->has_mesh = 0;
-  for (int i = 0; i < n; ++i) sc->has_mesh |= tab[i].kind == kObjMesh;
+  sc->flat_min = 3.0e38f;
+  for (int i = 0; i < n; ++i) {
+    sc->has_mesh |= tab[i].kind == kObjMesh;
+    sc->flat_min = std::min(sc->flat_min, tab[i].flat_min);
+  }
   cudaError_t e = cudaMalloc(&sc->dev, sizeof(ObjDev) * n);
   if (e != cudaSuccess) {
     delete sc;
@@ -470,6 +474,7 @@ fg_status fg_contact_wrench(const fg_hand* h, const fg_scene* sc, const int* oc,
   a.objs = sc->dev;
   a.n_obj = sc->n;
   a.any_mesh = sc->has_mesh;
+  a.any_flat = sc->flat_min < r;
   a.obj_of_cand = oc;
   a.q = const_cast<float*>(q);
   a.B = B;
@@ -499,6 +504,7 @@ fg_status fg_loss_and_grad(const fg_hand* h, const fg_scene* sc, const int* oc, 
   a.objs = sc->dev;
   a.n_obj = sc->n;
   a.any_mesh = sc->has_mesh;
+  a.any_flat = sc->flat_min < r;
   a.obj_of_cand = oc;
   a.q = const_cast<float*>(q);
   a.B = B;
@@ -534,6 +540,7 @@ fg_status fg_optimize_step(const fg_hand* h, const fg_scene* sc, const int* oc, 
   a.objs = sc->dev;
   a.n_obj = sc->n;
   a.any_mesh = sc->has_mesh;
+  a.any_flat = sc->flat_min < p->r0;
   a.obj_of_cand = oc;
   a.q = q;
   a.B = B;
@@ -687,6 +694,7 @@ fg_status fg_autotune(const fg_hand* h, const fg_scene* sc, const int* oc, const
   a.objs = sc->dev;
   a.n_obj = sc->n;
   a.any_mesh = sc->has_mesh;
+  a.any_flat = sc->flat_min < p->r0;
   a.obj_of_cand = oc;
   a.q = const_cast<float*>(q);
   a.B = B;

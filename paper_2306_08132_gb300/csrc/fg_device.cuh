@@ -61,6 +61,7 @@ struct alignas(16) ObjDev {
   float ox, oy, oz;              // origin
   float inv_h, h;                // 1/pitch, pitch
   float inv_mass, inv_inertia;
+  float flat_min;                // smallest value of a cell whose 8 corners are equal (3e38: none): n = 0 there
   const float* pyr;              // min-pyramid, level k at pyr + pyr_off[k - 1]
   int pyr_off[kMaxPyrLevels];
   // kind 1: a watertight triangle mesh queried directly (Phong SDF); the grid
@@ -1007,7 +1008,8 @@ __device__ __forceinline__ void sim_dir(int m, float vd[3]) {
 // Tangential unit vector t = (v - (v.n) n)/|v - (v.n) n| of a moving simulation
 // and rho = |e_k - n_k n| = sin(angle(n, v_m)).  rho^2 is the sum of the squares
 // of the two other components of n (no cancellation of 1 - n_k^2).  Returns 0
-// (and t = 0) when m = 0 or n is parallel to the velocity.
+// (and t = 0) when m = 0 or n is parallel to the velocity; where the gradient is zero
+// (n = 0) the whole velocity is tangential: t = v/|v|, rho = 1.
 __device__ __forceinline__ float sim_tangent(const float n[3], int m, float t[3]) {
   t[0] = t[1] = t[2] = 0.0f;
   if (m == 0) return 0.0f;
@@ -1018,6 +1020,12 @@ __device__ __forceinline__ float sim_tangent(const float n[3], int m, float t[3]
   const float ea = k0 ? n[1] : n[0];
   const float eb = k2 ? n[1] : n[2];
   const float rho2 = fma_(ea, ea, mul_(eb, eb));
+  if (rho2 == 0.0f && nk == 0.0f) {
+    t[0] = k0 ? sg : 0.0f;
+    t[1] = k1 ? sg : 0.0f;
+    t[2] = k2 ? sg : 0.0f;
+    return 1.0f;
+  }
   if (!(rho2 > 0.0f)) return 0.0f;
   const float rr = rsqrtf(rho2);
   const float rho = mul_(rho2, rr);
@@ -1389,6 +1397,41 @@ __device__ __forceinline__ void point_contacts_adjoint(const PointState& ps, con
       dn[i] += fmaf(A, gi, fmaf(w, p[i], fmaf(e, n[i], -ku * p[j])));
       dn[j] += fmaf(A, gj, fmaf(w, p[j], fmaf(e, n[j], ku * p[i])));
     }
+  }
+}
+
+// Contacts where the SDF's gradient is zero (a constant cell, a truncated field): n = 0, the
+// normal correction vanishes, and the whole displacement is tangential, t = s e_k:
+//   f = B e_k,  B = -s min(c, mu C)/w_t,  w_t = 1/m + (p_i^2 + p_j^2)/I,
+// about the lever d whose components i, j are those of p.  The short forms above and
+// chunk_forces have rho = 0 there and give none of it.
+__device__ __forceinline__ bool flat_contact(const PointState& ps) {
+  return ps.phi_hat < 0.0f && ps.n[0] == 0.0f && ps.n[1] == 0.0f && ps.n[2] == 0.0f;
+}
+__device__ __forceinline__ float flat_force(const PointState& ps, int m, const SimConsts& K, float c, float& pi,
+                                            float& pj, float& rwt) {
+  const int k = sim_axis(m);
+  pi = k == 0 ? ps.p[1] : k == 1 ? ps.p[2] : ps.p[0];
+  pj = k == 0 ? ps.p[2] : k == 1 ? ps.p[0] : ps.p[1];
+  rwt = rcp_fast(fmaf(K.s[1], fmaf(pi, pi, pj * pj), K.s[0]));
+  return -sim_sign(m) * fminf(c, -K.s[4] * ps.phi_hat) * rwt;
+}
+// Their adjoint through the lever (dL/dphi_hat and dL/dn meet a gradient of zero), added to dp.
+__device__ __forceinline__ void flat_contact_adjoint(const PointState& ps, const SimAdjoints& G, const SimConsts& K,
+                                                     float c, float dp[3]) {
+#pragma unroll 1
+  for (int m = 1; m < kSims; ++m) {
+    const int k = sim_axis(m);
+    float gl[3], ga[3], pi, pj, rwt;
+    get_sim_adjoint(G, m, gl, ga);
+    const float B = flat_force(ps, m, K, c, pi, pj, rwt);
+    const float gk = k == 0 ? gl[0] : k == 1 ? gl[1] : gl[2];
+    const float gi = k == 0 ? ga[1] : k == 1 ? ga[2] : ga[0], gj = k == 0 ? ga[2] : k == 1 ? ga[0] : ga[1];
+    const float kt = -2.0f * K.s[1] * (B * fmaf(gi, pj, fmaf(-gj, pi, gk)) * rwt);
+    const float di = fmaf(kt, pi, -B * gj), dj = fmaf(kt, pj, B * gi);
+    dp[0] += k == 0 ? 0.0f : k == 1 ? dj : di;
+    dp[1] += k == 0 ? di : k == 1 ? 0.0f : dj;
+    dp[2] += k == 0 ? dj : k == 1 ? di : 0.0f;
   }
 }
 

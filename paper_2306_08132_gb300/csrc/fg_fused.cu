@@ -60,6 +60,7 @@ void fused_config_select(int i) { selected_slot() = i; }
 cudaError_t launch_fused(int mode, const FusedArgs& a, const fg_hand* h, cudaStream_t st) {
   (void)h;
   if (a.B <= 0) return cudaSuccess;
+  if (a.any_flat) return launch_fused_flat(mode, a, st);
   const int chosen = selected_slot(), cfg = chosen < 0 ? default_config(a) : chosen;
   if (a.any_mesh) {
     switch (mode) {
@@ -78,6 +79,7 @@ cudaError_t launch_fused(int mode, const FusedArgs& a, const fg_hand* h, cudaStr
 // One round of a request queue: every active request's candidates in one launch.
 cudaError_t launch_queue_round(const FusedArgs& a, cudaStream_t st) {
   if (a.B <= 0) return cudaSuccess;
+  if (a.any_flat) return launch_fused_flat(kModeQueue, a, st);
   if (a.any_mesh) return launch_queue_round_any(a, st);
   return launch_fused_cfg<kModeQueue, 4, 5, 1>(a, st);
 }
@@ -109,7 +111,8 @@ cudaError_t autotune_fused(const FusedArgs& base, int reps, float* times_ms, int
       e = cudaMemcpyAsync(qtmp, base.q, sizeof(float) * (size_t)base.B * D, cudaMemcpyDeviceToDevice, st);
       if (e != cudaSuccess) break;
       cudaEventRecord(t0, st);
-      e = (base.any_mesh ? kOptimizeLaunchAny : kOptimizeLaunch)[i](a, st);
+      e = base.any_flat ? launch_fused_flat(kModeOptimize, a, st)
+                        : (base.any_mesh ? kOptimizeLaunchAny : kOptimizeLaunch)[i](a, st);
       cudaEventRecord(t1, st);
       if (e == cudaSuccess) e = cudaEventSynchronize(t1);
       float ms = 0.0f;

@@ -63,6 +63,7 @@ struct FusedSmem {
   float* qout;
   float* lout;
   int cl, step0, total, nsteps;
+  int flat;                        // FLAT kernels: the candidate has contacts where the SDF's gradient is zero
 };
 
 __device__ __forceinline__ void store_frame(const Frame& F, float4* f4) {
@@ -277,7 +278,8 @@ __device__ __forceinline__ void unit_reduce_add_fixed(const float a[6], int lane
 
 // Forces and torques of a warp's 32 points in every simulation, added to the sums
 // wfix[m] (6 values and the count; the penetration of simulation 0 in its slot 7);
-// flags(m, word) takes the contact flags.  With the shared terms of the adjoint
+// flags(m, word) takes the contact flags; with FLAT, *flat is set when a contact's gradient is
+// zero (its friction: flat_forces).  With the shared terms of the adjoint
 // (point_sims_adjoint), lambda_t = min(sigma, mu C)/w_t and sigma = c rho,
 //   f = A n + B e_k,              B = -s lambda_t/rho,  A = -lambda_n - B n_k
 //   d x f = A (U - s c E_k) + B p x e_k
@@ -285,9 +287,9 @@ __device__ __forceinline__ void unit_reduce_add_fixed(const float a[6], int lane
 // products and selects of the axis took about 110.  One axis at a time, the components
 // rotated so that it comes first: one copy of the code.  8-superquadric batch
 // 0.963 -> 0.924 ms, 256-object sweep 8.91 -> 8.60 ms.
-template <class F>
+template <bool FLAT, class F>
 __device__ __forceinline__ void chunk_forces(const PointState& ps, const SimConsts& K, bool valid, float c, float w_pen,
-                                             int lane, unsigned long long (*wfix)[8], F flags) {
+                                             int lane, unsigned long long (*wfix)[8], int* flat, F flags) {
   const SimK4<float> k0 = simk4(K, 0.0f, 0);
   const float mu = K.s[4];
   SimShared<float> q;
@@ -304,6 +306,7 @@ __device__ __forceinline__ void chunk_forces(const PointState& ps, const SimCons
       const float w = unit_reduce(v, lane);
       if (holds) atomicAdd(&wfix[0][rank], to_fixed(w));
       if (lane == 0) atomicAdd(&wfix[0][6], (unsigned long long)__popc(bal));
+      if (FLAT && kap && flat_contact(ps)) *flat = 1;
       if (w_pen != 0.0f) {
         const float pen = warp_sum(kap ? -ps.phi_hat : 0.0f);
         if (lane == 0) atomicAdd(&wfix[0][7], to_fixed(pen));
@@ -454,8 +457,74 @@ __device__ __forceinline__ void adjoint_sweep(FusedSmem<NW>& S, const ObjDev& O,
   }
 }
 
-// ANY = false: grid objects only (the mesh lookup is compiled out).
-template <int MODE, int NW, int MINB, int PPT, bool ANY>
+// The friction of contacts where the gradient is zero, added to the forward sums, and its
+// adjoint, added to the sums of units [u0, u1): passes of their own over the points, for
+// candidates that have such contacts, compiled into the FLAT kernels only.  In the kernels for all scenes the same
+// terms as selects in the two sweeps cost the 256-object sweep 6%, as branches 4%,
+// and the two calls 2%.
+template <int NW>
+__device__ __noinline__ void flat_forces(FusedSmem<NW>& S, float r, float c, int lane, int warp) {
+  const HandDev& H = S.H;
+  for (int j = warp; j < H.nchunks; j += NW) {
+    const int i = 32 * j + lane;
+    const bool valid = i < H.P;
+    const float4 sp = __ldg(H.pts + (valid ? i : 32 * j));
+    float p[3];
+    world_point(S.frame4[(int)sp.w], sp, p);
+    SdfSample smp;
+    sdf_lookup<false, true>(S.O, p, smp);
+    PointState ps;
+    point_state(smp, p, r, ps);
+    const bool flat = valid && flat_contact(ps);
+    if (!__any_sync(kFull, flat)) continue;
+#pragma unroll 1
+    for (int m = 1; m < kSims; ++m) {
+      const int k = sim_axis(m);
+      float pi, pj, rwt;
+      float B = flat_force(ps, m, S.K, c, pi, pj, rwt);
+      if (!flat) B = 0.0f;
+      // f = B e_k, d x f = B (p_j e_i - p_i e_j)
+      const float v[6] = {k == 0 ? B : 0.0f, k == 1 ? B : 0.0f, k == 2 ? B : 0.0f,
+                          B * (k == 0 ? 0.0f : k == 1 ? -pi : pj), B * (k == 0 ? pj : k == 1 ? 0.0f : -pi),
+                          B * (k == 0 ? -pi : k == 1 ? pj : 0.0f)};
+      const float w = unit_reduce(v, lane);
+      const int rank = lane >> 2;
+      if ((lane & 3) == 0 && rank < 6) atomicAdd(&S.wfix[m][rank], to_fixed(w));
+    }
+  }
+}
+template <int NW>
+__device__ __noinline__ void flat_adjoint(FusedSmem<NW>& S, float r, float c, int u0, int u1, int lane, int warp) {
+  const HandDev& H = S.H;
+  for (int u = u0 + warp; u < u1; u += NW) {
+    const int4 U = __ldg(H.units + u);
+    float sum[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    for (int h = 0; h < U.y; h += 32) {
+      const bool valid = h + lane < U.y;
+      const float4 sp = __ldg(H.pts + (valid ? U.x + h + lane : U.x));
+      float p[3];
+      world_point(S.frame4[U.z], sp, p);
+      SdfSample smp;
+      sdf_lookup<false, true>(S.O, p, smp);
+      PointState ps;
+      point_state(smp, p, r, ps);
+      float dp[3] = {0.0f, 0.0f, 0.0f}, tq[3];
+      if (valid && flat_contact(ps)) flat_contact_adjoint(ps, S.G, S.K, c, dp);
+      const float rel[3] = {p[0] - S.q[0], p[1] - S.q[1], p[2] - S.q[2]};
+      cross3(rel, dp, tq);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        sum[k] += dp[k];
+        sum[3 + k] += tq[k];
+      }
+    }
+    unit_reduce_add(sum, lane, S.uacc[u - u0]);
+  }
+}
+
+// ANY = false: grid objects only (the mesh lookup is compiled out).  FLAT: contacts where the
+// SDF's gradient is zero may occur.
+template <int MODE, int NW, int MINB, int PPT, bool ANY, bool FLAT>
 __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) {
   __shared__ FusedSmem<NW> S;
   extern __shared__ int face_cache[];            // [face_cap], mesh objects
@@ -534,6 +603,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
       if (warp == 0) fk_warp(H, S.q, S.frame4, lane);
       for (int idx = tid; idx < kSims * 8; idx += NW * 32) (&S.wfix[0][0])[idx] = 0ull;
       if (tid == 0) S.next_chunk = 0;
+      if (FLAT && tid == 0) S.flat = 0;
       __syncthreads();
       const ObjDev& O = S.O;
 
@@ -628,7 +698,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
           }
           PointState ps;
           point_state(smp, p, r, ps);
-          chunk_forces(ps, S.K, valid, dtV, Pm.w_pen, lane, S.wfix, [&](int m, unsigned bal) {
+          chunk_forces<FLAT>(ps, S.K, valid, dtV, Pm.w_pen, lane, S.wfix, &S.flat, [&](int m, unsigned bal) {
             if (MODE == kModeWrench && lane == 0 && a.bits)
               a.bits[((size_t)c * kSims + m) * nwords + (base >> 5)] = bal;
           });
@@ -636,6 +706,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
         }
       }
       __syncthreads();
+      if (FLAT && S.flat) {
+        flat_forces(S, r, dtV, lane, warp);
+        __syncthreads();
+      }
 
       // ------------------------------------------------------------ reduction
       if (warp == 0) {
@@ -719,6 +793,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
         else
           adjoint_sweep<NW, PPT, ANY, false>(S, O, r, faces, u0, u1, lane);
         __syncthreads();
+        if (FLAT && S.flat) {
+          flat_adjoint(S, r, dtV, u0, u1, lane, warp);
+          __syncthreads();
+        }
         // per-link sums, one thread per link and component
         for (int idx = tid; idx < L * 6; idx += NW * 32) {
           const int l = idx / 6, k = idx - 6 * l;
@@ -799,9 +877,9 @@ constexpr int kMaxCachedFaces = 32 * kMaxCullChunks;
 
 // Launch of one compiled configuration: a persistent grid of (SMs x resident
 // CTAs) blocks, capped at B.
-template <int MODE, int NW, int MINB, int PPT, bool ANY = false>
+template <int MODE, int NW, int MINB, int PPT, bool ANY = false, bool FLAT = false>
 cudaError_t launch_fused_cfg(const FusedArgs& a, cudaStream_t st) {
-  auto kernel = fused_step_kernel<MODE, NW, MINB, PPT, ANY>;
+  auto kernel = fused_step_kernel<MODE, NW, MINB, PPT, ANY, FLAT>;
   FusedArgs b = a;
   b.face_cap = 0;
   if (ANY && a.any_mesh && MODE != kModeWrench) b.face_cap = a.hand_P < kMaxCachedFaces ? a.hand_P : kMaxCachedFaces;

@@ -23,13 +23,14 @@ struct fg_sdf {
   float* grid;
   float* pyr;
   size_t bytes;              // grid bytes
-  size_t pyr_bytes;          // min-pyramid bytes
+  size_t pyr_bytes;          // min-pyramid and flat_min, bytes
   float4* mesh;              // mesh objects: BVH, triangles and normals (one allocation); bytes is its size
 };
 
 struct fg_scene {
   int n;
   int has_mesh;              // some object is a mesh
+  float flat_min;            // smallest ObjDev::flat_min of its objects
   fg::ObjDev* dev;           // device [n]
 };
 
@@ -47,7 +48,9 @@ bool alloc_fault();
 ParamsDev params_from(const fg_params* p);
 int device_sm_count();
 size_t min_pyramid_floats(int nx, int ny, int nz, int* levels);
-cudaError_t build_min_pyramid(const float* grid, int nx, int ny, int nz, float* pyr, int levels, int* offsets);
+// pyr holds one float more than min_pyramid_floats; *flat_min: the smallest value of a cell of equal corners.
+cudaError_t build_min_pyramid(const float* grid, int nx, int ny, int nz, float* pyr, int levels, int* offsets,
+                              float* flat_min);
 
 // fused kernels (fg_fused.cu)
 enum FusedMode { kModeWrench = 0, kModeLossGrad = 1, kModeOptimize = 2, kModeQueue = 3 };
@@ -83,6 +86,8 @@ struct FusedArgs {
   const QueueSlotDev* slots;   // queue mode: slot table (device), sorted by cand_start
   int nslots;
   int any_mesh;                // some object is a mesh: the kernels with the mesh lookup
+  int any_flat;                // some grid has cells of gradient zero that can be in contact (flat_min < r): the kernels with
+                               // the friction of such contacts
   unsigned* work;              // fused kernels: candidate counter pair (set by the launcher)
 };
 typedef cudaError_t (*FusedLaunchFn)(const FusedArgs&, cudaStream_t);
@@ -90,6 +95,7 @@ typedef cudaError_t (*FusedLaunchFn)(const FusedArgs&, cudaStream_t);
 extern const FusedLaunchFn kOptimizeLaunch[];
 extern const FusedLaunchFn kOptimizeLaunchAny[];
 extern const FusedLaunchFn kLossGradLaunchAny[];
+cudaError_t launch_fused_flat(int mode, const FusedArgs& a, cudaStream_t st);
 cudaError_t launch_wrench_any(const FusedArgs& a, cudaStream_t st);
 cudaError_t launch_queue_round_any(const FusedArgs& a, cudaStream_t st);
 cudaError_t launch_fused(int mode, const FusedArgs& a, const fg_hand* h, cudaStream_t st);

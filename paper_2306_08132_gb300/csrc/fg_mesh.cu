@@ -546,6 +546,7 @@ extern "C" fg_status fg_sdf_create_mesh(const float* vertices, int nv, const int
   o.inv_inertia = 1.0f / inertia;
   o.h = 1.0f;          // unused by mesh queries
   o.inv_h = 1.0f;
+  o.flat_min = 3.0e38f;
   *out = s;
   return FG_OK;
 }

@@ -179,6 +179,7 @@ void scheduler(fg_queue* Q) {
     a.nslots = n;
     for (int i = 0; i < n; ++i) {
       a.any_mesh |= Q->h_slots[i].obj.kind == fg::kObjMesh;
+      a.any_flat |= Q->h_slots[i].obj.flat_min < Q->h_slots[i].P.r0;
       a.hand_P = std::max(a.hand_P, Q->active[i]->hand->host.P);
     }
     if (e == cudaSuccess) e = fg::launch_queue_round(a, Q->stream);

@@ -5,8 +5,12 @@
 // Level k (k >= 1) has one entry per block of 2^k x 2^k x 2^k cells: the minimum
 // of the grid nodes of those cells.  The trilinear interpolant inside a cell is
 // a convex combination of the cell's corners, so it never drops below the
-// minimum of any block that contains the cell.
+// minimum of any block that contains the cell.  The pass over the grid that makes level 1 also
+// finds the smallest value of a cell whose 8 corners are equal, where the gradient
+// is zero.
 #include <cuda_runtime.h>
+
+#include <cstring>
 
 #include "fg_internal.h"
 
@@ -14,17 +18,44 @@ namespace fg {
 
 namespace {
 
+// Floats as integers of the same order (no NaN).
+__device__ __forceinline__ int ordered(float x) {
+  const int i = __float_as_int(x);
+  return i >= 0 ? i : i ^ 0x7fffffff;
+}
+
+// *flat: the smallest value of a cell of equal corners, as an ordered integer.
 __global__ void pyr_level1_kernel(const float* __restrict__ G, int nx, int ny, int nz, float* __restrict__ out,
-                                  int bx, int by, int bz) {
+                                  int bx, int by, int bz, int* __restrict__ flat) {
   const size_t total = (size_t)bx * by * bz;
+  int lowest = ordered(3.0e38f);
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
     const int I = (int)(t % bx), J = (int)((t / bx) % by), K = (int)(t / ((size_t)bx * by));
-    float m = 3.0e38f;
-    for (int z = 2 * K; z <= min(2 * K + 2, nz - 1); ++z)
-      for (int y = 2 * J; y <= min(2 * J + 2, ny - 1); ++y)
-        for (int x = 2 * I; x <= min(2 * I + 2, nx - 1); ++x) m = fminf(m, G[((size_t)z * ny + y) * nx + x]);
+    float m = 3.0e38f, v[3][3][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int x = min(2 * I + a, nx - 1), y = min(2 * J + b, ny - 1), z = min(2 * K + c, nz - 1);
+          v[c][b][a] = G[((size_t)z * ny + y) * nx + x];
+          m = fminf(m, v[c][b][a]);
+        }
     out[t] = m;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int a = e & 1, b = (e >> 1) & 1, c = e >> 2;
+      if (2 * I + a > nx - 2 || 2 * J + b > ny - 2 || 2 * K + c > nz - 2) continue;      // no such cell
+      const float v0 = v[c][b][a];
+      bool same = true;
+#pragma unroll
+      for (int k = 1; k < 8; ++k) same = same && v[c + (k >> 2)][b + ((k >> 1) & 1)][a + (k & 1)] == v0;
+      if (same) lowest = min(lowest, ordered(v0));
+    }
   }
+  lowest = __reduce_min_sync(0xffffffffu, lowest);
+  if ((threadIdx.x & 31) == 0 && lowest < *flat) atomicMin(flat, lowest);
 }
 
 __global__ void pyr_level_kernel(const float* __restrict__ in, int ix, int iy, int iz, float* __restrict__ out,
@@ -55,7 +86,13 @@ size_t min_pyramid_floats(int nx, int ny, int nz, int* levels) {
   return total;
 }
 
-cudaError_t build_min_pyramid(const float* grid, int nx, int ny, int nz, float* pyr, int levels, int* offsets) {
+cudaError_t build_min_pyramid(const float* grid, int nx, int ny, int nz, float* pyr, int levels, int* offsets,
+                              float* flat_min) {
+  int unused = 0;
+  int* flat = reinterpret_cast<int*>(pyr + min_pyramid_floats(nx, ny, nz, &unused));
+  const float none = 3.0e38f;                                    // its own ordered integer
+  cudaError_t e0 = cudaMemcpy(flat, &none, sizeof(float), cudaMemcpyHostToDevice);
+  if (e0 != cudaSuccess) return e0;
   size_t off = 0;
   const float* prev = nullptr;
   int px = 0, py = 0, pz = 0;
@@ -67,7 +104,7 @@ cudaError_t build_min_pyramid(const float* grid, int nx, int ny, int nz, float* 
     const size_t cap = (size_t)device_sm_count() * 16;
     if (blocks > cap) blocks = cap;
     if (k == 1)
-      pyr_level1_kernel<<<(int)blocks, 256>>>(grid, nx, ny, nz, pyr + off, bx, by, bz);
+      pyr_level1_kernel<<<(int)blocks, 256>>>(grid, nx, ny, nz, pyr + off, bx, by, bz, flat);
     else
       pyr_level_kernel<<<(int)blocks, 256>>>(prev, px, py, pz, pyr + off, bx, by, bz);
     cudaError_t e = cudaGetLastError();
@@ -78,7 +115,11 @@ cudaError_t build_min_pyramid(const float* grid, int nx, int ny, int nz, float* 
     pz = bz;
     off += total;
   }
-  return cudaDeviceSynchronize();
+  int low = 0;
+  const cudaError_t e = cudaMemcpy(&low, flat, sizeof(int), cudaMemcpyDeviceToHost);      // waits for the levels
+  if (low < 0) low ^= 0x7fffffff;
+  std::memcpy(flat_min, &low, sizeof(float));
+  return e;
 }
 
 }  // namespace fg

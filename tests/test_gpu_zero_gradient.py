@@ -88,3 +88,79 @@ def test_zero_gradient_contacts_gauss_seidel(fg, case, mu):
     _check(loss, grad, ref, idx)
     W, N, _ = fg.contact_wrench(case.hand, case.scene, case.q, params, R)
     _check_wrench(W, N, ref, idx)
+
+
+@pytest.mark.parametrize("mu", [0.5, 0.05])
+def test_zero_gradient_contacts_averaged(fg, case, mu):
+    params = dict(case.w.params, mu=mu)
+    ref, idx = case.reference(params)
+    try:
+        for i in [-1] + list(range(len(fg.fused_configs()))):
+            fg.fused_config_select(i)
+            _check(*fg.loss_and_grad(case.hand, case.scene, case.q, params, R), ref, idx)
+    finally:
+        fg.fused_config_select(-1)
+    W, N, _ = fg.contact_wrench(case.hand, case.scene, case.q, params, R)
+    _check_wrench(W, N, ref, idx)
+
+
+@pytest.mark.parametrize("mu", [0.5, 0.05])
+def test_zero_gradient_contacts_per_stage(fg, case, mu):
+    params = dict(case.w.params, mu=mu, r0=R)
+    ref, idx = case.reference(params)
+    q = case.q.clone()
+    loss = fg.optimize_step_plain(case.hand, case.scene, q, params, 0, 10, 1)
+    _check(loss, (case.q - q) / params["lr"], ref, idx)
+
+
+def test_zero_gradient_contacts_in_the_queue_and_in_mixed_scenes(fg, case):
+    """The request queue steps such an object as fg_optimize_step does, and another object's candidates keep their
+    results, bit for bit, in a scene and in a round with it."""
+    params = dict(case.w.params, r0=R)
+    flat, plain = fg.Sdf.from_synth(case.obj), fg.Sdf.from_synth(case.w.objects[0])
+    expected = []
+    for sdf in (flat, plain):
+        q = case.q.clone()
+        loss = fg.optimize_step(case.hand, fg.Scene([sdf]), q, params, 0, 3, 1)
+        expected.append((q.cpu().numpy(), loss.cpu().numpy()))
+    q = torch.cat([case.q, case.q])
+    oc = torch.arange(2, device=q.device, dtype=torch.int32).repeat_interleave(len(case.q))
+    loss = fg.optimize_step(case.hand, fg.Scene([flat, plain]), q, params, 0, 3, 1, obj_of_cand=oc)
+    np.testing.assert_array_equal(q.cpu().numpy(), np.concatenate([expected[0][0], expected[1][0]]))
+    np.testing.assert_array_equal(loss.cpu().numpy(), np.concatenate([expected[0][1], expected[1][1]]))
+    queue = fg.Queue(1 << 30)
+    try:
+        ids = [queue.submit(case.hand, s, case.w.q0, 1, params) for s in (flat, plain)]
+        for rid, (qe, le) in zip(ids, expected):
+            queue.wait(rid, 120000)
+            qg, lg, _ = queue.result(rid)
+            np.testing.assert_array_equal(qg, qe)
+            np.testing.assert_array_equal(lg, le)
+    finally:
+        queue.close()
+
+
+def test_zero_gradient_cell_anywhere_in_the_grid(fg):
+    """One constant cell at each place of small odd and even grids, a hand of one point in it."""
+    hand_d = {"parent": np.array([-1]), "T_fix": np.eye(3, 4)[None], "axis": np.zeros((1, 3)), "q_low": np.zeros(0),
+              "q_up": np.zeros(0), "pts_local": np.array([[0.003, -0.002, 0.001]]), "link_of_point": np.array([0])}
+    hand = fg.Hand.from_synth(hand_d)
+    params = synth.tiny_sphere_workload(n_cand=1).params
+    rng = np.random.default_rng(4)
+    pitch = 0.02
+    for dims in ((4, 3, 5), (2, 5, 4)):                                    # nodes along z, y, x
+        cells = [(k, j, i) for k in range(dims[0] - 1) for j in range(dims[1] - 1) for i in range(dims[2] - 1)]
+        objs, q = [], np.zeros((len(cells), 6), dtype=np.float32)
+        for n, (k, j, i) in enumerate(cells):
+            g = rng.uniform(-0.02, 0.02, size=dims).astype(np.float32)
+            g[k:k + 2, j:j + 2, i:i + 2] = 0.0
+            objs.append({"kind": "cell", "grid": torch.tensor(g), "origin": np.array([-0.03, -0.02, -0.04], dtype=np.float32),
+                         "pitch": float(np.float32(pitch)), "mass": 0.7, "inertia": 4e-4, "bound_radius": 0.05, "params": {}})
+            q[n, :3] = objs[-1]["origin"] + pitch * (np.array([i, j, k]) + rng.uniform(0.3, 0.7, 3)) - hand_d["pts_local"][0]
+        oc = np.arange(len(cells), dtype=np.int32)
+        S = O.Setup(dict(hand_d, L=1, J=0, D=6, P=1), objs, params)
+        ref = O.batch_loss_and_grad(S, q, oc, R)
+        assert (ref["N"] == 1).all()
+        loss, grad = fg.loss_and_grad(hand, fg.Scene([fg.Sdf.from_synth(o) for o in objs]), torch.tensor(q, device="cuda:0"),
+                                      params, R, obj_of_cand=torch.tensor(oc, device="cuda:0"))
+        _check(loss, grad, ref, oc)
