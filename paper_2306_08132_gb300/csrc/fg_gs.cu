@@ -131,13 +131,15 @@ __device__ __forceinline__ float gs_tangent(const float n[3], const float D[3], 
 // What a point keeps while the state changes: un = d x n, 1/w_n, s_d = d . n and
 // w_t's constant part.  With t normal to n, |d x t|^2 = s_d^2 + (un . t)^2.  Where the
 // gradient is zero, n = 0 and all of D is tangential, so |d x t|^2 is formed from the
-// vectors, behind a branch that the warp takes only when some lane has such a point.
+// vectors, in the FLAT kernels alone, behind a branch that the warp takes only when some lane has
+// such a point (in all kernels it cost 8 objects x 256 candidates 1.3%).
 struct GsPoint {
   float d[3], un[3], rwn, wt0;
   bool some_flat;
 };
 __device__ __forceinline__ bool flat_normal(const float n[3]) { return n[0] == 0.0f && n[1] == 0.0f && n[2] == 0.0f; }
 // Every lane of the warp must call it.
+template <bool FLAT>
 __device__ __forceinline__ void gs_point(const PointState& ps, const float xt[3], const ObjDev& O, GsPoint& g) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) g.d[k] = sub_(ps.p[k], xt[k]);
@@ -145,7 +147,7 @@ __device__ __forceinline__ void gs_point(const PointState& ps, const float xt[3]
   g.rwn = rcp_fast(fma_(O.inv_inertia, dot3(g.un, g.un), O.inv_mass));
   const float sd = dot3(g.d, ps.n);
   g.wt0 = fma_(O.inv_inertia, mul_(sd, sd), O.inv_mass);
-  g.some_flat = __any_sync(kFull, flat_normal(ps.n));
+  g.some_flat = FLAT && __any_sync(kFull, flat_normal(ps.n));
 }
 
 // Correction of one projected point (phi < 0): force f = -(lambda_n n + lambda_t t) with
@@ -154,6 +156,7 @@ __device__ __forceinline__ void gs_point(const PointState& ps, const float xt[3]
 // computes its own from the common state (a branch for the projected lane and the terms
 // that do not depend on the state would lengthen the chain of projections).  With the
 // reverse's chain cut to gs_passage, 8 objects x 256 candidates: 0.98 -> 0.80 ms.
+template <bool FLAT>
 __device__ __forceinline__ void gs_force(const PointState& ps, const GsPoint& g, const float D[3], float phi,
                                          const ParamsDev& P, const ObjDev& O, float f[3], float tq[3]) {
   const float lam = mul_(-phi, g.rwn), sn = dot3(ps.n, D);
@@ -164,7 +167,7 @@ __device__ __forceinline__ void gs_force(const PointState& ps, const GsPoint& g,
   const float bound = fminf(mul_(s2, rs), mul_(P.mu, -phi));
   cross3(g.d, s, ds);
   float ut2 = mul_(us, us);
-  if (g.some_flat && flat_normal(ps.n)) ut2 = mul_(dot3(ds, ds), mul_(rs, rs));
+  if (FLAT && g.some_flat && flat_normal(ps.n)) ut2 = mul_(dot3(ds, ds), mul_(rs, rs));
   const float kt = mul_(mul_(bound, rs), rcp_fast(fma_(O.inv_inertia, ut2, g.wt0)));   // lambda_t / |s|
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -392,6 +395,7 @@ __device__ __forceinline__ void gs_contact_adjoint(const PointState& ps, const f
 struct GsPassage {
   float t[3], mr, k1, kt, k2;      // mr = [kinetic] mu/w_t, kt = [kinetic] k1 - k2 us
 };
+template <bool FLAT>
 __device__ __forceinline__ void gs_passage(const PointState& ps, GsPoint& g, const float xt[3],
                                            const float st[6], const ParamsDev& P, const ObjDev& O, GsPassage& q) {
   float d[3], D[3];
@@ -401,7 +405,7 @@ __device__ __forceinline__ void gs_passage(const PointState& ps, GsPoint& g, con
   for (int k = 0; k < 3; ++k) s[k] = fma_(-sn, ps.n[k], D[k]);
   const float s2 = dot3(s, s), rs = rsqrt_or_zero(s2), sig = s2 * rs;
   float us = dot3(g.un, s) * rs, ut2 = us * us, sgn = 1.0f;
-  if (g.some_flat && flat_normal(ps.n)) {
+  if (FLAT && g.some_flat && flat_normal(ps.n)) {
     float ds[3];
     cross3(g.d, s, ds);
     ut2 = dot3(ds, ds) * (rs * rs);
@@ -426,20 +430,21 @@ __device__ __forceinline__ void gs_passage(const PointState& ps, GsPoint& g, con
 // (smine) and the adjoint after it (amine), computes the general adjoint of the
 // projected lanes (into dphi, dn, dp) and returns in a the adjoint at the
 // chunk's start.
+template <bool FLAT>
 __device__ __forceinline__ void gs_chunk_reverse(const PointState& ps, const float xt[3], const float st0[6],
                                                  float a[6], unsigned mask, int m, int lane, const ParamsDev& P,
                                                  const ObjDev& O, float smine[6], float amine[6], float& dphi,
                                                  float dn[3], float dp[3]) {
   float st[6];
   GsPoint g;
-  gs_point(ps, xt, O, g);
+  gs_point<FLAT>(ps, xt, O, g);
 #pragma unroll
   for (int k = 0; k < 6; ++k) st[k] = smine[k] = st0[k];
   for (unsigned rest = mask; rest; rest &= rest - 1u) {   // forward re-run, lanes in order
     const int j = __ffs(rest) - 1;
     float d[3], D[3], f[3], tq[3];
     const float phi = gs_phi(ps, xt, st, d, D);
-    gs_force(ps, g, D, phi, P, O, f, tq);
+    gs_force<FLAT>(ps, g, D, phi, P, O, f, tq);
     gs_apply(st, f, tq, O, j);
     if (lane > j) {
 #pragma unroll
@@ -447,7 +452,7 @@ __device__ __forceinline__ void gs_chunk_reverse(const PointState& ps, const flo
     }
   }
   GsPassage q;
-  gs_passage(ps, g, xt, smine, P, O, q);
+  gs_passage<FLAT>(ps, g, xt, smine, P, O, q);
   const float extra = m == 0 ? P.w_pen : 0.0f;
   int hi = 32;
   for (unsigned rest = mask; rest;) {                     // events in reverse
@@ -491,7 +496,8 @@ __device__ __forceinline__ void gs_lookup(const ObjDev& O, const float p[3], con
 }
 
 // ANY = false: grid objects only; true: grids and meshes (the lookup dispatches on the kind).
-template <int MODE, bool ANY>
+// FLAT: contacts where the SDF's gradient is zero may occur.
+template <int MODE, bool ANY, bool FLAT>
 __global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_kernel(FusedArgs a) {
   constexpr int GW = ANY ? kGWMesh : kGW;
   __shared__ GsSmem<GW> S;
@@ -685,7 +691,7 @@ __global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_ke
             PointState ps;
             point_state(smp, p, r, ps);
             GsPoint g;
-            gs_point(ps, xt, O, g);
+            gs_point<FLAT>(ps, xt, O, g);
             int last = -1;
             for (;;) {
               float d[3], Dd[3];
@@ -694,7 +700,7 @@ __global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_ke
               if (!cand) break;
               const int jl = __ffs(cand) - 1;
               float f[3], tq[3];
-              gs_force(ps, g, Dd, phi, Pm, O, f, tq);
+              gs_force<FLAT>(ps, g, Dd, phi, Pm, O, f, tq);
               if (lane == jl) {
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
@@ -852,7 +858,7 @@ __global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_ke
             float st0[6], smine[6], amine[6], dphi = 0.0f, dn[3] = {0.0f, 0.0f, 0.0f}, dp[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
             for (int k = 0; k < 6; ++k) st0[k] = sn[k];
-            gs_chunk_reverse(ps, xt, st0, av, mask, m, lane, Pm, O, smine, amine, dphi, dn, dp);
+            gs_chunk_reverse<FLAT>(ps, xt, st0, av, mask, m, lane, Pm, O, smine, amine, dphi, dn, dp);
             if (!((mask >> lane) & 1u)) gs_leaky(ps, xt, smine, amine, m == 0 ? Pm.w_pen : 0.0f, Pm, O, dphi, dn, dp);
             sdf_adjoint<ANY>(smp, ps, dphi, dn, dp);
             float v[6];
@@ -1013,7 +1019,7 @@ __global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_ke
   work_done(a.work);
 }
 
-template <int MODE, bool ANY>
+template <int MODE, bool ANY, bool FLAT = false>
 cudaError_t launch_gs_mode(const FusedArgs& a, int nchunks, cudaStream_t st) {
   constexpr int GW = ANY ? kGWMesh : kGW;
   FusedArgs b = a;
@@ -1023,12 +1029,12 @@ cudaError_t launch_gs_mode(const FusedArgs& a, int nchunks, cudaStream_t st) {
   int dev = 0;
   cudaGetDevice(&dev);
   if (dyn > attr_set[dev & 63]) {
-    cudaError_t e = cudaFuncSetAttribute(gs_kernel<MODE, ANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    cudaError_t e = cudaFuncSetAttribute(gs_kernel<MODE, ANY, FLAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     if (e != cudaSuccess) return e;
     attr_set[dev & 63] = dyn;
   }
   int bps = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, gs_kernel<MODE, ANY>, GW * 32, dyn);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, gs_kernel<MODE, ANY, FLAT>, GW * 32, dyn);
   if (e != cudaSuccess) return e;
   if (bps < 1) bps = 1;
   long long grid = (long long)device_sm_count() * bps;
@@ -1036,7 +1042,7 @@ cudaError_t launch_gs_mode(const FusedArgs& a, int nchunks, cudaStream_t st) {
   if (grid < 1) return cudaSuccess;
   e = work_pair(&b.work, st);
   if (e != cudaSuccess) return e;
-  gs_kernel<MODE, ANY><<<(int)grid, GW * 32, dyn, st>>>(b);
+  gs_kernel<MODE, ANY, FLAT><<<(int)grid, GW * 32, dyn, st>>>(b);
   return cudaGetLastError();
 }
 
@@ -1045,6 +1051,11 @@ cudaError_t launch_gs_mode(const FusedArgs& a, int nchunks, cudaStream_t st) {
 cudaError_t launch_gs(int mode, const FusedArgs& a, int nchunks, cudaStream_t st) {
   if (a.B <= 0) return cudaSuccess;
   if (nchunks < 1 || nchunks > kMaxCullChunks) return cudaErrorInvalidValue;
+  if (a.any_flat) {
+    if (mode == kModeWrench) return launch_gs_mode<kModeWrench, true, true>(a, nchunks, st);
+    return mode == kModeLossGrad ? launch_gs_mode<kModeLossGrad, true, true>(a, nchunks, st)
+                                 : launch_gs_mode<kModeOptimize, true, true>(a, nchunks, st);
+  }
   if (a.any_mesh) {
     if (mode == kModeWrench) return launch_gs_mode<kModeWrench, true>(a, nchunks, st);
     return mode == kModeLossGrad ? launch_gs_mode<kModeLossGrad, true>(a, nchunks, st)

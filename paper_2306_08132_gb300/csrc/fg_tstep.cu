@@ -344,11 +344,12 @@ __device__ __forceinline__ void rotate_from(int k, const float o[3], float v[3])
 // velocity's axis first; s its sign, 0 at rest): U = d x n, s_d = d . n and the inverse
 // masses, |d x t|^2 = s_d^2 + (U_0/rho)^2 (t normal to n).  Where the gradient is zero
 // (flat: n = 0) the whole displacement is tangential: t = s e_0, rho = 1,
-// |d x t|^2 = d_1^2 + d_2^2.
+// |d x t|^2 = d_1^2 + d_2^2 (FLAT kernels; in all kernels it cost 8 x 512 candidates 0.7%).
 struct FirstContact {
   float U[3], sd, rho2, rr, rwn, rwt;
   bool flat;
 };
+template <bool FLAT>
 __device__ __forceinline__ void first_contact(const float d[3], const float n[3], const ObjDev& O, FirstContact& q) {
   cross3(d, n, q.U);
   q.sd = dot3(d, n);
@@ -356,7 +357,7 @@ __device__ __forceinline__ void first_contact(const float d[3], const float n[3]
   q.rr = rsqrt_bounded(q.rho2);
   const float Ur = q.U[0] * q.rr;
   float ut2 = fmaf(Ur, Ur, q.sd * q.sd);
-  q.flat = q.rho2 == 0.0f && n[0] == 0.0f;
+  q.flat = FLAT && q.rho2 == 0.0f && n[0] == 0.0f;
   if (q.flat) {
     q.rho2 = q.rr = 1.0f;
     ut2 = d[1] * d[1] + d[2] * d[2];
@@ -366,10 +367,11 @@ __device__ __forceinline__ void first_contact(const float d[3], const float n[3]
 }
 // Its force f = A n + B e_0 and torque A U + B d x e_0, with lambda_t = min(c rho, mu C)/w_t,
 // B = -s lambda_t/rho, A = -C/w_n - B n_0.
+template <bool FLAT>
 __device__ __forceinline__ void first_force(const float d[3], const float n[3], float s, float c, float C, float mu,
                                             const ObjDev& O, float f[3], float tq[3]) {
   FirstContact q;
-  first_contact(d, n, O, q);
+  first_contact<FLAT>(d, n, O, q);
   const float B = -s * fminf(c * (q.rho2 * q.rr), mu * C) * q.rwt * q.rr, A = -fmaf(C, q.rwn, B * n[0]);
   f[0] = fmaf(A, n[0], B);
   f[1] = A * n[1];
@@ -381,11 +383,12 @@ __device__ __forceinline__ void first_force(const float d[3], const float n[3], 
 // Its adjoint (the terms of point_contacts_adjoint without the plane's): dL/dphi_hat,
 // dL/dn (up to a multiple of n) and dL/dd, for the wrench adjoint (gl, ga).  8 x 512
 // candidates at T = 1: 1.37 -> 1.32 ms against the chain through d x n, t and d x t.
+template <bool FLAT>
 __device__ __forceinline__ void first_contact_adjoint(const float d[3], const float n[3], float s, float c, float C,
                                                       float mu, const float gl[3], const float ga[3], float extra_dC,
                                                       const ObjDev& O, float& dphi, float dn[3], float dd[3]) {
   FirstContact q;
-  first_contact(d, n, O, q);
+  first_contact<FLAT>(d, n, O, q);
   float gf[3];
   cross3(ga, d, gf);
 #pragma unroll
@@ -413,7 +416,7 @@ __device__ __forceinline__ void first_contact_adjoint(const float d[3], const fl
 
 // Forward of one 32-point chunk in every simulation: the contacts' wrenches and counts
 // are added to the warp's sums (red[m]) in a fixed order.
-template <bool ANY>
+template <bool ANY, bool FLAT>
 __device__ __forceinline__ void first_forward_chunk(const ObjDev& O, const ParamsDev& Pm, const float p[3], bool valid,
                                                     float rdil, float c, int lane, float (*red)[12]) {
 #pragma unroll 1
@@ -438,7 +441,7 @@ __device__ __forceinline__ void first_forward_chunk(const ObjDev& O, const Param
       float d[3], n[3], f[3], tq[3];
       rotate_to(k, r, d);
       rotate_to(k, ps.n, n);
-      first_force(d, n, m > 0 ? sim_sign(m) : 0.0f, c, -ps.phi_hat, Pm.mu, O, f, tq);
+      first_force<FLAT>(d, n, m > 0 ? sim_sign(m) : 0.0f, c, -ps.phi_hat, Pm.mu, O, f, tq);
       rotate_from(k, f, v);
       rotate_from(k, tq, v + 3);
     }
@@ -459,7 +462,7 @@ __device__ __forceinline__ void first_forward_chunk(const ObjDev& O, const Param
 // a moved query replaces one plane of 4 where it has left the cell, 8 + 6 x 4 predicated loads
 // a point instead of 56.  Same batch: 1.86 -> 1.54 ms, L1 data pipe 72% -> 49%; the four warps a
 // scheduler that 128 registers leave no longer cover the latencies.
-template <bool ANY, bool NEAR>
+template <bool ANY, bool NEAR, bool FLAT>
 __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const ParamsDev& Pm, const float (*G)[6],
                                                     const float p[3], bool valid, float rdil, float c, float pb[3]) {
   pb[0] = pb[1] = pb[2] = 0.0f;
@@ -558,7 +561,7 @@ __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const Param
       rotate_to(k, ps.n, n);
       rotate_to(k, G[m], gl);
       rotate_to(k, G[m] + 3, ga);
-      first_contact_adjoint(d, n, m > 0 ? sim_sign(m) : 0.0f, c, -ps.phi_hat, Pm.mu, gl, ga, m == 0 ? Pm.w_pen : 0.0f,
+      first_contact_adjoint<FLAT>(d, n, m > 0 ? sim_sign(m) : 0.0f, c, -ps.phi_hat, Pm.mu, gl, ga, m == 0 ? Pm.w_pen : 0.0f,
                             O, dphi, dnr, ddr);
       rotate_from(k, dnr, dn);
       rotate_from(k, ddr, dd);
@@ -591,7 +594,7 @@ __device__ __forceinline__ void point_wrench(const float p[3], const float t0[3]
 // The first step's reverse sweep: per-link sums of (g, (p - t0) x g), by work units
 // claimed from a counter (as in the one-step kernel), or by fixed ranges of points for
 // hands with more units than uacc holds.
-template <bool ANY, bool NEAR, int TW>
+template <bool ANY, bool NEAR, int TW, bool FLAT>
 __device__ __forceinline__ void first_reverse_sweep(TstepSmem& S, const ObjDev& O, float rdil, int lane, int warp) {
   const HandDev& H = S.H;
   const float c = mul_(S.Pm.dt, S.Pm.V);
@@ -610,7 +613,7 @@ __device__ __forceinline__ void first_reverse_sweep(TstepSmem& S, const ObjDev& 
         const float4 sp = __ldg(H.pts + (valid ? U.x + h + lane : U.x));
         float p[3], pb[3], v[6];
         world_point(S.frame4[U.z], sp, p);
-        first_reverse_point<ANY, NEAR>(O, S.Pm, S.G, p, valid, rdil, c, pb);
+        first_reverse_point<ANY, NEAR, FLAT>(O, S.Pm, S.G, p, valid, rdil, c, pb);
         point_wrench(p, t0, pb, valid, v);
 #pragma unroll
         for (int k = 0; k < 6; ++k) sum[k] += v[k];
@@ -629,7 +632,7 @@ __device__ __forceinline__ void first_reverse_sweep(TstepSmem& S, const ObjDev& 
         const int link = (int)sp.w;
         float p[3], pb[3], v[6];
         world_point(S.frame4[link], sp, p);
-        first_reverse_point<ANY, NEAR>(O, S.Pm, S.G, p, valid, rdil, c, pb);
+        first_reverse_point<ANY, NEAR, FLAT>(O, S.Pm, S.G, p, valid, rdil, c, pb);
         point_wrench(p, t0, pb, valid, v);
         link_accumulate(S.lacc[slot], lane, link, valid, v, cur, acc);
       }
@@ -640,7 +643,8 @@ __device__ __forceinline__ void first_reverse_sweep(TstepSmem& S, const ObjDev& 
 }
 
 // ANY = false: grid objects only; true: grids and meshes (the lookup dispatches on the kind).
-template <int MODE, bool ANY, int TW>
+// FLAT: contacts where the SDF's gradient is zero may occur.
+template <int MODE, bool ANY, int TW, bool FLAT>
 __global__ void __launch_bounds__(TW * 32, 16 / TW) tstep_kernel(FusedArgs a) {
   __shared__ TstepSmem S;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -743,7 +747,7 @@ __global__ void __launch_bounds__(TW * 32, 16 / TW) tstep_kernel(FusedArgs a) {
               const float4 sp = __ldg(H.pts + (valid ? i : 32 * j));
               float p[3];
               world_point(S.frame4[(int)sp.w], sp, p);
-              first_forward_chunk<ANY>(O, Pm, p, valid, rdil, c, lane, S.red[slot]);
+              first_forward_chunk<ANY, FLAT>(O, Pm, p, valid, rdil, c, lane, S.red[slot]);
             }
         } else {
         if (cull) {
@@ -906,9 +910,9 @@ __global__ void __launch_bounds__(TW * 32, 16 / TW) tstep_kernel(FusedArgs a) {
         __syncthreads();
         if (t == 0) {               // the adjoint of the initial state is not needed
           if (near_queries(O, mul_(dt, Pm.V)))
-            first_reverse_sweep<ANY, true, TW>(S, O, rdil, lane, warp);
+            first_reverse_sweep<ANY, true, TW, FLAT>(S, O, rdil, lane, warp);
           else
-            first_reverse_sweep<ANY, false, TW>(S, O, rdil, lane, warp);
+            first_reverse_sweep<ANY, false, TW, FLAT>(S, O, rdil, lane, warp);
           __syncthreads();
           break;
         }
@@ -1154,14 +1158,14 @@ __global__ void __launch_bounds__(TW * 32, 16 / TW) tstep_kernel(FusedArgs a) {
   work_done(a.work);
 }
 
-template <int MODE, bool ANY, int TW>
+template <int MODE, bool ANY, int TW, bool FLAT = false>
 cudaError_t launch_tstep_mode(const FusedArgs& a, cudaStream_t st) {
   static int blocks_per_sm[64] = {0};
   int dev = 0;
   cudaGetDevice(&dev);
   int& bps = blocks_per_sm[dev & 63];
   if (bps <= 0) {
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, tstep_kernel<MODE, ANY, TW>, TW * 32, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, tstep_kernel<MODE, ANY, TW, FLAT>, TW * 32, 0);
     if (e != cudaSuccess) return e;
     if (bps < 1) bps = 1;
   }
@@ -1171,7 +1175,7 @@ cudaError_t launch_tstep_mode(const FusedArgs& a, cudaStream_t st) {
   FusedArgs b = a;
   cudaError_t e = work_pair(&b.work, st);
   if (e != cudaSuccess) return e;
-  tstep_kernel<MODE, ANY, TW><<<(int)grid, TW * 32, 0, st>>>(b);
+  tstep_kernel<MODE, ANY, TW, FLAT><<<(int)grid, TW * 32, 0, st>>>(b);
   return cudaGetLastError();
 }
 
@@ -1189,6 +1193,9 @@ cudaError_t launch_tstep_warps(int mode, const FusedArgs& a, cudaStream_t st) {
 cudaError_t launch_tstep(int mode, const FusedArgs& a, cudaStream_t st) {
   if (a.B <= 0) return cudaSuccess;
   if (a.P.sim_steps < 1 || a.P.sim_steps > kTSteps) return cudaErrorInvalidValue;
+  if (a.any_flat)
+    return mode == kModeLossGrad ? launch_tstep_mode<kModeLossGrad, true, kTWide, true>(a, st)
+                                 : launch_tstep_mode<kModeOptimize, true, kTWide, true>(a, st);
   // Eight warps a candidate shorten its phases and fill the chip with few candidates (4,352
   // points, T = 1: 152 candidates 0.217 -> 0.136 ms, 912: 0.444 -> 0.364, 2,048: 0.693 -> 0.663,
   // 4,096: 1.197 -> 1.235; 640 points: 304 candidates 0.082 -> 0.065, 608: 0.085 -> 0.092), and the sweeps
