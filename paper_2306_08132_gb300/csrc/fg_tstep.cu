@@ -460,7 +460,9 @@ __device__ __forceinline__ void first_forward_chunk(const ObjDev& O, const Param
 // NEAR: the queries lie at most one cell from the point (near_queries), so along each
 // axis they read the point's own cell or the next one: the 8 corners are read once and
 // a moved query replaces one plane of 4 where it has left the cell, 8 + 6 x 4 predicated loads
-// a point instead of 56.  Same batch: 1.86 -> 1.54 ms, L1 data pipe 72% -> 49%; the four warps a
+// a point instead of 56.  An axis clamped at its upper end stands at the boundary node, as in
+// sdf_lookup, with that node's plane read as the upper one too (stride 0): the value is
+// then the forward sweep's, bit for bit.  Same batch: 1.86 -> 1.54 ms, L1 data pipe 72% -> 49%; the four warps a
 // scheduler that 128 registers leave no longer cover the latencies.
 template <bool ANY, bool NEAR, bool FLAT>
 __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const ParamsDev& Pm, const float (*G)[6],
@@ -469,20 +471,23 @@ __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const Param
   unsigned touch = 0u;
   const float mu = c > 0.0f ? Pm.mu : 0.0f;      // no displacement, no friction
   SdfIndex ix;
-  int cell[3];
+  int cell[3], st[3];                            // st: distance to the cell's upper plane
   float c0[8];
   if constexpr (NEAR) {
+    const int stride[3] = {1, O.sy, O.sz};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const AxisIndex a = sdf_axis<false>(O, k, p[k]);
+      const AxisIndex a = sdf_axis<true>(O, k, p[k]);
       ix.f[k] = a.f;
       ix.du[k] = a.du;
       ix.clamped[k] = a.clamped;
       cell[k] = a.i;
+      st[k] = a.clamped && a.i > 0 ? 0 : stride[k];
     }
     ix.cell = sdf_cell(O, cell[0], cell[1], cell[2]);
-    const bool all[3] = {true, true, true};        // whole cells: a plane that is skipped costs more tests here than it saves
-    sdf_gather(O, ix.cell, all, c0);
+    // whole cells: a plane that is skipped costs more tests here than it saves
+#pragma unroll
+    for (int e = 0; e < 8; ++e) c0[e] = __ldg(ix.cell + (e & 1) * st[0] + ((e >> 1) & 1) * st[1] + (e >> 2) * st[2]);
   }
 #pragma unroll
   for (int m = 0; m < kSims; ++m) {
@@ -498,13 +503,14 @@ __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const Param
         // the query moves against the velocity: down for m odd, up for m even
         const int k = sim_axis(m);
         const bool down = m & 1;
-        const AxisIndex a = sdf_axis<false>(O, k, r[k]);
+        const AxisIndex a = sdf_axis<true>(O, k, r[k]);
         q.f[k] = a.f;
         q.du[k] = a.du;
         q.clamped[k] = a.clamped;
         const bool moved = a.i != cell[k];
-        const int st[3] = {1, O.nx, O.nx * O.ny}, u = (k + 1) % 3, v = (k + 2) % 3;
-        const float* E = ix.cell + (down ? -st[k] : 2 * st[k]);
+        const int u = (k + 1) % 3, v = (k + 2) % 3, step = k == 0 ? 1 : k == 1 ? O.sy : O.sz;
+        // the plane below the cell, or the one above it (at the boundary node, its own plane again)
+        const float* E = ix.cell + (down ? -step : a.clamped ? step : 2 * step);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int lo = ((e & 1) << u) | ((e >> 1) << v), hi = lo | (1 << k);

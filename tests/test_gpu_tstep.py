@@ -199,3 +199,35 @@ def test_tstep_pitch_against_the_displacement(fg, T, nodes, pitch, v_test):
         clean &= ref["N"].reshape(len(clean), -1).sum(axis=1) > 0
     assert clean.sum() >= 3
     _compare(loss.cpu().numpy(), grad.cpu().numpy(), ref, clean)
+
+
+@pytest.mark.parametrize("T", [1, 2])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_tstep_contacts_past_an_upper_face(fg, T, axis):
+    """A hand past a grid's last plane along one axis, where the field is that plane's value plus the excess
+    distance.  The plane before it (1e6) must not enter the value, whose rounding would be 0.03 m against contacts
+    of 0.02 m: the reverse sweep would miss contacts of the forward sweep."""
+    w = synth.tiny_sphere_workload(n_cand=24)
+    n, pitch = 200, 0.002
+    wide, o = pitch * np.arange(n), [a for a in range(3) if a != axis]
+    origin = np.array([-0.1995, -0.2003, -0.1998])
+    origin[axis] = -0.0055
+    plane = -0.02 + 0.15 * (wide + origin[o[0]])[:, None] - 0.1 * (wide + origin[o[1]])[None, :]
+    g = np.full((4, n, n), 1e6)
+    g[-1] = plane
+    g = np.moveaxis(g, 0, axis)                                              # [x, y, z]
+    obj = {"kind": "top", "grid": torch.tensor(np.ascontiguousarray(g.transpose(2, 1, 0)), dtype=torch.float32),
+           "origin": origin.astype(np.float32), "pitch": float(np.float32(pitch)), "mass": 1.0, "inertia": 1e-3,
+           "bound_radius": 0.05, "params": {}}
+    params = dict(w.params, sim_steps=T)
+    S = O.Setup(w.hand, [obj], params)
+    q = w.q0.copy()
+    q[:, :3] = 0.0
+    pts = O.hand_points(S.hand, *O.forward_kinematics(S.hand, torch.tensor(q.astype(np.float64)))).numpy()
+    q[:, axis] = float(obj["origin"][axis]) + 3 * obj["pitch"] + 0.004 - pts[..., axis].min(axis=1)
+    loss, grad = fg.loss_and_grad(fg.Hand.from_synth(w.hand), fg.Scene([fg.Sdf.from_synth(obj)]),
+                                  torch.tensor(q, device=_dev()), params, 0.004)
+    ref = O.batch_loss_and_grad(S, q, np.zeros(len(q), dtype=np.int32), 0.004, chunk=len(q))
+    clean = O.clean_candidates(S.hand, S.objs[0], q, 0.004, S.prm)
+    assert clean.sum() >= 0.25 * len(clean) and (ref["N"].sum(axis=1) > 0).all()
+    _compare(loss.cpu().numpy(), grad.cpu().numpy(), ref, clean)
