@@ -579,9 +579,12 @@ __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const Param
 }
 
 // Whether every query p - s c e_k lies within one cell of p: c below the pitch, with room for
-// the rounding of the index coordinates (below 2^12 + 1 nodes an axis, 2^-11 cells).
+// rounding.  At most 4,096 nodes an axis and an origin at most 4,096 cells away keep the
+// positions of points by the grid below 2^13 cells: p - s c e_k rounds by 2^-11 cells, the two index coordinates
+// by 2^-13 each, together half of the 0.002 left here.  (Points farther out are clamped with their queries.)
 __device__ __forceinline__ bool near_queries(const ObjDev& O, float c) {
-  return O.kind == kObjGrid && c * O.inv_h < 0.998f && max(O.nx, max(O.ny, O.nz)) <= 4096;
+  return O.kind == kObjGrid && c * O.inv_h < 0.998f && max(O.nx, max(O.ny, O.nz)) <= 4096 &&
+         fmaxf(fabsf(O.axis.y), fmaxf(fabsf(O.axis.z), fabsf(O.axis.w))) <= 4096.0f;
 }
 
 // (g, (p - t0) x g) of one point, zero for a lane without one.

@@ -231,3 +231,27 @@ def test_tstep_contacts_past_an_upper_face(fg, T, axis):
     clean = O.clean_candidates(S.hand, S.objs[0], q, 0.004, S.prm)
     assert clean.sum() >= 0.25 * len(clean) and (ref["N"].sum(axis=1) > 0).all()
     _compare(loss.cpu().numpy(), grad.cpu().numpy(), ref, clean)
+
+
+def test_tstep_queries_of_a_frame_far_from_its_origin(fg):
+    """300 m from the origin a position is a multiple of 2^-15 m, 0.0305 cells, so dt V = 0.9979 cells moves a query
+    by 33 of them, 1.007 cells, and some queries land two cells away.  A displacement of 0.9981 cells moves every
+    query by the same 33 multiples: the two gradients differ by the displacement's 2e-4 in friction and test
+    velocity only (2e-3 allowed, and two candidates in which a contact's friction regime changes)."""
+    w = synth.tiny_sphere_workload(n_cand=24)
+    rng = np.random.default_rng(3)
+    centre = np.array([300.0, -290.0, 310.0])
+    base = synth.sphere_grid(0.05, 160, 0.001)
+    rough = torch.tensor(rng.standard_normal((160, 160, 160)), dtype=torch.float32)
+    obj = dict(base, grid=base["grid"] + 0.0015 * rough,
+               origin=(base["origin"].astype(np.float64) + centre).astype(np.float32))
+    q = w.q0.copy()
+    q[:, :3] += centre.astype(np.float32)
+    hand, scene = fg.Hand.from_synth(w.hand), fg.Scene([fg.Sdf.from_synth(obj)])
+    G = []
+    for v_test in (0.9979, 0.9981):
+        _, g = fg.loss_and_grad(hand, scene, torch.tensor(q, device=_dev()),
+                                dict(w.params, sim_steps=1, v_test=v_test), 0.004)
+        G.append(g.cpu().numpy().astype(np.float64))
+    rel = np.sort(_rel_rows(G[0], G[1]))
+    assert rel[-3] < 2e-3, rel
