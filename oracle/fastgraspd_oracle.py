@@ -610,15 +610,19 @@ def evaluate_gs(hand: Hand, obj: Obj, q: torch.Tensor, r: float, prm: Params,
     dth = torch.zeros(B, M_SIMS, 3, dtype=F64)
     Wsum = torch.zeros(B, M_SIMS, 6, dtype=F64)
     phi_ms, Cs, sigs = [], [], []
+    single = anchor_mode or not take or GS_RUN == 1
+    if single:                                   # per-point views (split: the reverse pass gathers their gradients once)
+        views = list(zip(p.split(1, 1), nrm.split(1, 1), phi_hat.split(1, 1)))
     a = 0
     while a < P:
         # points a .. b-1 see the same state: one point, or a run of points without contact
-        b = a + 1 if anchor_mode or not take else _gs_run_end(p, nrm, phi_hat, x_pred, dx, dth, a, force)
-        n_ = nrm[:, a:b, None, :].expand(B, b - a, M_SIMS, 3)
-        d = p[:, a:b, None, :] - x_pred                               # [B,n,M,3]
+        b = a + 1 if single else _gs_run_end(p, nrm, phi_hat, x_pred, dx, dth, a, force)
+        p_i, n_i, ph_i = views[a] if single else (p[:, a:b], nrm[:, a:b], phi_hat[:, a:b])
+        n_ = n_i[:, :, None, :].expand(B, b - a, M_SIMS, 3)
+        d = p_i[:, :, None, :] - x_pred                               # [B,n,M,3]
         x_, th_ = dx[:, None], dth[:, None].expand(B, b - a, M_SIMS, 3)
         Dsp = x_pred + x_ + _cross(th_, d)                            # material point's displacement
-        phi_m = phi_hat[:, a:b, None] - _dot(n_, Dsp)                 # [B,n,M]
+        phi_m = ph_i[:, :, None] - _dot(n_, Dsp)                      # [B,n,M]
         if take:
             dec.state[:, a:b] = torch.cat([dx, dth], -1).detach()[:, None]
             dec.kappa[:, a:b] = _forced(phi_m.detach() < 0, force, "kappa", slice(a, b))
@@ -627,7 +631,7 @@ def evaluate_gs(hand: Hand, obj: Obj, q: torch.Tensor, r: float, prm: Params,
             dx_c, dth_c = st[..., :3], st[..., 3:]
         else:
             dx_c, dth_c = x_.detach(), th_.detach()
-        phi_p = phi_hat[:, a:b, None] - _dot(n_, x_pred + dx_c + _cross(dth_c, d))
+        phi_p = ph_i[:, :, None] - _dot(n_, x_pred + dx_c + _cross(dth_c, d))
         if take:
             dec.anchor[:, a:b] = phi_p.detach()
         anchor = dec.anchor[:, a:b].clone() if anchor_mode else phi_p.detach()

@@ -99,13 +99,18 @@ class FlopCounter(TorchDispatchMode):
 
 def count_step(setup: O.Setup, q32: np.ndarray, obj_index: int, r: float, want_grad: bool = True) -> dict:
     """Flops of the oracle's loss (and gradient) for candidates q32 [B, D] on one object.
-    Returns totals and per point-step figures (divided by B x P)."""
+    Returns totals and per point-step figures (divided by B x P).  The Gauss-Seidel sweep is counted
+    one point at a time (its search for runs of points is not the method's work)."""
     hand, obj = setup.hand, setup.objs[obj_index]
     q = torch.as_tensor(np.asarray(q32, dtype=np.float64)).clone().requires_grad_(want_grad)
-    with FlopCounter() as fc:
-        out = O.evaluate_any(hand, obj, q, r, setup.prm)
-        if want_grad:
-            torch.autograd.grad(out["L"].sum(), q)
+    run, O.GS_RUN = O.GS_RUN, 1
+    try:
+        with FlopCounter() as fc:
+            out = O.evaluate_any(hand, obj, q, r, setup.prm)
+            if want_grad:
+                torch.autograd.grad(out["L"].sum(), q)
+    finally:
+        O.GS_RUN = run
     units = q.shape[0] * hand.P
     return {"flops": fc.flops, "special": fc.special, "point_steps": units,
             "flops_per_point_step": fc.flops / units, "special_per_point_step": fc.special / units,
