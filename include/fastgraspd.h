@@ -422,11 +422,17 @@ fg_status fg_grasp_epsilon(const fg_hand* hand, const fg_scene* scene, const int
  * per SM the register allocation is held to, and the points each thread carries
  * per iteration of the adjoint sweep (independent dependency chains).  The selection is
  * per device (the current one) and applies to fg_loss_and_grad and
- * fg_optimize_step; it changes no result beyond float32 summation order. */
+ * fg_optimize_step.  Configurations of one point per thread give the same results bit
+ * for bit; those of two add a work unit's halves in another order. */
 fg_status fg_fused_config_count(int* n);
 fg_status fg_fused_config_info(int index, int* warps_per_candidate, int* min_ctas_per_sm,
                                int* points_per_thread);
-/* index in [0, count) selects a configuration; -1 restores the default. */
+/* index in [0, count) selects a configuration for all launches; -1 restores the
+ * default: each launch takes 4, 8 or 16 warps per candidate by its number of
+ * candidates, the hand's points and the scene's objects.  (Scenes with grids of
+ * constant cells that can be in contact have one configuration, whatever is selected.)
+ * current gives the selected index, or -1 when none is, so that its value can be
+ * selected again later.  fg_contact_wrench and the request queue always use 4 warps. */
 fg_status fg_fused_config_select(int index);
 fg_status fg_fused_config_current(int* index);
 

@@ -301,10 +301,12 @@ def fused_configs() -> list[tuple[int, int, int]]:
 
 
 def fused_config_select(index: int) -> None:
+    """Select a configuration by its index, or -1: by the size of each launch."""
     check(_lib.load().fg_fused_config_select(int(index)), "fg_fused_config_select")
 
 
 def fused_config_current() -> int:
+    """The selected configuration's index, -1 when none is selected."""
     i = C.c_int()
     check(_lib.load().fg_fused_config_current(C.byref(i)), "fg_fused_config_current")
     return i.value

@@ -15,7 +15,7 @@ static const int kCfgMinB[] = {FG_FUSED_CONFIGS(FG_CFG_MB)};
 static const int kCfgPPT[] = {FG_FUSED_CONFIGS(FG_CFG_PPT)};
 static const FusedLaunchFn kLossGradLaunch[] = {FG_FUSED_CONFIGS(FG_CFG_LOSSGRAD)};
 constexpr int kNumCfg = sizeof(kCfgNW) / sizeof(kCfgNW[0]);
-constexpr int kDefaultCfg = 1;   // 4 warps per candidate, >= 5 CTAs per SM, 1 point per thread
+constexpr int kCfg4 = 1;         // 4 warps per candidate, >= 5 CTAs per SM, 1 point per thread
 constexpr int kCfg8 = 4;         // 8 warps, >= 3 CTAs per SM
 constexpr int kCfg16 = 11;       // 16 warps, >= 1 CTA per SM
 
@@ -32,7 +32,7 @@ static int default_config(const FusedArgs& a) {
   const bool large = a.hand_P >= 2048;
   if (a.any_mesh) return B <= 32 * sms ? kCfg16 : kCfg8;
   if (B <= (large ? 3 : 1) * sms) return kCfg16;
-  return B <= (large ? 12 : 4) * sms ? kCfg8 : kDefaultCfg;
+  return B <= (large ? 12 : 4) * sms ? kCfg8 : kCfg4;
 }
 
 static int g_selected[64] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1,
@@ -51,10 +51,8 @@ static int& selected_slot() {
   cudaGetDevice(&dev);
   return g_selected[dev & 63];
 }
-int fused_config_current() {
-  int s = selected_slot();
-  return s < 0 ? kDefaultCfg : s;
-}
+// -1 when none is selected (each launch then follows default_config).
+int fused_config_current() { return selected_slot(); }
 void fused_config_select(int i) { selected_slot() = i; }
 
 cudaError_t launch_fused(int mode, const FusedArgs& a, const fg_hand* h, cudaStream_t st) {
@@ -101,7 +99,7 @@ cudaError_t autotune_fused(const FusedArgs& base, int reps, float* times_ms, int
   cudaEventCreate(&t0);
   cudaEventCreate(&t1);
   float best_ms = 3.0e38f;
-  int best_i = kDefaultCfg;
+  int best_i = kCfg4;
   for (int i = 0; i < kNumCfg && e == cudaSuccess; ++i) {
     FusedArgs a = base;
     a.q = qtmp;

@@ -180,3 +180,18 @@ def test_mesh_description_on_the_host(lib):
     assert db["fan_vertices"] == len(V) - 1            # the shared vertex: two fans
     with pytest.raises(Exception, match="watertight"):
         fg.Sdf.describe_mesh(sq["vertices"], sq["faces"][:-1])
+
+
+def test_fused_config_current_can_be_selected_again(lib):
+    """Without a selection each launch picks its warps by size: current says -1, and selecting what current said
+    restores that state."""
+    i = C.c_int()
+    assert lib.fg_fused_config_select(-1) == 0
+    assert lib.fg_fused_config_current(C.byref(i)) == 0 and i.value == -1
+    try:
+        assert lib.fg_fused_config_select(3) == 0
+        assert lib.fg_fused_config_current(C.byref(i)) == 0 and i.value == 3
+    finally:
+        assert lib.fg_fused_config_select(-1) == 0
+    assert lib.fg_fused_config_current(C.byref(i)) == 0 and i.value == -1
+    assert lib.fg_fused_config_select(i.value) == 0
