@@ -1,12 +1,12 @@
 // Device-side data layouts and per-point arithmetic of the grasp-search step.
 //
-// Everything a kernel needs about one step of one candidate lives here, written
-// once and used by the fused kernel (fg_fused.cu) and the per-stage kernels
-// (fg_plain.cu).  The arithmetic that decides a branch (point position, grid
-// cell, interpolated value and normal, contact flag, friction regime) is spelled
-// with explicit round-to-nearest intrinsics so that every call site rounds
-// identically and the forward sweep, the adjoint sweep and the per-stage form
-// agree bit for bit on every decision.
+// What a kernel needs about one step of one candidate lives here, for the fused
+// kernel (fg_fused.cu) and the per-stage kernels (fg_plain.cu).  The forces and their
+// adjoints are written twice, in the short forms of the fused kernel and as vectors for the per-stage
+// form; the arithmetic that decides a branch (point position, grid cell, interpolated
+// value and normal, contact flag, friction regime) has the same operations in both, spelled
+// with explicit round-to-nearest intrinsics, so that the forward sweep, the
+// adjoint sweep and the per-stage form agree bit for bit on every decision.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -307,6 +307,8 @@ __device__ __forceinline__ float rsqrt_fast(float x) {
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// With x bounded away from 0.
+__device__ __forceinline__ float rsqrt_bounded(float x) { return rsqrt_fast(fmaxf(x, 1e-30f)); }
 // 0 where x is not a positive normal float (zero, subnormal, NaN).
 __device__ __forceinline__ float rsqrt_or_zero(float x) { return x >= 1.17549435e-38f ? rsqrt_fast(x) : 0.0f; }
 // Reciprocal of a positive, normal float (the effective inverse masses w_n, w_t
@@ -1019,7 +1021,7 @@ __device__ __forceinline__ float sim_tangent(const float n[3], int m, float t[3]
   const float nk = k0 ? n[0] : (k2 ? n[2] : n[1]);
   const float ea = k0 ? n[1] : n[0];
   const float eb = k2 ? n[1] : n[2];
-  const float rho2 = fma_(ea, ea, mul_(eb, eb));
+  const float rho2 = add_(mul_(ea, ea), mul_(eb, eb));      // as in sim_axis_terms: it decides the regime
   if (rho2 == 0.0f && nk == 0.0f) {
     t[0] = k0 ? sg : 0.0f;
     t[1] = k1 ? sg : 0.0f;
@@ -1027,7 +1029,7 @@ __device__ __forceinline__ float sim_tangent(const float n[3], int m, float t[3]
     return 1.0f;
   }
   if (!(rho2 > 0.0f)) return 0.0f;
-  const float rr = rsqrtf(rho2);
+  const float rr = rsqrt_bounded(rho2);
   const float rho = mul_(rho2, rr);
   const float cc = -sg * nk * rr;
   t[0] = k0 ? sg * rho : cc * n[0];
@@ -1275,7 +1277,6 @@ template <class V>
 struct SimAxis {
   V rho2, rr, wn0, wn1, wt0, wt1;
 };
-__device__ __forceinline__ float rsqrt_bounded(float x) { return rsqrt_fast(fmaxf(x, 1e-30f)); }
 template <class V>
 __device__ __forceinline__ void sim_axis_terms(const V n[3], const SimShared<V>& q, const SimK4<V>& k0, int k,
                                                SimAxis<V>& x) {

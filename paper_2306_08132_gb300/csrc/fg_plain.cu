@@ -10,7 +10,8 @@
 //   6 contact_adj    -> dL/dp                    SoA [3][B*P]
 //   7 link_reduce    -> per-link sums            [B][L][6]       (one CTA per candidate)
 //   8 fk_adj_update  -> dL/dq, q update          [B][D]
-// The per-point arithmetic is the same device code as the fused kernel.
+// Lookups and everything that decides a branch are the fused kernel's operations; the forces and
+// their adjoint are the vector forms (contact_force, sim_adjoint).
 #include <cuda_runtime.h>
 
 #include "fg_fused_kernel.cuh"

@@ -423,3 +423,40 @@ def test_large_hand_results_do_not_depend_on_the_batch(fg):
     clean = case.clean(case.w.q0, 0.004)
     assert clean.sum() >= 1
     _compare_loss_grad(l0.cpu().numpy(), g0.cpu().numpy(), ref, clean)
+
+
+def test_per_stage_form_takes_the_fused_kernel_s_friction_regime(fg):
+    """One point on planes of 256 normals, the dilation scanned float by float across sigma = mu C of one simulation:
+    the per-stage step and the fused step switch from kinetic to static at the same float."""
+    rng = np.random.default_rng(11)
+    hand = fg.Hand([-1], np.eye(3, 4), np.zeros((1, 3)), [], [], np.zeros((1, 3)), [0])
+    r0, c, mu, n_obj, steps = 0.0008, 1e-3, 0.5, 256, 1000
+    sdfs = []
+    for _ in range(n_obj):
+        n = rng.standard_normal(3)
+        n /= np.linalg.norm(n)
+        offset = r0 + c * n[0] - c * np.sqrt(1 - n[0] ** 2) / mu            # at the origin C = sigma/mu for v = +x
+        sdfs.append(fg.Sdf.from_synth(synth.linear_grid(tuple(n), offset, 8, 0.01)))
+    scene = fg.Scene(sdfs)
+    oc = torch.arange(n_obj, device=_dev(), dtype=torch.int32)
+    q0 = torch.zeros(n_obj, 6, device=_dev())
+    q0[:, 3:] = torch.tensor(rng.standard_normal((n_obj, 3)) * 1e-3, device=_dev(), dtype=torch.float32)
+    params = dict(synth.tiny_sphere_workload(n_cand=1).params, alpha_leak=0.0, lr=1.0, mu=mu)
+    ws = torch.empty(fg.plain_workspace_size(hand, n_obj) + 256, dtype=torch.uint8, device=_dev())
+    mismatches = torch.zeros(n_obj, device=_dev(), dtype=torch.int32)
+    switched = torch.zeros(n_obj, device=_dev(), dtype=torch.bool)
+    before = None
+    r = np.float32(r0) - np.float32(steps // 2) * np.spacing(np.float32(r0))
+    for _ in range(steps):
+        p = dict(params, r0=float(r))
+        _, grad = fg.loss_and_grad(hand, scene, q0, p, float(r), obj_of_cand=oc)
+        q = q0.clone()
+        fg.optimize_step_plain(hand, scene, q, p, 0, 10, 1, obj_of_cand=oc, workspace=ws)
+        size = grad.norm(dim=1).clamp(min=1e-6)
+        mismatches += (grad - (q0 - q)).norm(dim=1) > 1e-3 * size
+        if before is not None:
+            switched |= (grad - before).norm(dim=1) > 1e-3 * size
+        before = grad
+        r = np.nextafter(r, np.float32(1))
+    assert int(switched.sum()) >= 32
+    assert int(mismatches.sum()) == 0, mismatches.nonzero().flatten().tolist()
