@@ -1141,7 +1141,7 @@ __device__ __forceinline__ void sim_adjoint(const PointState& ps, int m, float p
       dtt[0] += tmp[0]; dtt[1] += tmp[1]; dtt[2] += tmp[2];
       // t = s/sigma, sigma = |s|: ds = (dt - (t.dt) t)/sigma + dsig t
       const float tdt = dot3(t, dtt);
-      const float rs = __fdividef(1.0f, sigma);
+      const float rs = sigma > 0.0f ? __fdividef(1.0f, sigma) : 0.0f;    // at v_test = 0 nothing slides
       float ds[3];
 #pragma unroll
       for (int k = 0; k < 3; ++k) ds[k] = (dtt[k] - tdt * t[k]) * rs + dsig * t[k];

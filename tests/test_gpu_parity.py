@@ -460,3 +460,16 @@ def test_per_stage_form_takes_the_fused_kernel_s_friction_regime(fg):
         r = np.nextafter(r, np.float32(1))
     assert int(switched.sum()) >= 32
     assert int(mismatches.sum()) == 0, mismatches.nonzero().flatten().tolist()
+
+
+def test_per_stage_form_at_zero_test_velocity(fg, tiny):
+    """v_test = 0 is accepted: the displacement is 0, friction and its derivative vanish, and the per-stage step is
+    finite and the fused step's."""
+    params = dict(tiny.w.params, v_test=0.0, w_pen=0.5)
+    q0 = torch.tensor(tiny.w.q0, device=_dev())
+    a, b = q0.clone(), q0.clone()
+    la = fg.optimize_step(tiny.hand, tiny.scene, a, params, 0, 10, 1, obj_of_cand=tiny.oc)
+    lb = fg.optimize_step_plain(tiny.hand, tiny.scene, b, params, 0, 10, 1, obj_of_cand=tiny.oc)
+    assert torch.isfinite(a).all() and torch.isfinite(b).all()
+    assert torch.allclose(la, lb, rtol=LOSS_TOL, atol=1e-6)
+    assert rel_rows((q0 - b).cpu().numpy(), (q0 - a).cpu().numpy()).max() < GRAD_TOL
