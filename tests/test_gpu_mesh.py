@@ -400,3 +400,21 @@ def test_mesh_hand_beyond_the_kept_faces(fg):
     ref = O.batch_loss_and_grad(c.S, qs, c.oc_np, 0.004)
     assert np.all(np.abs(loss.cpu().numpy() - ref["L"]) <= 1e-3 * np.abs(ref["L"]) + 1e-4)
     assert torch.isfinite(grad).all()
+
+
+@pytest.mark.parametrize("points_per_link,gauss_seidel,subdivisions", [(21, 0, 2), (21, 1, 2), (840, 0, 1)])
+def test_mesh_gradients_of_ragged_and_large_hands_match_oracle(fg, points_per_link, gauss_seidel, subdivisions):
+    """The adjoint from kept faces on links of 21 points (chunks and work units that end inside a link), in both
+    constraint orders, and from a second search with 8,400 points, whose faces are not kept."""
+    w = synth.tiny_sphere_workload(n_cand=3)
+    h = synth.make_hand(3, points_per_link)
+    n = 12 if points_per_link < 100 else 6
+    qs = synth.sample_candidates(np.random.default_rng(9), h, n, 0.09)
+    params = dict(w.params, gauss_seidel=gauss_seidel)
+    c = Case(fg, h, [SM.icosphere(0.04, subdivisions)], np.zeros(n, dtype=np.int32), qs, params)
+    S = O.Setup(h, c.objects, params)
+    loss, grad = fg.loss_and_grad(c.hand, c.scene, torch.tensor(qs, device=_dev()), params, 0.004)
+    ref = O.batch_loss_and_grad(S, qs, c.oc_np, 0.004)
+    clean = O.clean_candidates(S.hand, S.objs[0], qs, 0.004, S.prm)
+    assert (clean & (ref["N"].sum(axis=1) > 0)).sum() >= 1
+    _compare(loss.cpu().numpy(), grad.cpu().numpy(), ref, clean)
