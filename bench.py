@@ -496,8 +496,8 @@ class Bound:
 def roofline_of(w, S_in, kern_ms, peak, hbm_gbs, hbm_basis, prof):
     """Roofline of one fused launch: the ALU time of the method's work at the measured
     FP32 peak against the DRAM time of the launch's measured traffic at the HBM
-    bandwidth; the slower one bounds it.  Three fractions of the ALU peak, by the
-    basis of the flop count."""
+    bandwidth.  Three fractions of the ALU peak, by the basis of the flop count: the oracle's
+    count is above what the kernel executes, so its time is no lower bound of the kernel's."""
     units = w.B * w.hand["P"] * S_in
     kern_s = kern_ms / 1000.0
     P = peak["tflops"]
@@ -510,7 +510,8 @@ def roofline_of(w, S_in, kern_ms, peak, hbm_gbs, hbm_basis, prof):
     fractions = {
         "oracle_count": {"flops_per_point_step": FLOPS_PER_POINT_STEP, "frac": alu_tflops / P,
                          "basis": "the method's work as the FP64 oracle computes it (oracle/flop_count.py: "
-                                  "forward pass + reverse mode, both arms of every select)"},
+                                  "forward pass + reverse mode, both arms of every select); the kernel takes fewer "
+                                  "operations (executed_fp32), so this is no bound and can exceed 1"},
         "kernel_minimal": {"flops_per_point_step": KERNEL_MIN_FLOPS_PER_POINT_STEP,
                            "frac": KERNEL_MIN_FLOPS_PER_POINT_STEP * units / kern_s / 1e12 / P,
                            "basis": "the fused kernel's own operation count for a point of a candidate without contacts "

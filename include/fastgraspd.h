@@ -430,7 +430,8 @@ fg_status fg_fused_config_info(int index, int* warps_per_candidate, int* min_cta
 /* index in [0, count) selects a configuration for all launches; -1 restores the
  * default: each launch takes 4, 8 or 16 warps per candidate by its number of
  * candidates, the hand's points and the scene's objects.  (Scenes with grids of
- * constant cells that can be in contact have one configuration, whatever is selected.)
+ * constant cells that can be in contact have kernels of 4 and of 8 warps only: the
+ * selection's warps above 4 mean 8, with a mesh object all take 8.)
  * current gives the selected index, or -1 when none is, so that its value can be
  * selected again later.  fg_contact_wrench and the request queue always use 4 warps. */
 fg_status fg_fused_config_select(int index);

@@ -333,7 +333,7 @@ fg_status fg_sdf_create(const float* grid, int nx, int ny, int nz, const float* 
   o.inv_inertia = 1.0f / inertia;
   o.axis = make_float4(o.inv_h, -origin[0] * o.inv_h, -origin[1] * o.inv_h, -origin[2] * o.inv_h);
   o.n_max = make_float4((float)(nx - 1), (float)(ny - 1), (float)(nz - 1), pitch);
-  o.cap = make_int4(nx - 2, ny - 2, nz - 2, ny);
+  o.cap = make_int4(nx - 2, ny - 2, nz - 2, 0);
   o.sy = nx;
   o.sz = nx * ny;
   int levels = 0;

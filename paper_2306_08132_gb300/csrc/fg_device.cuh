@@ -53,7 +53,7 @@ struct alignas(16) ObjDev {
   // 4-byte load costs the same wavefront).
   float4 axis;                   // 1/pitch, then uo = -origin / pitch per axis: index coordinate u = p / pitch + uo
   float4 n_max;                  // nx - 1, ny - 1, nz - 1 as floats, pitch
-  int4 cap;                      // nx - 2, ny - 2, nz - 2 (last cell), ny
+  int4 cap;                      // nx - 2, ny - 2, nz - 2 (last cell); w unused
   const float* grid;             // [nz][ny][nx]
   int sy, sz;                    // strides nx, nx ny
   int nx, ny, nz;

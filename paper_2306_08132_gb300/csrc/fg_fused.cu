@@ -25,8 +25,10 @@ constexpr int kCfg16 = 11;       // 16 warps, >= 1 CTA per SM
 // 0.150, 0.166; 1,824: 0.251, 0.225, 0.297; 4,096: 0.433, 0.445, 0.626.  A small hand has too
 // few chunks to share (640 points: 152 candidates 0.041, 0.033, 0.028; 304: 0.044, 0.037,
 // 0.044; 912: 0.058, 0.059, 0.092).  On a mesh a candidate inside the object costs many
-// times the others, so more warps shorten the end of the launch (2,208 faces: 1,024
-// candidates 2.11, 1.40, 1.29; 4,096: 6.03, 4.49, 4.08; 8,192: 9.19, 7.65, 7.55).
+// times the others, so more warps shorten the end of the launch (4,352 points, 2,208 faces: 1,024
+// candidates 2.11, 1.40, 1.29; 4,096: 6.03, 4.49, 4.08; 8,192: 9.19, 7.65, 7.55: 16 warps are
+// ahead at every size measured, by 1% where the line to 8 lies; other hands on meshes were not measured).
+// The configuration changes no result: units, chunks and sums are the same at any number of warps.
 static int default_config(const FusedArgs& a) {
   const long long sms = device_sm_count(), B = a.B;
   const bool large = a.hand_P >= 2048;
@@ -58,8 +60,8 @@ void fused_config_select(int i) { selected_slot() = i; }
 cudaError_t launch_fused(int mode, const FusedArgs& a, const fg_hand* h, cudaStream_t st) {
   (void)h;
   if (a.B <= 0) return cudaSuccess;
-  if (a.any_flat) return launch_fused_flat(mode, a, st);
   const int chosen = selected_slot(), cfg = chosen < 0 ? default_config(a) : chosen;
+  if (a.any_flat) return launch_fused_flat(mode, kCfgNW[cfg] > 4, a, st);
   if (a.any_mesh) {
     switch (mode) {
       case kModeWrench: return launch_wrench_any(a, st);
@@ -77,7 +79,7 @@ cudaError_t launch_fused(int mode, const FusedArgs& a, const fg_hand* h, cudaStr
 // One round of a request queue: every active request's candidates in one launch.
 cudaError_t launch_queue_round(const FusedArgs& a, cudaStream_t st) {
   if (a.B <= 0) return cudaSuccess;
-  if (a.any_flat) return launch_fused_flat(kModeQueue, a, st);
+  if (a.any_flat) return launch_fused_flat(kModeQueue, false, a, st);
   if (a.any_mesh) return launch_queue_round_any(a, st);
   return launch_fused_cfg<kModeQueue, 4, 5, 1>(a, st);
 }
@@ -109,7 +111,7 @@ cudaError_t autotune_fused(const FusedArgs& base, int reps, float* times_ms, int
       e = cudaMemcpyAsync(qtmp, base.q, sizeof(float) * (size_t)base.B * D, cudaMemcpyDeviceToDevice, st);
       if (e != cudaSuccess) break;
       cudaEventRecord(t0, st);
-      e = base.any_flat ? launch_fused_flat(kModeOptimize, a, st)
+      e = base.any_flat ? launch_fused_flat(kModeOptimize, kCfgNW[i] > 4, a, st)
                         : (base.any_mesh ? kOptimizeLaunchAny : kOptimizeLaunch)[i](a, st);
       cudaEventRecord(t1, st);
       if (e == cudaSuccess) e = cudaEventSynchronize(t1);

@@ -63,7 +63,8 @@ struct FusedSmem {
   float* qout;
   float* lout;
   int cl, step0, total, nsteps;
-  int flat;                        // FLAT kernels: the candidate has contacts where the SDF's gradient is zero
+  int flat;                        // FLAT kernels: the candidate has contacts where the SDF's gradient is zero,
+  unsigned flat_bits[kMaxCullChunks / 32];   // and its chunks that hold them
 };
 
 __device__ __forceinline__ void store_frame(const Frame& F, float4* f4) {
@@ -278,8 +279,8 @@ __device__ __forceinline__ void unit_reduce_add_fixed(const float a[6], int lane
 
 // Forces and torques of a warp's 32 points in every simulation, added to the sums
 // wfix[m] (6 values and the count; the penetration of simulation 0 in its slot 7);
-// flags(m, word) takes the contact flags; with FLAT, *flat is set when a contact's gradient is
-// zero (its friction: flat_forces).  With the shared terms of the adjoint
+// flags(m, word) takes the contact flags; contacts where the gradient is zero get no friction
+// here (flat_forces).  With the shared terms of the adjoint
 // (point_sims_adjoint), lambda_t = min(sigma, mu C)/w_t and sigma = c rho,
 //   f = A n + B e_k,              B = -s lambda_t/rho,  A = -lambda_n - B n_k
 //   d x f = A (U - s c E_k) + B p x e_k
@@ -287,9 +288,9 @@ __device__ __forceinline__ void unit_reduce_add_fixed(const float a[6], int lane
 // products and selects of the axis took about 110.  One axis at a time, the components
 // rotated so that it comes first: one copy of the code.  8-superquadric batch
 // 0.963 -> 0.924 ms, 256-object sweep 8.91 -> 8.60 ms.
-template <bool FLAT, class F>
+template <class F>
 __device__ __forceinline__ void chunk_forces(const PointState& ps, const SimConsts& K, bool valid, float c, float w_pen,
-                                             int lane, unsigned long long (*wfix)[8], int* flat, F flags) {
+                                             int lane, unsigned long long (*wfix)[8], F flags) {
   const SimK4<float> k0 = simk4(K, 0.0f, 0);
   const float mu = K.s[4];
   SimShared<float> q;
@@ -306,7 +307,6 @@ __device__ __forceinline__ void chunk_forces(const PointState& ps, const SimCons
       const float w = unit_reduce(v, lane);
       if (holds) atomicAdd(&wfix[0][rank], to_fixed(w));
       if (lane == 0) atomicAdd(&wfix[0][6], (unsigned long long)__popc(bal));
-      if (FLAT && kap && flat_contact(ps)) *flat = 1;
       if (w_pen != 0.0f) {
         const float pen = warp_sum(kap ? -ps.phi_hat : 0.0f);
         if (lane == 0) atomicAdd(&wfix[0][7], to_fixed(pen));
@@ -459,20 +459,25 @@ __device__ __forceinline__ void adjoint_sweep(FusedSmem<NW>& S, const ObjDev& O,
 
 // The friction of contacts where the gradient is zero, added to the forward sums, and its
 // adjoint, added to the sums of units [u0, u1): passes of their own over the points, for
-// candidates that have such contacts, compiled into the FLAT kernels only.  In the kernels for all scenes the same
+// candidates and chunks that have such contacts, compiled into the FLAT kernels only.  In the kernels for all scenes the same
 // terms as selects in the two sweeps cost the 256-object sweep 6%, as branches 4%,
 // and the two calls 2%.
 template <int NW>
+__device__ __forceinline__ bool flat_chunk(const FusedSmem<NW>& S, int j) {
+  return S.H.nchunks > kMaxCullChunks || ((S.flat_bits[j >> 5] >> (j & 31)) & 1u);
+}
+template <int NW, bool ANY>
 __device__ __noinline__ void flat_forces(FusedSmem<NW>& S, float r, float c, int lane, int warp) {
   const HandDev& H = S.H;
   for (int j = warp; j < H.nchunks; j += NW) {
+    if (!flat_chunk(S, j)) continue;
     const int i = 32 * j + lane;
     const bool valid = i < H.P;
     const float4 sp = __ldg(H.pts + (valid ? i : 32 * j));
     float p[3];
     world_point(S.frame4[(int)sp.w], sp, p);
     SdfSample smp;
-    sdf_lookup<false, true>(S.O, p, smp);
+    sdf_lookup<false, ANY>(S.O, p, smp);
     PointState ps;
     point_state(smp, p, r, ps);
     const bool flat = valid && flat_contact(ps);
@@ -487,17 +492,18 @@ __device__ __noinline__ void flat_forces(FusedSmem<NW>& S, float r, float c, int
       const float v[6] = {k == 0 ? B : 0.0f, k == 1 ? B : 0.0f, k == 2 ? B : 0.0f,
                           B * (k == 0 ? 0.0f : k == 1 ? -pi : pj), B * (k == 0 ? pj : k == 1 ? 0.0f : -pi),
                           B * (k == 0 ? -pi : k == 1 ? pj : 0.0f)};
-      const float w = unit_reduce(v, lane);
-      const int rank = lane >> 2;
-      if ((lane & 3) == 0 && rank < 6) atomicAdd(&S.wfix[m][rank], to_fixed(w));
+      unit_reduce_add_fixed(v, lane, S.wfix[m]);
     }
   }
 }
-template <int NW>
+template <int NW, bool ANY>
 __device__ __noinline__ void flat_adjoint(FusedSmem<NW>& S, float r, float c, int u0, int u1, int lane, int warp) {
   const HandDev& H = S.H;
   for (int u = u0 + warp; u < u1; u += NW) {
     const int4 U = __ldg(H.units + u);
+    bool some = false;
+    for (int j = U.x >> 5; j <= (U.x + U.y - 1) >> 5; ++j) some = some || flat_chunk(S, j);
+    if (!some) continue;
     float sum[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
     for (int h = 0; h < U.y; h += 32) {
       const bool valid = h + lane < U.y;
@@ -505,7 +511,7 @@ __device__ __noinline__ void flat_adjoint(FusedSmem<NW>& S, float r, float c, in
       float p[3];
       world_point(S.frame4[U.z], sp, p);
       SdfSample smp;
-      sdf_lookup<false, true>(S.O, p, smp);
+      sdf_lookup<false, ANY>(S.O, p, smp);
       PointState ps;
       point_state(smp, p, r, ps);
       float dp[3] = {0.0f, 0.0f, 0.0f}, tq[3];
@@ -604,6 +610,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
       for (int idx = tid; idx < kSims * 8; idx += NW * 32) (&S.wfix[0][0])[idx] = 0ull;
       if (tid == 0) S.next_chunk = 0;
       if (FLAT && tid == 0) S.flat = 0;
+      if (FLAT && tid < kMaxCullChunks / 32) S.flat_bits[tid] = 0u;
       __syncthreads();
       const ObjDev& O = S.O;
 
@@ -698,7 +705,11 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
           }
           PointState ps;
           point_state(smp, p, r, ps);
-          chunk_forces<FLAT>(ps, S.K, valid, dtV, Pm.w_pen, lane, S.wfix, &S.flat, [&](int m, unsigned bal) {
+          if (FLAT && __any_sync(kFull, valid && flat_contact(ps)) && lane == 0) {
+            S.flat = 1;
+            if (H.nchunks <= kMaxCullChunks) atomicOr(&S.flat_bits[base >> 10], 1u << ((base >> 5) & 31));
+          }
+          chunk_forces(ps, S.K, valid, dtV, Pm.w_pen, lane, S.wfix, [&](int m, unsigned bal) {
             if (MODE == kModeWrench && lane == 0 && a.bits)
               a.bits[((size_t)c * kSims + m) * nwords + (base >> 5)] = bal;
           });
@@ -707,7 +718,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
       }
       __syncthreads();
       if (FLAT && S.flat) {
-        flat_forces(S, r, dtV, lane, warp);
+        flat_forces<NW, ANY>(S, r, dtV, lane, warp);
         __syncthreads();
       }
 
@@ -794,7 +805,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_step_kernel(FusedArgs a) 
           adjoint_sweep<NW, PPT, ANY, false>(S, O, r, faces, u0, u1, lane);
         __syncthreads();
         if (FLAT && S.flat) {
-          flat_adjoint(S, r, dtV, u0, u1, lane, warp);
+          flat_adjoint<NW, ANY>(S, r, dtV, u0, u1, lane, warp);
           __syncthreads();
         }
         // per-link sums, one thread per link and component

@@ -558,8 +558,9 @@ __global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_ke
       // A mesh object whose adjoint follows has every point's closest face searched here,
       // once, by all warps (each later lookup evaluates from the face, where the seven
       // simulations' walks used to search again), and lb is the chunk's smallest phi_hat itself.
-      // GS_8 objects x 128 candidates of 4,352 points, 2,208 faces
-      // each: 3.7-4.6 -> 2.6 ms, with 16 warps a candidate 1.3-1.7 ms.
+      // 4 objects x 128 candidates of 4,352 points, 2,208 faces each: 12.4-16.9 -> 1.25-1.5 ms with
+      // 14 warps a candidate and planes rejected first.  Two CTAs of 14 warps leave 72 registers a
+      // thread, and the reverse walk spills 450 bytes of them.
       int* faces = nullptr;
       if (ANY && MODE != kModeWrench && O.kind == kObjMesh && P <= a.face_cap && (MODE == kModeOptimize || a.grad != nullptr))
         faces = reinterpret_cast<int*>(dyn + (size_t)nch * kSims * kSnapWords);
@@ -1019,7 +1020,7 @@ __global__ void __launch_bounds__((ANY ? kGWMesh : kGW) * 32, ANY ? 2 : 3) gs_ke
   work_done(a.work);
 }
 
-template <int MODE, bool ANY, bool FLAT = false>
+template <int MODE, bool ANY, bool FLAT>
 cudaError_t launch_gs_mode(const FusedArgs& a, int nchunks, cudaStream_t st) {
   constexpr int GW = ANY ? kGWMesh : kGW;
   FusedArgs b = a;
@@ -1048,22 +1049,19 @@ cudaError_t launch_gs_mode(const FusedArgs& a, int nchunks, cudaStream_t st) {
 
 }  // namespace
 
+template <bool ANY, bool FLAT>
+static cudaError_t launch_gs_kind(int mode, const FusedArgs& a, int nchunks, cudaStream_t st) {
+  if (mode == kModeWrench) return launch_gs_mode<kModeWrench, ANY, FLAT>(a, nchunks, st);
+  return mode == kModeLossGrad ? launch_gs_mode<kModeLossGrad, ANY, FLAT>(a, nchunks, st)
+                               : launch_gs_mode<kModeOptimize, ANY, FLAT>(a, nchunks, st);
+}
+
 cudaError_t launch_gs(int mode, const FusedArgs& a, int nchunks, cudaStream_t st) {
   if (a.B <= 0) return cudaSuccess;
   if (nchunks < 1 || nchunks > kMaxCullChunks) return cudaErrorInvalidValue;
-  if (a.any_flat) {
-    if (mode == kModeWrench) return launch_gs_mode<kModeWrench, true, true>(a, nchunks, st);
-    return mode == kModeLossGrad ? launch_gs_mode<kModeLossGrad, true, true>(a, nchunks, st)
-                                 : launch_gs_mode<kModeOptimize, true, true>(a, nchunks, st);
-  }
-  if (a.any_mesh) {
-    if (mode == kModeWrench) return launch_gs_mode<kModeWrench, true>(a, nchunks, st);
-    return mode == kModeLossGrad ? launch_gs_mode<kModeLossGrad, true>(a, nchunks, st)
-                                 : launch_gs_mode<kModeOptimize, true>(a, nchunks, st);
-  }
-  if (mode == kModeWrench) return launch_gs_mode<kModeWrench, false>(a, nchunks, st);
-  return mode == kModeLossGrad ? launch_gs_mode<kModeLossGrad, false>(a, nchunks, st)
-                               : launch_gs_mode<kModeOptimize, false>(a, nchunks, st);
+  if (a.any_flat)
+    return a.any_mesh ? launch_gs_kind<true, true>(mode, a, nchunks, st) : launch_gs_kind<false, true>(mode, a, nchunks, st);
+  return a.any_mesh ? launch_gs_kind<true, false>(mode, a, nchunks, st) : launch_gs_kind<false, false>(mode, a, nchunks, st);
 }
 
 }  // namespace fg

@@ -95,12 +95,13 @@ typedef cudaError_t (*FusedLaunchFn)(const FusedArgs&, cudaStream_t);
 extern const FusedLaunchFn kOptimizeLaunch[];
 extern const FusedLaunchFn kOptimizeLaunchAny[];
 extern const FusedLaunchFn kLossGradLaunchAny[];
-cudaError_t launch_fused_flat(int mode, const FusedArgs& a, cudaStream_t st);
+cudaError_t launch_fused_flat(int mode, bool wide, const FusedArgs& a, cudaStream_t st);
 cudaError_t launch_wrench_any(const FusedArgs& a, cudaStream_t st);
 cudaError_t launch_queue_round_any(const FusedArgs& a, cudaStream_t st);
 cudaError_t launch_fused(int mode, const FusedArgs& a, const fg_hand* h, cudaStream_t st);
 // T-step metric (params.sim_steps >= 1): loss and gradient, or optimisation steps (fg_tstep.cu)
 cudaError_t launch_tstep(int mode, const FusedArgs& a, cudaStream_t st);
+cudaError_t launch_tstep_flat(int mode, const FusedArgs& a, cudaStream_t st);
 // Gauss-Seidel form (params.gauss_seidel = 1): loss and gradient, or optimisation steps (fg_gs.cu)
 cudaError_t launch_gs(int mode, const FusedArgs& a, int nchunks, cudaStream_t st);
 int fused_config_count();

@@ -7,7 +7,7 @@
 // a convex combination of the cell's corners, so it never drops below the
 // minimum of any block that contains the cell.  The pass over the grid that makes level 1 also
 // finds the smallest value of a cell whose 8 corners are equal, where the gradient
-// is zero.
+// is zero (in other cells it can be zero at single points or along lines only).
 #include <cuda_runtime.h>
 
 #include <cstring>

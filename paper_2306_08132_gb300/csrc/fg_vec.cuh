@@ -53,9 +53,6 @@ __device__ __forceinline__ float2 vfnma(float2 a, float2 b, float2 c) { return v
 // a b - c d (not used for decisions)
 __device__ __forceinline__ float vdiff(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
 __device__ __forceinline__ float2 vdiff(float2 a, float2 b, float2 c, float2 d) { return vsub(vmul(a, b), vmul(c, d)); }
-// -(a b)
-__device__ __forceinline__ float vnmul(float a, float b) { return -__fmul_rn(a, b); }
-__device__ __forceinline__ float2 vnmul(float2 a, float2 b) { return vmul(vmul(a, b), make_float2(-1.0f, -1.0f)); }
 
 template <class V>
 __device__ __forceinline__ V vsplat(float x);
@@ -88,8 +85,6 @@ __device__ __forceinline__ float2 vmap(float2 a, F f) {
 // --------------------------------------------------------------------- masks
 __device__ __forceinline__ bool vlt(float a, float b) { return a < b; }
 __device__ __forceinline__ bool2 vlt(float2 a, float2 b) { return {a.x < b.x, a.y < b.y}; }
-__device__ __forceinline__ bool vgt(float a, float b) { return a > b; }
-__device__ __forceinline__ bool2 vgt(float2 a, float2 b) { return {a.x > b.x, a.y > b.y}; }
 __device__ __forceinline__ bool vne(float a, float b) { return a != b; }
 __device__ __forceinline__ bool2 vne(float2 a, float2 b) { return {a.x != b.x, a.y != b.y}; }
 

@@ -164,3 +164,13 @@ def test_zero_gradient_cell_anywhere_in_the_grid(fg):
         loss, grad = fg.loss_and_grad(hand, fg.Scene([fg.Sdf.from_synth(o) for o in objs]), torch.tensor(q, device="cuda:0"),
                                       params, R, obj_of_cand=torch.tensor(oc, device="cuda:0"))
         _check(loss, grad, ref, oc)
+
+
+@pytest.mark.parametrize("form", [{}, {"gauss_seidel": 1}, {"sim_steps": 1}])
+def test_zero_gradient_contacts_in_a_scene_with_a_mesh(fg, case, form):
+    import synth.meshes
+    params = dict(case.w.params, **form)
+    ref, idx = case.reference(params)
+    scene = fg.Scene([fg.Sdf.from_synth(synth.meshes.icosphere(0.04, 1)), fg.Sdf.from_synth(case.obj)])
+    oc = torch.ones(len(case.q), device=case.q.device, dtype=torch.int32)
+    _check(*fg.loss_and_grad(case.hand, scene, case.q, params, R, obj_of_cand=oc), ref, idx)
