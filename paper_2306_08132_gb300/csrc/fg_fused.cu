@@ -26,8 +26,8 @@ constexpr int kCfg16 = 11;       // 16 warps, >= 1 CTA per SM
 // few chunks to share (640 points: 152 candidates 0.041, 0.033, 0.028; 304: 0.044, 0.037,
 // 0.044; 912: 0.058, 0.059, 0.092).  On a mesh a candidate inside the object costs many
 // times the others, so more warps shorten the end of the launch (4,352 points, 2,208 faces: 1,024
-// candidates 2.11, 1.40, 1.29; 4,096: 6.03, 4.49, 4.08; 8,192: 9.19, 7.65, 7.55: 16 warps are
-// ahead at every size measured, by 1% where the line to 8 lies; other hands on meshes were not measured).
+// candidates 2.11, 1.40, 1.29; 4,096: 6.03, 4.49, 4.08; 8,192: 9.55, 7.15, 7.34; other hands on
+// meshes were not measured).
 // The configuration changes no result: units, chunks and sums are the same at any number of warps.
 static int default_config(const FusedArgs& a) {
   const long long sms = device_sm_count(), B = a.B;

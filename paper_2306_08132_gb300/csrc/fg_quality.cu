@@ -224,7 +224,7 @@ __device__ __forceinline__ int float_order(float x) {
 __device__ __forceinline__ float order_float(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
 // Bound: issue in the fold, 13 instructions a (direction, contact) pair with 8 edges.
-// 8,192 candidates, 76 contacts each, 1,024 directions, 8 edges: 2.27 -> 0.77 ms (FMA
+// 8,192 candidates, 76 contacts each, 1,024 directions, 8 edges: 2.27 -> 0.77 to 0.80 ms (FMA
 // pipe 33%; the SMs are busy 73% of the launch: candidates with over a
 // thousand contacts end last).
 template <bool ANY>
