@@ -174,3 +174,21 @@ def test_zero_gradient_contacts_in_a_scene_with_a_mesh(fg, case, form):
     scene = fg.Scene([fg.Sdf.from_synth(synth.meshes.icosphere(0.04, 1)), fg.Sdf.from_synth(case.obj)])
     oc = torch.ones(len(case.q), device=case.q.device, dtype=torch.int32)
     _check(*fg.loss_and_grad(case.hand, scene, case.q, params, R, obj_of_cand=oc), ref, idx)
+
+
+@pytest.mark.parametrize("points_per_link", [21, 1300])
+def test_zero_gradient_contacts_of_ragged_and_large_hands(fg, case, points_per_link):
+    """Chunks that span links, and 13,000 points (more chunks than are flagged, two parts of the adjoint sweep): the
+    fused step against the per-stage form, which takes the same decisions at every point."""
+    h = synth.make_hand(3, points_per_link)
+    hand = fg.Hand.from_synth(h)
+    q0 = torch.tensor(synth.sample_candidates(np.random.default_rng(5), h, 24, 0.1), device="cuda:0")
+    for mu in (0.5, 0.05):
+        params = dict(case.w.params, r0=R, mu=mu)
+        a, b = q0.clone(), q0.clone()
+        la = fg.optimize_step(hand, case.scene, a, params, 0, 10, 1)
+        lb = fg.optimize_step_plain(hand, case.scene, b, params, 0, 10, 1)
+        assert torch.allclose(la, lb, rtol=LOSS_TOL, atol=1e-6)
+        ga, gb = (q0 - a).double(), (q0 - b).double()
+        rel = (ga - gb).norm(dim=1) / gb.norm(dim=1).clamp(min=1e-9)
+        assert float(rel.max()) < GRAD_TOL, rel
