@@ -462,10 +462,11 @@ __device__ __forceinline__ void first_forward_chunk(const ObjDev& O, const Param
 // NEAR: the queries lie at most one cell from the point (near_queries), so along each
 // axis they read the point's own cell or the next one: the 8 corners are read once and
 // a moved query replaces one plane of 4 where it has left the cell, 8 + 6 x 4 predicated loads
-// a point instead of 56.  An axis clamped at its upper end stands at the boundary node, as in
-// sdf_lookup, with that node's plane read as the upper one too (stride 0): the value is
-// then the forward sweep's, bit for bit.  Same batch: 1.86 -> 1.54 ms, L1 data pipe 72% -> 49%; the four warps a
-// scheduler that 128 registers leave no longer cover the latencies.
+// a point instead of 56.  Same batch: 1.86 -> 1.54 ms, L1 data pipe 72% -> 49%; the four warps a
+// scheduler that 128 registers leave no longer cover the latencies.  An axis clamped at its
+// upper end stands at the boundary node, as in sdf_lookup, with that node's plane read as the
+// upper one too (stride 0): the value is the forward sweep's, bit for bit (8 x 512
+// candidates 1.353 -> 1.371 ms).
 template <bool ANY, bool NEAR, bool FLAT>
 __device__ __forceinline__ void first_reverse_point(const ObjDev& O, const ParamsDev& Pm, const float (*G)[6],
                                                     const float p[3], bool valid, float rdil, float c, float pb[3]) {

@@ -12,7 +12,6 @@ import pytest
 import torch
 
 import synth
-import synth.meshes
 from oracle import fastgraspd_oracle as O
 
 pytestmark = pytest.mark.gpu
@@ -398,7 +397,8 @@ def test_large_hand_results_do_not_depend_on_the_batch(fg):
     for B in (600, 2400):
         l, g = fg.loss_and_grad(hand, scene, q[:B].contiguous(), w.params, 0.004)
         assert torch.equal(l[:12], l0) and torch.equal(g[:12], g0), B
-    mesh = fg.Scene([fg.Sdf.from_synth(synth.meshes.icosphere(0.04, 2))])
+    from synth.meshes import icosphere
+    mesh = fg.Scene([fg.Sdf.from_synth(icosphere(0.04, 2))])
     lm, gm = fg.loss_and_grad(hand, mesh, first, w.params, 0.004)
     try:
         for i, (_, _, ppt) in enumerate(fg.fused_configs()):
